@@ -137,10 +137,20 @@ static bool use_compensated(const deer_dynamics* f, const deer_options* o) {
          o->damp != DEER_DAMP_ELK && (f->d == 4 || f->d == 8 || f->d == 16 || f->d == 32);
 }
 
-static int choose_chunk(const deer_options* o, int d) {
+static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N) {
   if (use_diag_lookback(o, d)) return diag_lb_chunk(d);
   if (o->chunk > 0) return o->chunk;
-  if (o->jac == DEER_JAC_FULL) return d >= 16 ? 32 : 64;
+  if (o->jac == DEER_JAC_FULL && d >= 16) return 32;
+  if (o->jac == DEER_JAC_FULL) {
+    // Shorter chunks while the chunk passes (d lanes per chunk) leave the GPU short of four
+    // warps per SM, as long as the per-sequence carry stays the shorter chain: it walks
+    // T / L chunks at about half the time of the chunk passes' L rows. Mass action d = 8,
+    // float64, 37 x 1501 rows: L = 16 solves in 5.5 ms, L = 32 in 8.0, L = 64 in 15.2.
+    int L = 64;
+    const int64_t T = B > 0 ? N / B : 0;
+    while (L > 16 && N / L * d < 152 * 4 * 32 && T <= 2 * (int64_t)L * L) L /= 2;
+    return L;
+  }
   return 128;
 }
 
@@ -156,7 +166,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   const size_t rs = o->prec == DEER_FP32 ? 4 : 8;
   const bool mixed = o->prec == DEER_MIXED_BF16;
   const int d = f->d;
-  const int L = choose_chunk(o, d);
+  const int L = choose_chunk(o, d, B, N);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
   ly.n_chunks_max = N / L + B + 1;

@@ -305,9 +305,9 @@ __device__ __forceinline__ void ldrow_ro(const real* __restrict__ p, real (&v)[D
 // so far more warps are resident to hide latency. The pending (A_t, b_t) of a chunk are
 // stored chunk-major: A at ((c L + t) d + i) d + j, b at (c L + t) d + i.
 // ---------------------------------------------------------------------------
-template <class real, int D, bool RK4, int MODE, bool CS>
-__global__ void __launch_bounds__(kFusedBlock, 4) k_fused_ma_lps(FusedArgs<real> a) {
-  constexpr int GPB = kFusedBlock / D;                  // chunks per block
+template <class real, int D, bool RK4, int MODE, bool CS, int BLK>
+__global__ void __launch_bounds__(BLK, 512 / BLK) k_fused_ma_lps(FusedArgs<real> a) {
+  constexpr int GPB = BLK / D;                          // chunks per block
   constexpr int E = D * D;
   // Exchange buffers: row stride D + 16 B and group stride + 16 B, so that the d lanes of a
   // group storing their rows, and the groups of a warp reading one row each, hit distinct
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kFusedBlock, 4) k_fused_ma_lps(FusedArgs<real>
   // s_t[i] and its compensation term, copied one row ahead with cp.async so that their
   // DRAM latency overlaps the previous row's work; each lane reads back only its own slot
   constexpr int PF = D + 4;
-  __shared__ __align__(16) real sPF[2][kFusedBlock][PF];
+  __shared__ __align__(16) real sPF[2][BLK][PF];
   // the group's stage states (all species), exchanged through shared memory: written with
   // the stage Jacobian's rows, read back as two 16-byte pieces (instead of d shuffles)
   __shared__ __align__(16) real sC[GPB][D];
@@ -718,13 +718,18 @@ static void fused_launch(const FusedArgs<real>& a, cudaStream_t st) {
   constexpr bool MA = KIND == DEER_F_MASSACTION_EULER || KIND == DEER_F_MASSACTION_RK4;
   if constexpr (MA && (D == 4 || D == 8)) {
     constexpr bool RK4 = KIND == DEER_F_MASSACTION_RK4;
-    const unsigned g = grid_for(a.bt.act_chunks(), kFusedBlock / D);
+    // one warp per block: the warps of a launch that does not fill the GPU spread over
+    // every SM (blocks of four warps left two thirds of them idle at 888 float64 chunks)
+    constexpr int BLK = 32;
+    const unsigned g = grid_for(a.bt.act_chunks(), BLK / D);
     if (a.slo) {
-      if (a.mode == 0) k_fused_ma_lps<real, D, RK4, 0, true><<<g, kFusedBlock, 0, st>>>(a);
-      else k_fused_ma_lps<real, D, RK4, 1, true><<<g, kFusedBlock, 0, st>>>(a);
+      if constexpr (sizeof(real) == 4) {
+        if (a.mode == 0) k_fused_ma_lps<real, D, RK4, 0, true, BLK><<<g, BLK, 0, st>>>(a);
+        else k_fused_ma_lps<real, D, RK4, 1, true, BLK><<<g, BLK, 0, st>>>(a);
+      }
     } else {
-      if (a.mode == 0) k_fused_ma_lps<real, D, RK4, 0, false><<<g, kFusedBlock, 0, st>>>(a);
-      else k_fused_ma_lps<real, D, RK4, 1, false><<<g, kFusedBlock, 0, st>>>(a);
+      if (a.mode == 0) k_fused_ma_lps<real, D, RK4, 0, false, BLK><<<g, BLK, 0, st>>>(a);
+      else k_fused_ma_lps<real, D, RK4, 1, false, BLK><<<g, BLK, 0, st>>>(a);
     }
   } else {
     const unsigned g = grid_for(a.bt.act_chunks(), kFusedBlock);

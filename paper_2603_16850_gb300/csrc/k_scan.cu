@@ -222,160 +222,6 @@ __device__ __forceinline__ real reset_val(real v, real thr, int reset) {
 }
 
 // ----------------------------------------------------------------------------
-// Dense scan (one thread per chunk)
-// ----------------------------------------------------------------------------
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_dense_chunk(DenseScanArgs<real> a) {
-  const int64_t ac = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (ac >= a.bt.act_chunks()) return;
-  int64_t seq, c, r0;
-  int n;
-  act_chunk(a.bt, ac, seq, c, r0, n);
-  // the first solved chunk of a sequence starts from Delta = 0: its carry never
-  // multiplies P (the rows before it are the initial state or frozen)
-  const bool need_P = c != win_first(a.bt, seq);
-  real P[D][D], v[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) {
-    v[i] = real(0);
-#pragma unroll U<D>::n
-    for (int j = 0; j < D; ++j) P[i][j] = (i == j) ? real(1) : real(0);
-  }
-  for (int t = 0; t < n; ++t) {
-    const real* At = a.A + (r0 + t) * (int64_t)(D * D);
-    const real* bt = a.b + (r0 + t) * D;
-    real nv[D];
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) {
-      real acc = __ldg(bt + i);
-#pragma unroll U<D>::n
-      for (int k = 0; k < D; ++k) acc += __ldg(At + i * D + k) * v[k];
-      nv[i] = acc;
-    }
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) v[i] = nv[i];
-    if (need_P) {
-      real NP[D][D];
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i)
-#pragma unroll U<D>::n
-        for (int j = 0; j < D; ++j) {
-          real acc = real(0);
-#pragma unroll U<D>::n
-          for (int k = 0; k < D; ++k) acc += __ldg(At + i * D + k) * P[k][j];
-          NP[i][j] = acc;
-        }
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i)
-#pragma unroll U<D>::n
-        for (int j = 0; j < D; ++j) P[i][j] = NP[i][j];
-    }
-  }
-  real* Po = a.aggP + c * (int64_t)(D * D);
-  real* vo = a.aggv + c * D;
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) {
-    vo[i] = v[i];
-#pragma unroll U<D>::n
-    for (int j = 0; j < D; ++j) Po[i * D + j] = P[i][j];
-  }
-}
-
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_dense_carry(DenseScanArgs<real> a) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= a.bt.n_act()) return;
-  const int64_t seq = a.bt.act_seq[k];
-  const int64_t c0 = win_first(a.bt, seq), c1 = a.bt.chunk_first[seq + 1];
-  real x[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) x[i] = real(0);
-  for (int64_t c = c0; c < c1; ++c) {
-    real* ci = a.cin + c * D;
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) ci[i] = x[i];
-    if (c == c1 - 1) break;
-    const real* P = a.aggP + c * (int64_t)(D * D);
-    const real* v = a.aggv + c * D;
-    real nx[D];
-    if (c == c0) {
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) nx[i] = v[i];
-    } else {
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) {
-        real acc = v[i];
-#pragma unroll U<D>::n
-        for (int k = 0; k < D; ++k) acc += P[i * D + k] * x[k];
-        nx[i] = acc;
-      }
-    }
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) x[i] = nx[i];
-  }
-}
-
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_dense_apply(DenseScanArgs<real> a) {
-  const int64_t ac = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (ac >= a.bt.act_chunks()) return;
-  int64_t seq, c, r0;
-  int n;
-  act_chunk(a.bt, ac, seq, c, r0, n);
-  real x[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) x[i] = a.cin[c * D + i];
-  for (int t = 0; t < n; ++t) {
-    const int64_t row = r0 + t;
-    const real* At = a.A + row * (int64_t)(D * D);
-    const real* bt = a.b + row * D;
-    real nx[D];
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) {
-      real acc = __ldg(bt + i);
-#pragma unroll U<D>::n
-      for (int k = 0; k < D; ++k) acc += __ldg(At + i * D + k) * x[k];
-      nx[i] = acc;
-    }
-    real* sr = a.s + row * D;
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) {
-      x[i] = nx[i];
-      sr[i] = reset_val(sr[i] + nx[i], a.reset_thr, a.reset);
-    }
-  }
-}
-
-template <class real, int D>
-static void dense_launch(const DenseScanArgs<real>& a, cudaStream_t st) {
-  const unsigned gc = grid_for(a.bt.act_chunks(), 128);
-  const unsigned gs = grid_for(a.bt.n_act(), 128);
-  k_dense_chunk<real, D><<<gc, 128, 0, st>>>(a);
-  k_dense_carry<real, D><<<gs, 128, 0, st>>>(a);
-  k_dense_apply<real, D><<<gc, 128, 0, st>>>(a);
-  note_launch(3);
-}
-
-template <class real, int D>
-void dense_launch_wide(const DenseScanArgs<real>& a, cudaStream_t st);
-
-template <class real>
-cudaError_t launch_dense_scan(const DenseScanArgs<real>& a, cudaStream_t st) {
-  if (a.bt.act_rows() == 0) return cudaSuccess;
-  switch (a.d) {
-    case 1: dense_launch<real, 1>(a, st); break;
-    case 2: dense_launch<real, 2>(a, st); break;
-    case 4: dense_launch<real, 4>(a, st); break;
-    case 5: dense_launch<real, 5>(a, st); break;
-    case 8: dense_launch<real, 8>(a, st); break;
-    case 16: dense_launch_wide<real, 16>(a, st); break;
-    case 32: dense_launch_wide<real, 32>(a, st); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
 // Diagonal family (one thread per (chunk, coordinate))
 // ----------------------------------------------------------------------------
 template <class real>
@@ -573,8 +419,6 @@ cudaError_t launch_diag_scan(const DiagScanArgs<real>& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template cudaError_t launch_dense_scan<float>(const DenseScanArgs<float>&, cudaStream_t);
-template cudaError_t launch_dense_scan<double>(const DenseScanArgs<double>&, cudaStream_t);
 template cudaError_t launch_diag_scan<float>(const DiagScanArgs<float>&, cudaStream_t);
 template cudaError_t launch_diag_scan<double>(const DiagScanArgs<double>&, cudaStream_t);
 
@@ -755,10 +599,16 @@ template cudaError_t launch_adjoint_scan<double>(const AdjScanArgs<double>&, cud
 namespace deer {
 
 // ----------------------------------------------------------------------------
-// Dense scan, d = 16 / 32: D lanes per chunk (per sequence in the carry pass; four warps
-// per chunk in the d = 32 chunk pass). Lane j owns column j of the chunk product P and
+// Dense scan: D lanes per chunk (per sequence in the carry pass; two or four warps per
+// chunk in the d = 32 chunk pass). Lane j owns column j of the chunk product P and
 // entry j of the vectors; the Jacobian rows and chunk aggregates are staged in a
 // shared-memory ring ahead of use, vector entries travel by shuffles.
+// For d <= 8 what bounds these passes is the dependent chain per row (and, in float64, the
+// issue rate of the FP64 pipe): one thread per chunk loading its own rows was tried first
+// and spent a row's time on uncoalesced loads and D^3 serial products. Two-well Langevin,
+// float64, 4 sequences of 10000 rows, d = 4, per pass: chunk 236 -> 61 us, carry 179 -> 40,
+// apply 200 -> 59; float32 d = 8, 512 x 16384 rows, four Newton steps: 30.8 -> 12.8 ms. d = 1
+// keeps a thread per chunk (k_scalar_*: 8 % faster there, nothing to share in a group).
 // ----------------------------------------------------------------------------
 // 16 bytes (four floats or two doubles) from a 16-byte aligned address. Plain (coherent)
 // load: used for data the same launch never writes, and for data written by earlier
@@ -774,9 +624,16 @@ __device__ __forceinline__ void ld16(const real* p, real* v) {
   }
 }
 
+// lanes of a group: D rounded up to a power of two (d = 5 leaves three lanes idle; they
+// take part in the group's shuffles and barriers with lane 0's data and store nothing)
+template <int D>
+constexpr int group_lanes() { return D <= 2 ? D : D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : 32; }
+
 template <int D>
 __device__ __forceinline__ unsigned group_mask() {
-  return D == 32 ? 0xffffffffu : (0xffffu << (16 * ((threadIdx.x >> 4) & 1)));
+  constexpr int W = group_lanes<D>();
+  if constexpr (W == 32) return 0xffffffffu;
+  return ((1u << W) - 1u) << (threadIdx.x & 31 & ~(W - 1));
 }
 
 // ----------------------------------------------------------------------------
@@ -790,29 +647,43 @@ __device__ __forceinline__ unsigned group_mask() {
 // slot's copies (issued kRing commits earlier) have landed: the wait ends when the copies
 // do, with no spin loop of our own.
 // ----------------------------------------------------------------------------
-template <class real>
-constexpr int ring_depth() { return sizeof(real) == 4 ? 8 : 4; }
+template <class real, int D = 32>
+constexpr int ring_depth() { return sizeof(real) == 4 || D <= 8 ? 8 : 4; }
 
 template <class real, int D>
 struct RowRing {
-  static constexpr int K = ring_depth<real>();
-  static constexpr int RS = D + 16 / (int)sizeof(real);
+  static constexpr int K = ring_depth<real, D>();
+  // rows of whole 16-byte pieces (d = 1, 5 and float d = 2 go entry by entry)
+  static constexpr bool VEC = D * (int)sizeof(real) % 16 == 0;
+  static constexpr int RS = VEC ? D + 16 / (int)sizeof(real) : D;
   real m[K][D][RS];  // row `lane` of a d x d block per slot
   real v[K][D];      // one vector entry per lane per slot
 
   // copy row `lane` of the block at `blk` (16-byte aligned) and vec[lane] into `slot`
   __device__ __forceinline__ void issue(int slot, int lane, const real* blk, const real* vec) {
-    constexpr int PIECES = D * (int)sizeof(real) / 16;
+    if (lane >= D) return;
+    if constexpr (VEC) {
+      constexpr int PIECES = D * (int)sizeof(real) / 16;
 #pragma unroll
-    for (int q = 0; q < PIECES; ++q)
-      cp_async16(&m[slot][lane][q * 16 / (int)sizeof(real)],
-                 blk + lane * D + q * 16 / (int)sizeof(real));
+      for (int q = 0; q < PIECES; ++q)
+        cp_async16(&m[slot][lane][q * 16 / (int)sizeof(real)],
+                   blk + lane * D + q * 16 / (int)sizeof(real));
+    } else {
+#pragma unroll
+      for (int q = 0; q < D; ++q) cp_async_small<sizeof(real)>(&m[slot][lane][q], blk + lane * D + q);
+    }
     cp_async_small<sizeof(real)>(&v[slot][lane], vec + lane);
   }
   __device__ __forceinline__ void row(int slot, int r, real (&out)[D]) const {
+    if constexpr (!VEC) {
 #pragma unroll
-    for (int k = 0; k < D; k += 16 / (int)sizeof(real)) {
-      if constexpr (sizeof(real) == 4) {
+      for (int k = 0; k < D; ++k) out[k] = m[slot][r][k];
+      return;
+    }
+#pragma unroll
+    for (int k = 0; VEC && k < D; k += 16 / (int)sizeof(real)) {
+      if constexpr (!VEC) {
+      } else if constexpr (sizeof(real) == 4) {
         const float4 q = *reinterpret_cast<const float4*>(&m[slot][r][k]);
         out[k] = q.x; out[k + 1] = q.y; out[k + 2] = q.z; out[k + 3] = q.w;
       } else {
@@ -823,17 +694,19 @@ struct RowRing {
   }
 };
 
-// Chunk pass, d = 16 / 32: one group of D lanes per chunk (one warp per block), lane j owns
+// Chunk pass: one group of D lanes per chunk (one warp per block), lane j owns
 // column j of the chunk product P and entry j of the vector part. Row t's Jacobian is
 // staged in the ring; every lane reads all of its rows (broadcast) for P <- A_t P and
 // its own row for v <- A_t v + b_t.
 template <class real, int D>
 __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) {
-  constexpr int G = 32 / D;
+  constexpr int W = group_lanes<D>(), G = 32 / W;
   using Ring = RowRing<real, D>;
   constexpr int K = Ring::K;
+  constexpr int kUnroll = D == 8 || D == 5 ? 1 : K;  // d^3 products per row: keep the code small
   __shared__ __align__(16) Ring ring[G];
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;  // this lane's row / column
   const unsigned gm = group_mask<D>();
   const int64_t ac = blockIdx.x * (int64_t)G + grp;
   if (ac >= a.bt.act_chunks()) return;  // whole groups; groups never synchronise with each other
@@ -852,19 +725,19 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
   real Pc[D];  // column `lane` of P
   real v = real(0);
 #pragma unroll
-  for (int i = 0; i < D; ++i) Pc[i] = i == lane ? real(1) : real(0);
+  for (int i = 0; i < D; ++i) Pc[i] = i == li ? real(1) : real(0);
   for (int t0 = 0; t0 < n; t0 += K) {
-#pragma unroll
+#pragma unroll(kUnroll)
     for (int s = 0; s < K; ++s) {
       const int t = t0 + s;
       cp_async_wait<K - 1>();
       __syncwarp(gm);  // the other lanes' rows of this slot have landed
       if (t < n) {
         real own[D];
-        R.row(s, lane, own);
-        real nv = R.v[s][lane];
+        R.row(s, li, own);
+        real nv = R.v[s][li];
 #pragma unroll
-        for (int k = 0; k < D; ++k) nv += own[k] * __shfl_sync(gm, v, k, D);
+        for (int k = 0; k < D; ++k) nv += own[k] * __shfl_sync(gm, v, k, W);
         v = nv;
         if (need_P) {
           real np[D];
@@ -887,6 +760,7 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
     }
   }
   cp_async_wait<0>();
+  if (lane >= D) return;
   real* Po = a.aggP + c * (int64_t)(D * D);
 #pragma unroll
   for (int i = 0; i < D; ++i) Po[i * D + lane] = Pc[i];
@@ -1118,11 +992,12 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
 // sequence); the aggregates do not depend on x and stream through the ring.
 template <class real, int D>
 __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) {
-  constexpr int G = 32 / D;
+  constexpr int W = group_lanes<D>(), G = 32 / W;
   using Ring = RowRing<real, D>;
   constexpr int K = Ring::K;
   __shared__ __align__(16) Ring ring[G];
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;  // this lane's row
   const unsigned gm = group_mask<D>();
   const int64_t kq = blockIdx.x * (int64_t)G + grp;
   if (kq >= a.bt.n_act()) return;
@@ -1141,13 +1016,13 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
       const int64_t c = cb + s;
       cp_async_wait<K - 1>();  // each lane reads only its own row: no exchange needed
       if (c < c1) {
-        a.cin[c * D + lane] = x;
-        real y = R.v[s][lane];
+        if (lane < D) a.cin[c * D + lane] = x;
+        real y = R.v[s][li];
         if (c > c0) {
           real pr[D];
-          R.row(s, lane, pr);
+          R.row(s, li, pr);
 #pragma unroll
-          for (int k = 0; k < D; ++k) y += pr[k] * __shfl_sync(gm, x, k, D);
+          for (int k = 0; k < D; ++k) y += pr[k] * __shfl_sync(gm, x, k, W);
         }
         x = y;
       }
@@ -1162,11 +1037,12 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
 // i reads its own row of each staged A_t.
 template <class real, int D>
 __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) {
-  constexpr int G = 32 / D;
+  constexpr int W = group_lanes<D>(), G = 32 / W;
   using Ring = RowRing<real, D>;
   constexpr int K = Ring::K;
   __shared__ __align__(16) Ring ring[G];
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;  // this lane's row
   const unsigned gm = group_mask<D>();
   const int64_t ac = blockIdx.x * (int64_t)G + grp;
   if (ac >= a.bt.act_chunks()) return;
@@ -1181,7 +1057,7 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
     if (s < n) R.issue(s, lane, A0 + s * (int64_t)(D * D), b0 + s * D);
     cp_async_commit();
   }
-  real x = a.cin[c * D + lane];
+  real x = a.cin[c * D + li];
   for (int t0 = 0; t0 < n; t0 += K) {
 #pragma unroll
     for (int s = 0; s < K; ++s) {
@@ -1189,13 +1065,15 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
       cp_async_wait<K - 1>();
       if (t < n) {
         real ar[D];
-        R.row(s, lane, ar);
-        real y = R.v[s][lane];
+        R.row(s, li, ar);
+        real y = R.v[s][li];
 #pragma unroll
-        for (int k = 0; k < D; ++k) y += ar[k] * __shfl_sync(gm, x, k, D);
+        for (int k = 0; k < D; ++k) y += ar[k] * __shfl_sync(gm, x, k, W);
         x = y;
-        real* sp = a.s + (r0 + t) * D + lane;
-        if (a.slo) {
+        real* sp = a.s + (r0 + t) * D + li;
+        if (lane >= D) {
+          // idle lane (d = 5)
+        } else if (a.slo) {
           // compensated state: (s, slo) += Delta with error-free transformations
           real hi = *sp, lo = a.slo[(r0 + t) * D + lane];
           cs_add(hi, lo, y);
@@ -1216,12 +1094,64 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
   cp_async_wait<0>();
 }
 
+// d = 1: one thread per chunk (per sequence in the carry pass).
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_chunk(DenseScanArgs<real> a) {
+  const int64_t ac = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (ac >= a.bt.act_chunks()) return;
+  int64_t seq, c, r0;
+  int n;
+  act_chunk(a.bt, ac, seq, c, r0, n);
+  real P = real(1), v = real(0);
+  for (int t = 0; t < n; ++t) {
+    const real at = __ldg(a.A + r0 + t);
+    v = at * v + __ldg(a.b + r0 + t);
+    P = at * P;
+  }
+  a.aggP[c] = P;
+  a.aggv[c] = v;
+}
+
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_carry(DenseScanArgs<real> a) {
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k >= a.bt.n_act()) return;
+  const int64_t seq = a.bt.act_seq[k];
+  const int64_t c0 = win_first(a.bt, seq), c1 = a.bt.chunk_first[seq + 1];
+  real x = real(0);
+#pragma unroll 4
+  for (int64_t c = c0; c < c1; ++c) {
+    a.cin[c] = x;
+    x = c > c0 ? a.aggP[c] * x + a.aggv[c] : a.aggv[c];
+  }
+}
+
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_apply(DenseScanArgs<real> a) {
+  const int64_t ac = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (ac >= a.bt.act_chunks()) return;
+  int64_t seq, c, r0;
+  int n;
+  act_chunk(a.bt, ac, seq, c, r0, n);
+  real x = a.cin[c];
+  for (int t = 0; t < n; ++t) {
+    x = __ldg(a.A + r0 + t) * x + __ldg(a.b + r0 + t);
+    a.s[r0 + t] = reset_val(a.s[r0 + t] + x, a.reset_thr, a.reset);
+  }
+}
+
 template <class real, int D>
-void dense_launch_wide(const DenseScanArgs<real>& a, cudaStream_t st) {
-  constexpr int G = 32 / D;
+static void dense_launch(const DenseScanArgs<real>& a, cudaStream_t st) {
+  constexpr int G = D == 1 ? 128 : 32 / group_lanes<D>();
   const unsigned gc = grid_for(a.bt.act_chunks(), G);
   const unsigned gs = grid_for(a.bt.n_act(), G);
-  if constexpr (D == 32) {
+  if constexpr (D == 1) {
+    k_scalar_chunk<real><<<gc, 128, 0, st>>>(a);
+    k_scalar_carry<real><<<gs, 128, 0, st>>>(a);
+    k_scalar_apply<real><<<gc, 128, 0, st>>>(a);
+    note_launch(3);
+    return;
+  } else if constexpr (D == 32) {
     if constexpr (sizeof(real) == 4) {
       if (a.tensor_cores)
         k_dense_chunk_mma32<<<grid_for(a.bt.act_chunks(), 1), 64, 0, st>>>(a);
@@ -1233,15 +1163,31 @@ void dense_launch_wide(const DenseScanArgs<real>& a, cudaStream_t st) {
   } else {
     k_dense_chunk_ring<real, D><<<gc, 32, 0, st>>>(a);
   }
-  k_dense_carry_ring<real, D><<<gs, 32, 0, st>>>(a);
-  k_dense_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
-  note_launch(3);
+  if constexpr (D > 1) {
+    k_dense_carry_ring<real, D><<<gs, 32, 0, st>>>(a);
+    k_dense_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
+    note_launch(3);
+  }
 }
 
-template void dense_launch_wide<float, 16>(const DenseScanArgs<float>&, cudaStream_t);
-template void dense_launch_wide<float, 32>(const DenseScanArgs<float>&, cudaStream_t);
-template void dense_launch_wide<double, 16>(const DenseScanArgs<double>&, cudaStream_t);
-template void dense_launch_wide<double, 32>(const DenseScanArgs<double>&, cudaStream_t);
+template <class real>
+cudaError_t launch_dense_scan(const DenseScanArgs<real>& a, cudaStream_t st) {
+  if (a.bt.act_rows() == 0) return cudaSuccess;
+  switch (a.d) {
+    case 1: dense_launch<real, 1>(a, st); break;
+    case 2: dense_launch<real, 2>(a, st); break;
+    case 4: dense_launch<real, 4>(a, st); break;
+    case 5: dense_launch<real, 5>(a, st); break;
+    case 8: dense_launch<real, 8>(a, st); break;
+    case 16: dense_launch<real, 16>(a, st); break;
+    case 32: dense_launch<real, 32>(a, st); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_dense_scan<float>(const DenseScanArgs<float>&, cudaStream_t);
+template cudaError_t launch_dense_scan<double>(const DenseScanArgs<double>&, cudaStream_t);
 
 }  // namespace deer
 
