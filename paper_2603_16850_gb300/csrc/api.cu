@@ -154,6 +154,14 @@ static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N) {
   return 128;
 }
 
+// Chunk length of the adjoint where the caller leaves it to the library: fixed by d in
+// float32, whose gradient carries the rounding of the chunk products (near equilibrium the
+// same in every chunk, so it adds up over T: the length is part of the result's rounding).
+static int grad_chunk(const deer_dynamics* f, const deer_options* o) {
+  if (o->chunk > 0 || o->prec != DEER_FP32) return o->chunk;
+  return f->d >= 16 ? 32 : 64;
+}
+
 // Largest row count any layout accepts: keeps every size product below (N + C) d^2 * 8
 // far from overflowing 64 bits (d <= 64).
 constexpr int64_t kMaxRows = int64_t(1) << 44;
@@ -1053,6 +1061,7 @@ size_t deer_grad_workspace_bytes(const deer_dynamics* f, int64_t batch, int64_t 
   o.jac = DEER_JAC_FULL;
   o.damp = DEER_DAMP_NONE;
   o.compensate = 0;
+  o.chunk = grad_chunk(f, &o);
   if (check_common(f, &o) != DEER_OK) return 0;
   const int64_t W = grad_window_rows(f, batch, T, &o);
   if (W < T) {
@@ -1131,6 +1140,18 @@ static deer_status jacobians_at(const deer_dynamics* f, int64_t B, int64_t T, co
   la.jac = DEER_JAC_FULL;
   la.damp = DEER_DAMP_NONE;
   la.dparam = real(0);
+  if (ly.adj_off != ly.adj_e) {
+    // mass action, d = 16 / 32: the per-species reaction lists of the wide linearisation
+    // (walking all 48 reactions per lane took twice as long: 30.4 against 15.2 ms for 2.1 M
+    // rows, d = 32)
+    const int64_t nseq = f->topology_stride ? B : 1;
+    DEER_CK(launch_ma_adjacency(nseq, d, f->n_reactions, f->topology, f->topology_stride,
+                                reinterpret_cast<int32_t*>(ws + ly.adj_off),
+                                reinterpret_cast<int32_t*>(ws + ly.adj_e), st));
+    la.adj_off = reinterpret_cast<const int32_t*>(ws + ly.adj_off);
+    la.adj_e = reinterpret_cast<const int32_t*>(ws + ly.adj_e);
+    la.adj_stride = f->topology_stride ? 4 * (int64_t)f->n_reactions : 0;
+  }
   DEER_CK(launch_linearize<real>(la, st));
   return DEER_OK;
 }
@@ -1175,7 +1196,13 @@ static deer_status grad_core(const deer_dynamics* f, int64_t B, int64_t T, const
   pa.pstride = f->kind == DEER_F_BRUSSELATOR_EULER ? 2 : f->n_reactions;
   pa.ds0 = static_cast<real*>(ds0_);
   if (pa.dparams && zero_dp) DEER_CK(cudaMemsetAsync(pa.dparams, 0, B * pa.pstride * rs, st));
-  DEER_CK(launch_param_grad<real>(pa, st));
+  DEER_CK(launch_adj_ds0<real>(pa, st));
+  if (pa.dparams && ma_param_grad_supported(f->kind, d, f->n_reactions)) {
+    MaGradArgs<real> ma{dv, B, T, la.s0, la.s, sa.lam, pa.dparams, pa.pstride};
+    DEER_CK(launch_ma_param_grad<real>(ma, st));
+  } else {
+    DEER_CK(launch_param_grad<real>(pa, st));
+  }
   if (dx_) {
     InputGradArgs<real> ia{dv, bt, la.s0, la.s, sa.lam, static_cast<real*>(dx_)};
     DEER_CK(launch_input_grad<real>(ia, st));
@@ -1363,6 +1390,7 @@ deer_status deer_grad_ex(const deer_dynamics* f, int64_t batch, int64_t T, const
   o.jac = DEER_JAC_FULL;
   o.damp = DEER_DAMP_NONE;
   o.compensate = 0;
+  o.chunk = grad_chunk(f, &o);
   if (o.prec == DEER_MIXED_BF16) return DEER_ERR_UNSUPPORTED;
   deer_status c = check_common(f, &o);
   if (c != DEER_OK) return c;

@@ -207,8 +207,8 @@ __global__ void k_gru_setup(int d, const real* __restrict__ params, int d_in, re
 // Adjoint parameter gradient (one thread per row): the vector-Jacobian product
 // lambda_t^T df_t/dtheta (s_{t-1}) by reverse-mode through the integrator stages, summed
 // over the rows of each sequence (warp reduction, then one atomic per warp and
-// parameter), and dl/ds0 = A_1^T lambda_1. Mass action: theta = rate constants k;
-// Brusselator: theta = (a, b).
+// parameter). Mass action: theta = rate constants k (d <= 8, or more reactions than
+// k_ma_grad.cu takes); Brusselator: theta = (a, b).
 // ----------------------------------------------------------------------------
 constexpr int kMaxD = 32;
 
@@ -255,15 +255,6 @@ __global__ void __launch_bounds__(128) k_param_grad(ParamGradArgs<real> a, int r
   const int64_t first = valid ? a.bt.offsets[seq] : 0;
   const real* sp = valid ? (row == first ? a.s0 + seq * d : a.s + (row - 1) * d) : a.s0;
   const real* lam = a.lam + (valid ? row : 0) * d;
-  if (valid && a.ds0 && row == first) {
-    const real* A1 = a.A + row * (int64_t)d * d;
-    for (int j = 0; j < d; ++j) {
-      real acc = real(0);
-      for (int i = 0; i < d; ++i) acc += A1[i * d + j] * lam[i];
-      a.ds0[seq * d + j] = acc;
-    }
-  }
-  if (!a.dparams) return;
   const unsigned full = 0xffffffffu;
   const unsigned vm = __ballot_sync(full, valid);
   if (vm == 0) return;
@@ -333,9 +324,33 @@ __global__ void __launch_bounds__(128) k_param_grad(ParamGradArgs<real> a, int r
   }
 }
 
+// dl/ds0 = A_1^T lambda_1 (one thread per sequence and coordinate)
+template <class real>
+__global__ void __launch_bounds__(128) k_adj_ds0(ParamGradArgs<real> a) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int d = a.dv.d;
+  if (e >= a.bt.B * d) return;
+  const int64_t seq = e / d, row = a.bt.offsets[seq];
+  const int j = (int)(e - seq * d);
+  if (row == a.bt.offsets[seq + 1]) return;
+  const real* A1 = a.A + row * (int64_t)d * d;
+  const real* lam = a.lam + row * d;
+  real acc = real(0);
+  for (int i = 0; i < d; ++i) acc += A1[i * d + j] * lam[i];
+  a.ds0[e] = acc;
+}
+
+template <class real>
+cudaError_t launch_adj_ds0(const ParamGradArgs<real>& a, cudaStream_t st) {
+  if (a.bt.N == 0 || !a.ds0) return cudaSuccess;
+  k_adj_ds0<real><<<grid_for(a.bt.B * a.dv.d, 128), 128, 0, st>>>(a);
+  note_launch();
+  return cudaGetLastError();
+}
+
 template <class real>
 cudaError_t launch_param_grad(const ParamGradArgs<real>& a, cudaStream_t st) {
-  if (a.bt.N == 0) return cudaSuccess;
+  if (a.bt.N == 0 || !a.dparams) return cudaSuccess;
   if (a.dv.d > kMaxD) return cudaErrorInvalidValue;
   const int rk4 = a.dv.kind == DEER_F_MASSACTION_RK4;
   k_param_grad<real><<<grid_for(a.bt.N, 128), 128, 0, st>>>(a, rk4);
@@ -507,6 +522,7 @@ cudaError_t launch_input_grad(const InputGradArgs<real>& a, cudaStream_t st) {
   template cudaError_t launch_linearize<real>(const LinArgs<real>&, cudaStream_t);             \
   template cudaError_t launch_rollout<real>(const RolloutArgs<real>&, cudaStream_t);          \
   template cudaError_t launch_gru_setup<real>(int, const real*, int, real*, cudaStream_t);   \
+  template cudaError_t launch_adj_ds0<real>(const ParamGradArgs<real>&, cudaStream_t);       \
   template cudaError_t launch_param_grad<real>(const ParamGradArgs<real>&, cudaStream_t);
 DEER_INST(float)
 DEER_INST(double)

@@ -212,9 +212,6 @@ cudaError_t launch_check(const CheckArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int D>
-struct U { static constexpr int n = D <= 8 ? D : 1; };
-
 template <class real>
 __device__ __forceinline__ real reset_val(real v, real thr, int reset) {
   if (reset && !(v <= thr && v >= -thr)) return real(0);
@@ -427,178 +424,6 @@ template cudaError_t launch_diag_scan<double>(const DiagScanArgs<double>&, cudaS
 namespace deer {
 
 // ----------------------------------------------------------------------------
-// Reverse dense scan for the adjoint (one thread per chunk / per sequence), rows visited
-// from the end of the sequence: lambda_t = M_t lambda_{t+1} + g_t with M_t = A_{t+1}^T and
-// lambda_{T+1} = 0. Chunk aggregates compose in reverse row order.
-// ----------------------------------------------------------------------------
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_chunk(AdjScanArgs<real> a) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= a.bt.n_chunks) return;
-  int64_t seq, r0;
-  int n;
-  chunk_rows(a.bt, c, seq, r0, n);
-  const int64_t rend = __ldg(a.bt.offsets + seq + 1);  // one past the last row
-  const bool need_P = c != __ldg(a.bt.chunk_first + seq + 1) - 1;  // last chunk: carry 0
-  real P[D][D], v[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) {
-    v[i] = real(0);
-#pragma unroll U<D>::n
-    for (int j = 0; j < D; ++j) P[i][j] = (i == j) ? real(1) : real(0);
-  }
-  for (int t = n - 1; t >= 0; --t) {
-    const int64_t row = r0 + t;
-    const real* gt = a.g + row * D;
-    if (row + 1 < rend) {
-      const real* An = a.A + (row + 1) * (int64_t)(D * D);  // M_t = A_{t+1}^T
-      real nv[D];
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) {
-        real acc = __ldg(gt + i);
-#pragma unroll U<D>::n
-        for (int k = 0; k < D; ++k) acc += __ldg(An + k * D + i) * v[k];
-        nv[i] = acc;
-      }
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) v[i] = nv[i];
-      if (need_P) {
-        real NP[D][D];
-#pragma unroll U<D>::n
-        for (int i = 0; i < D; ++i)
-#pragma unroll U<D>::n
-          for (int j = 0; j < D; ++j) {
-            real acc = real(0);
-#pragma unroll U<D>::n
-            for (int k = 0; k < D; ++k) acc += __ldg(An + k * D + i) * P[k][j];
-            NP[i][j] = acc;
-          }
-#pragma unroll U<D>::n
-        for (int i = 0; i < D; ++i)
-#pragma unroll U<D>::n
-          for (int j = 0; j < D; ++j) P[i][j] = NP[i][j];
-      }
-    } else {
-      // last row of the sequence: lambda_T = g_T, the carry (lambda_{T+1} = 0) is dropped
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) {
-        v[i] = __ldg(gt + i);
-#pragma unroll U<D>::n
-        for (int j = 0; j < D; ++j) P[i][j] = real(0);
-      }
-    }
-  }
-  real* Po = a.aggP + c * (int64_t)(D * D);
-  real* vo = a.aggv + c * D;
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) {
-    vo[i] = v[i];
-#pragma unroll U<D>::n
-    for (int j = 0; j < D; ++j) Po[i * D + j] = P[i][j];
-  }
-}
-
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_carry(AdjScanArgs<real> a) {
-  const int64_t seq = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (seq >= a.bt.B) return;
-  const int64_t c0 = a.bt.chunk_first[seq], c1 = a.bt.chunk_first[seq + 1];
-  real x[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) x[i] = real(0);
-  for (int64_t c = c1 - 1; c >= c0; --c) {
-    real* ci = a.cin + c * D;
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) ci[i] = x[i];
-    const real* P = a.aggP + c * (int64_t)(D * D);
-    const real* v = a.aggv + c * D;
-    real nx[D];
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) {
-      real acc = v[i];
-#pragma unroll U<D>::n
-      for (int k = 0; k < D; ++k) acc += P[i * D + k] * x[k];
-      nx[i] = acc;
-    }
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) x[i] = nx[i];
-  }
-}
-
-template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_apply(AdjScanArgs<real> a) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= a.bt.n_chunks) return;
-  int64_t seq, r0;
-  int n;
-  chunk_rows(a.bt, c, seq, r0, n);
-  const int64_t rend = __ldg(a.bt.offsets + seq + 1);
-  real x[D];
-#pragma unroll U<D>::n
-  for (int i = 0; i < D; ++i) x[i] = a.cin[c * D + i];
-  for (int t = n - 1; t >= 0; --t) {
-    const int64_t row = r0 + t;
-    const real* gt = a.g + row * D;
-    real nx[D];
-    if (row + 1 < rend) {
-      const real* An = a.A + (row + 1) * (int64_t)(D * D);
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) {
-        real acc = __ldg(gt + i);
-#pragma unroll U<D>::n
-        for (int k = 0; k < D; ++k) acc += __ldg(An + k * D + i) * x[k];
-        nx[i] = acc;
-      }
-    } else {
-#pragma unroll U<D>::n
-      for (int i = 0; i < D; ++i) nx[i] = __ldg(gt + i);
-    }
-    real* lr = a.lam + row * D;
-#pragma unroll U<D>::n
-    for (int i = 0; i < D; ++i) {
-      x[i] = nx[i];
-      lr[i] = nx[i];
-    }
-  }
-}
-
-template <class real, int D>
-static void adj_launch(const AdjScanArgs<real>& a, cudaStream_t st) {
-  const unsigned gc = grid_for(a.bt.n_chunks, 128);
-  const unsigned gs = grid_for(a.bt.B, 128);
-  k_adj_chunk<real, D><<<gc, 128, 0, st>>>(a);
-  k_adj_carry<real, D><<<gs, 128, 0, st>>>(a);
-  k_adj_apply<real, D><<<gc, 128, 0, st>>>(a);
-  note_launch(3);
-}
-
-template <class real, int D>
-void adj_launch_wide(const AdjScanArgs<real>& a, cudaStream_t st);
-
-template <class real>
-cudaError_t launch_adjoint_scan(const AdjScanArgs<real>& a, cudaStream_t st) {
-  if (a.bt.N == 0) return cudaSuccess;
-  switch (a.d) {
-    case 1: adj_launch<real, 1>(a, st); break;
-    case 2: adj_launch<real, 2>(a, st); break;
-    case 4: adj_launch<real, 4>(a, st); break;
-    case 5: adj_launch<real, 5>(a, st); break;
-    case 8: adj_launch<real, 8>(a, st); break;
-    case 16: adj_launch_wide<real, 16>(a, st); break;
-    case 32: adj_launch_wide<real, 32>(a, st); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
-template cudaError_t launch_adjoint_scan<float>(const AdjScanArgs<float>&, cudaStream_t);
-template cudaError_t launch_adjoint_scan<double>(const AdjScanArgs<double>&, cudaStream_t);
-
-}  // namespace deer
-
-namespace deer {
-
-// ----------------------------------------------------------------------------
 // Dense scan: D lanes per chunk (per sequence in the carry pass; two or four warps per
 // chunk in the d = 32 chunk pass). Lane j owns column j of the chunk product P and
 // entry j of the vectors; the Jacobian rows and chunk aggregates are staged in a
@@ -637,9 +462,9 @@ __device__ __forceinline__ unsigned group_mask() {
 }
 
 // ----------------------------------------------------------------------------
-// Asynchronous row staging for the wide dense scans. Lane i of a group copies its own row
-// (D values, 16-byte pieces) of a d x d block, and one entry of a vector, from global
-// memory into a slot of a shared-memory ring with cp.async; the ring runs kRing slots
+// Asynchronous row staging for the dense scans. The lanes of a group copy a d x d block in
+// 16-byte pieces, and one entry of a vector each, from global
+// memory into a slot of a shared-memory ring with cp.async; the ring runs K slots
 // ahead of the rows being consumed, so the DRAM latency of a row is hidden behind the
 // dependent work on the rows before it. Rows are padded to D + 16 B so that 128-bit
 // reads of eight lanes' rows hit distinct banks. Every stage commits one (possibly empty)
@@ -659,18 +484,24 @@ struct RowRing {
   real m[K][D][RS];  // row `lane` of a d x d block per slot
   real v[K][D];      // one vector entry per lane per slot
 
-  // copy row `lane` of the block at `blk` (16-byte aligned) and vec[lane] into `slot`
+  // copy the block at `blk` (16-byte aligned; the group's lanes take consecutive pieces:
+  // lane-owned rows cost a separate memory transaction per lane, 2063 against 1335 us for the
+  // adjoint's apply pass over 2.1 M rows, d = 32) and vec[lane] into `slot`
   __device__ __forceinline__ void issue(int slot, int lane, const real* blk, const real* vec) {
     if (lane >= D) return;
     if constexpr (VEC) {
-      constexpr int PIECES = D * (int)sizeof(real) / 16;
+      constexpr int VW = 16 / (int)sizeof(real), PR = D / VW;  // pieces per row
 #pragma unroll
-      for (int q = 0; q < PIECES; ++q)
-        cp_async16(&m[slot][lane][q * 16 / (int)sizeof(real)],
-                   blk + lane * D + q * 16 / (int)sizeof(real));
+      for (int q = 0; q < PR; ++q) {
+        const int e = q * D + lane;  // consecutive lanes copy consecutive pieces
+        cp_async16(&m[slot][e / PR][e % PR * VW], blk + e * VW);
+      }
     } else {
 #pragma unroll
-      for (int q = 0; q < D; ++q) cp_async_small<sizeof(real)>(&m[slot][lane][q], blk + lane * D + q);
+      for (int q = 0; q < D; ++q) {
+        const int e = q * D + lane;
+        cp_async_small<sizeof(real)>(&m[slot][e / D][e % D], blk + e);
+      }
     }
     cp_async_small<sizeof(real)>(&v[slot][lane], vec + lane);
   }
@@ -1014,7 +845,8 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
 #pragma unroll
     for (int s = 0; s < K; ++s) {
       const int64_t c = cb + s;
-      cp_async_wait<K - 1>();  // each lane reads only its own row: no exchange needed
+      cp_async_wait<K - 1>();
+      __syncwarp(gm);  // the other lanes' pieces of this slot have landed
       if (c < c1) {
         if (lane < D) a.cin[c * D + lane] = x;
         real y = R.v[s][li];
@@ -1026,6 +858,7 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
         }
         x = y;
       }
+      __syncwarp(gm);  // every lane is done with the slot before it is refilled
       if (c + K < c1) R.issue(s, lane, a.aggP + (c + K) * (int64_t)(D * D), a.aggv + (c + K) * D);
       cp_async_commit();
     }
@@ -1063,6 +896,7 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
     for (int s = 0; s < K; ++s) {
       const int t = t0 + s;
       cp_async_wait<K - 1>();
+      __syncwarp(gm);
       if (t < n) {
         real ar[D];
         R.row(s, li, ar);
@@ -1087,6 +921,7 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
           *sp = reset_val(*sp + y, a.reset_thr, a.reset);
         }
       }
+      __syncwarp(gm);
       if (t + K < n) R.issue(s, lane, A0 + (t + K) * (int64_t)(D * D), b0 + (t + K) * D);
       cp_async_commit();
     }
@@ -1194,120 +1029,305 @@ template cudaError_t launch_dense_scan<double>(const DenseScanArgs<double>&, cud
 namespace deer {
 
 // ----------------------------------------------------------------------------
-// Reverse (adjoint) dense scan, d = 16 / 32: D lanes per chunk / sequence; lane i owns
-// entry i of the vectors and column i of the reversed chunk product. M_t = A_{t+1}^T is
-// read column-wise (entry (k, i) of A_{t+1} for lane i), i.e. coalesced across lanes.
+// Reverse (adjoint) dense scan, rows visited from the end of the sequence:
+// lambda_t = M_t lambda_{t+1} + g_t with M_t = A_{t+1}^T and lambda_{T+1} = 0; chunk
+// aggregates compose in reverse row order. Groups, rings and staging as in the forward scan
+// (lane i owns entry i of the vectors and column i of the chunk product; A_{t+1} and g_t
+// share a slot); every sum runs over k in ascending order, so the results do not depend on
+// which kernel forms them. Thread-per-chunk kernels (d <= 8) and direct global reads (d = 16,
+// 32) took, per pass: d = 8, 512 x 2047 rows: chunk 446, carry 182, apply 359 us (now 116, 9,
+// 75); d = 32, 128 x 16384 rows: chunk 7990, carry 1090, apply 1390 us (now 2835, 88, 1335: A
+// is 8.6 GB).
 // ----------------------------------------------------------------------------
 template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_chunk_wide(AdjScanArgs<real> a) {
-  constexpr int G = 128 / D;
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+__device__ __forceinline__ void adj_issue(RowRing<real, D>& R, int slot, int lane,
+                                          const AdjScanArgs<real>& a, int64_t row, int64_t rend) {
+  if (row + 1 < rend)
+    R.issue(slot, lane, a.A + (row + 1) * (int64_t)(D * D), a.g + row * D);
+  else if (lane < D)
+    cp_async_small<sizeof(real)>(&R.v[slot][lane], a.g + row * D + lane);
+}
+
+template <class real, int D>
+__global__ void __launch_bounds__(32) k_adj_chunk_ring(AdjScanArgs<real> a) {
+  constexpr int W = group_lanes<D>(), G = 32 / W;
+  using Ring = RowRing<real, D>;
+  constexpr int K = Ring::K;
+  __shared__ __align__(16) Ring ring[G];
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;
   const unsigned gm = group_mask<D>();
   const int64_t c = blockIdx.x * (int64_t)G + grp;
-  const bool valid = c < a.bt.n_chunks;
-  int64_t seq = 0, r0 = 0;
-  int n = 0;
-  if (valid) chunk_rows(a.bt, c, seq, r0, n);
-  const int64_t rend = valid ? __ldg(a.bt.offsets + seq + 1) : 0;
-  const bool need_P = valid && c != __ldg(a.bt.chunk_first + seq + 1) - 1;
-  real Pc[D];
+  if (c >= a.bt.n_chunks) return;  // whole groups
+  int64_t seq, r0;
+  int n;
+  chunk_rows(a.bt, c, seq, r0, n);
+  const int64_t rend = __ldg(a.bt.offsets + seq + 1);              // one past the last row
+  const bool need_P = c != __ldg(a.bt.chunk_first + seq + 1) - 1;  // last chunk: carry 0
+  Ring& R = ring[grp];
+#pragma unroll
+  for (int s = 0; s < K; ++s) {
+    if (s < n) adj_issue<real, D>(R, s, lane, a, r0 + n - 1 - s, rend);
+    cp_async_commit();
+  }
+  real Pc[D];  // column `lane` of P
   real v = real(0);
 #pragma unroll
-  for (int i = 0; i < D; ++i) Pc[i] = i == lane ? real(1) : real(0);
-  for (int t = n - 1; t >= 0; --t) {
-    const int64_t row = r0 + t;
-    const real gt = __ldg(a.g + row * D + lane);
+  for (int i = 0; i < D; ++i) Pc[i] = i == li ? real(1) : real(0);
+  for (int j = 0; j < n; ++j) {
+    const int s = j & (K - 1);
+    const int64_t row = r0 + n - 1 - j;
+    cp_async_wait<K - 1>();
+    __syncwarp(gm);  // the other lanes' rows of this slot have landed
+    real nv = R.v[s][li];
     if (row + 1 < rend) {
-      const real* An = a.A + (row + 1) * (int64_t)(D * D);
-      real nv = gt;
 #pragma unroll
-      for (int k = 0; k < D; ++k) nv += __ldg(An + k * D + lane) * __shfl_sync(gm, v, k, D);
-      v = nv;
+      for (int k = 0; k < D; ++k) nv += R.m[s][k][li] * __shfl_sync(gm, v, k, W);
       if (need_P) {
         real np[D];
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-          real x = real(0);
+        for (int i = 0; i < D; ++i) np[i] = real(0);
 #pragma unroll
-          for (int k = 0; k < D; ++k) x += __ldg(An + k * D + i) * Pc[k];
-          np[i] = x;
+        for (int k = 0; k < D; ++k) {
+          real ar[D];
+          R.row(s, k, ar);
+          axpy_row<D>(Pc[k], ar, np);
         }
 #pragma unroll
         for (int i = 0; i < D; ++i) Pc[i] = np[i];
       }
     } else {
-      v = gt;
+      // last row of the sequence: lambda_T = g_T, the carry (lambda_{T+1} = 0) is dropped
 #pragma unroll
       for (int i = 0; i < D; ++i) Pc[i] = real(0);
     }
+    v = nv;
+    __syncwarp(gm);  // every lane is done with the slot before it is refilled
+    if (j + K < n) adj_issue<real, D>(R, s, lane, a, row - K, rend);
+    cp_async_commit();
   }
-  if (valid) {
-    real* Po = a.aggP + c * (int64_t)(D * D);
+  cp_async_wait<0>();
+  if (lane >= D) return;
+  real* Po = a.aggP + c * (int64_t)(D * D);
 #pragma unroll
-    for (int i = 0; i < D; ++i) Po[i * D + lane] = Pc[i];
-    a.aggv[c * D + lane] = v;
+  for (int i = 0; i < D; ++i) Po[i * D + lane] = Pc[i];
+  a.aggv[c * D + lane] = v;
+}
+
+// Chunk pass, d = 32, float32: one warp per chunk, each lane an 8 x 4 tile of the chunk
+// product (lane / 8 picks the rows, lane % 8 the columns), so that one 16-byte read of P and
+// two of A_{t+1} feed 32 multiply-adds instead of eight reads; P alternates between two
+// shared buffers. Bound by the FP32 pipe (32768 multiply-adds per row: 1.8 of its 2.8 ms
+// for 2.1 M rows).
+__global__ void __launch_bounds__(32) k_adj_chunk_tile32(AdjScanArgs<float> a) {
+  constexpr int D = 32, K = 4;
+  __shared__ __align__(16) float sA[K][D][D];
+  __shared__ __align__(16) float sG[K][D];
+  __shared__ __align__(16) float sP[2][D][D];
+  __shared__ __align__(16) float sV[2][D];
+  const int lane = threadIdx.x, i0 = 8 * (lane >> 3), j0 = 4 * (lane & 7);
+  const int64_t c = blockIdx.x;
+  int64_t seq, r0;
+  int n;
+  chunk_rows(a.bt, c, seq, r0, n);
+  const int64_t rend = __ldg(a.bt.offsets + seq + 1);
+  const bool need_P = c != __ldg(a.bt.chunk_first + seq + 1) - 1;
+  auto issue = [&](int slot, int64_t row) {
+    if (row + 1 < rend) {
+      const float* src = a.A + (row + 1) * (int64_t)(D * D);
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+        cp_async16(&sA[slot][0][0] + (p * 32 + lane) * 4, src + (p * 32 + lane) * 4);
+    }
+    cp_async_small<4>(&sG[slot][lane], a.g + row * D + lane);
+  };
+#pragma unroll
+  for (int s = 0; s < K; ++s) {
+    if (s < n) issue(s, r0 + n - 1 - s);
+    cp_async_commit();
   }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sP[0][i0 + i][j0 + j] = i0 + i == j0 + j ? 1.f : 0.f;
+  float v = 0.f;
+  int cur = 0;
+  for (int t = 0; t < n; ++t) {
+    const int s = t & (K - 1);
+    const int64_t row = r0 + n - 1 - t;
+    cp_async_wait<K - 1>();
+    sV[t & 1][lane] = v;
+    __syncwarp();
+    float nv = sG[s][lane];
+    if (row + 1 < rend) {
+#pragma unroll
+      for (int k = 0; k < D; k += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(&sV[t & 1][k]);
+        nv += sA[s][k][lane] * x.x;
+        nv += sA[s][k + 1][lane] * x.y;
+        nv += sA[s][k + 2][lane] * x.z;
+        nv += sA[s][k + 3][lane] * x.w;
+      }
+      if (need_P) {
+        float2 acc[4][4];  // rows i0 + 2 q, + 1; column j0 + j
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[q][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int k = 0; k < D; ++k) {
+          const float4 x = *reinterpret_cast<const float4*>(&sA[s][k][i0]);
+          const float4 y = *reinterpret_cast<const float4*>(&sA[s][k][i0 + 4]);
+          const float4 p = *reinterpret_cast<const float4*>(&sP[cur][k][j0]);
+          const float2 m[4] = {make_float2(x.x, x.y), make_float2(x.z, x.w),
+                               make_float2(y.x, y.y), make_float2(y.z, y.w)};
+          const float pj[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 pp = make_float2(pj[j], pj[j]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q][j] = __ffma2_rn(m[q], pp, acc[q][j]);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          *reinterpret_cast<float4*>(&sP[cur ^ 1][i0 + 2 * q][j0]) =
+              make_float4(acc[q][0].x, acc[q][1].x, acc[q][2].x, acc[q][3].x);
+          *reinterpret_cast<float4*>(&sP[cur ^ 1][i0 + 2 * q + 1][j0]) =
+              make_float4(acc[q][0].y, acc[q][1].y, acc[q][2].y, acc[q][3].y);
+        }
+        cur ^= 1;
+      }
+    } else {
+      // last row of the sequence: the carry (lambda_{T+1} = 0) is dropped
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4*>(&sP[cur][i0 + i][j0]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    v = nv;
+    __syncwarp();  // every lane is done with the slot before it is refilled
+    if (t + K < n) issue(s, row - K);
+    cp_async_commit();
+  }
+  cp_async_wait<0>();
+  __syncwarp();
+  float* Po = a.aggP + c * (int64_t)(D * D);
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+    reinterpret_cast<float4*>(Po)[p * 32 + lane] =
+        reinterpret_cast<const float4*>(&sP[cur][0][0])[p * 32 + lane];
+  a.aggv[c * D + lane] = v;
 }
 
 template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_carry_wide(AdjScanArgs<real> a) {
-  constexpr int G = 128 / D;
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+__global__ void __launch_bounds__(32) k_adj_carry_ring(AdjScanArgs<real> a) {
+  constexpr int W = group_lanes<D>(), G = 32 / W;
+  using Ring = RowRing<real, D>;
+  constexpr int K = Ring::K;
+  __shared__ __align__(16) Ring ring[G];
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;
   const unsigned gm = group_mask<D>();
   const int64_t seq = blockIdx.x * (int64_t)G + grp;
-  const bool valid = seq < a.bt.B;
-  const int64_t c0 = valid ? a.bt.chunk_first[seq] : 0;
-  const int64_t c1 = valid ? a.bt.chunk_first[seq + 1] : 0;
-  real x = real(0);
-  for (int64_t c = c1 - 1; c >= c0; --c) {
-    a.cin[c * D + lane] = x;
-    const real* P = a.aggP + c * (int64_t)(D * D);
-    real y = a.aggv[c * D + lane];
+  if (seq >= a.bt.B) return;
+  const int64_t c0 = a.bt.chunk_first[seq], c1 = a.bt.chunk_first[seq + 1];
+  Ring& R = ring[grp];
 #pragma unroll
-    for (int k = 0; k < D; ++k) y += P[lane * D + k] * __shfl_sync(gm, x, k, D);
-    x = y;
+  for (int s = 0; s < K; ++s) {
+    if (c1 - 1 - s >= c0)
+      R.issue(s, lane, a.aggP + (c1 - 1 - s) * (int64_t)(D * D), a.aggv + (c1 - 1 - s) * D);
+    cp_async_commit();
   }
+  real x = real(0);
+  int s = 0;
+  for (int64_t c = c1 - 1; c >= c0; --c) {
+    cp_async_wait<K - 1>();
+    __syncwarp(gm);
+    if (lane < D) a.cin[c * D + lane] = x;
+    real y = R.v[s][li];
+    real pr[D];
+    R.row(s, li, pr);
+#pragma unroll
+    for (int k = 0; k < D; ++k) y += pr[k] * __shfl_sync(gm, x, k, W);
+    x = y;
+    __syncwarp(gm);
+    if (c - K >= c0)
+      R.issue(s, lane, a.aggP + (c - K) * (int64_t)(D * D), a.aggv + (c - K) * D);
+    cp_async_commit();
+    s = (s + 1) & (K - 1);
+  }
+  cp_async_wait<0>();
 }
 
 template <class real, int D>
-__global__ void __launch_bounds__(128) k_adj_apply_wide(AdjScanArgs<real> a) {
-  constexpr int G = 128 / D;
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
+__global__ void __launch_bounds__(32) k_adj_apply_ring(AdjScanArgs<real> a) {
+  constexpr int W = group_lanes<D>(), G = 32 / W;
+  using Ring = RowRing<real, D>;
+  constexpr int K = Ring::K;
+  __shared__ __align__(16) Ring ring[G];
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int li = lane < D ? lane : 0;
   const unsigned gm = group_mask<D>();
   const int64_t c = blockIdx.x * (int64_t)G + grp;
-  const bool valid = c < a.bt.n_chunks;
-  int64_t seq = 0, r0 = 0;
-  int n = 0;
-  if (valid) chunk_rows(a.bt, c, seq, r0, n);
-  const int64_t rend = valid ? __ldg(a.bt.offsets + seq + 1) : 0;
-  real x = valid ? a.cin[c * D + lane] : real(0);
-  for (int t = n - 1; t >= 0; --t) {
-    const int64_t row = r0 + t;
-    real y = __ldg(a.g + row * D + lane);
-    if (row + 1 < rend) {
-      const real* An = a.A + (row + 1) * (int64_t)(D * D);
+  if (c >= a.bt.n_chunks) return;
+  int64_t seq, r0;
+  int n;
+  chunk_rows(a.bt, c, seq, r0, n);
+  const int64_t rend = __ldg(a.bt.offsets + seq + 1);
+  Ring& R = ring[grp];
 #pragma unroll
-      for (int k = 0; k < D; ++k) y += __ldg(An + k * D + lane) * __shfl_sync(gm, x, k, D);
+  for (int s = 0; s < K; ++s) {
+    if (s < n) adj_issue<real, D>(R, s, lane, a, r0 + n - 1 - s, rend);
+    cp_async_commit();
+  }
+  real x = a.cin[c * D + li];
+  for (int j = 0; j < n; ++j) {
+    const int s = j & (K - 1);
+    const int64_t row = r0 + n - 1 - j;
+    cp_async_wait<K - 1>();
+    __syncwarp(gm);
+    real y = R.v[s][li];
+    if (row + 1 < rend) {
+#pragma unroll
+      for (int k = 0; k < D; ++k) y += R.m[s][k][li] * __shfl_sync(gm, x, k, W);
     }
     x = y;
-    a.lam[row * D + lane] = y;
+    if (lane < D) a.lam[row * D + lane] = y;
+    __syncwarp(gm);
+    if (j + K < n) adj_issue<real, D>(R, s, lane, a, row - K, rend);
+    cp_async_commit();
   }
+  cp_async_wait<0>();
 }
 
 template <class real, int D>
-void adj_launch_wide(const AdjScanArgs<real>& a, cudaStream_t st) {
-  constexpr int G = 128 / D;
+static void adj_launch(const AdjScanArgs<real>& a, cudaStream_t st) {
+  constexpr int G = 32 / group_lanes<D>();
   const unsigned gc = grid_for(a.bt.n_chunks, G);
-  const unsigned gs = grid_for(a.bt.B, G);
-  k_adj_chunk_wide<real, D><<<gc, 128, 0, st>>>(a);
-  k_adj_carry_wide<real, D><<<gs, 128, 0, st>>>(a);
-  k_adj_apply_wide<real, D><<<gc, 128, 0, st>>>(a);
+  if constexpr (D == 32 && sizeof(real) == 4) k_adj_chunk_tile32<<<gc, 32, 0, st>>>(a);
+  else k_adj_chunk_ring<real, D><<<gc, 32, 0, st>>>(a);
+  k_adj_carry_ring<real, D><<<grid_for(a.bt.B, G), 32, 0, st>>>(a);
+  k_adj_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
   note_launch(3);
 }
 
-template void adj_launch_wide<float, 16>(const AdjScanArgs<float>&, cudaStream_t);
-template void adj_launch_wide<float, 32>(const AdjScanArgs<float>&, cudaStream_t);
-template void adj_launch_wide<double, 16>(const AdjScanArgs<double>&, cudaStream_t);
-template void adj_launch_wide<double, 32>(const AdjScanArgs<double>&, cudaStream_t);
+template <class real>
+cudaError_t launch_adjoint_scan(const AdjScanArgs<real>& a, cudaStream_t st) {
+  if (a.bt.N == 0) return cudaSuccess;
+  switch (a.d) {
+    case 1: adj_launch<real, 1>(a, st); break;
+    case 2: adj_launch<real, 2>(a, st); break;
+    case 4: adj_launch<real, 4>(a, st); break;
+    case 5: adj_launch<real, 5>(a, st); break;
+    case 8: adj_launch<real, 8>(a, st); break;
+    case 16: adj_launch<real, 16>(a, st); break;
+    case 32: adj_launch<real, 32>(a, st); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_adjoint_scan<float>(const AdjScanArgs<float>&, cudaStream_t);
+template cudaError_t launch_adjoint_scan<double>(const AdjScanArgs<double>&, cudaStream_t);
 
 }  // namespace deer

@@ -239,6 +239,23 @@ template <class real>
 cudaError_t launch_adjoint_scan(const AdjScanArgs<real>& a, cudaStream_t st);
 
 // Parameter gradient sum_t lambda_t^T df_t/dtheta (s_{t-1}) and dl/ds0 = A_1^T lambda_1.
+// Rate-constant gradient of the mass-action kinetics by lane groups (k_ma_grad.cu): B
+// sequences of T rows
+template <class real>
+struct MaGradArgs {
+  DynView<real> dv;
+  int64_t B, T;
+  const real* s0;    // [B][d]
+  const real* s;     // fixed point [B][T][d]
+  const real* lam;   // adjoints [B][T][d]
+  real* dparams;     // [B][R] (added to)
+  int64_t pstride;   // R
+  int rows = 64;     // rows per group (set by the launcher)
+};
+bool ma_param_grad_supported(int kind, int d, int R);
+template <class real>
+cudaError_t launch_ma_param_grad(const MaGradArgs<real>& a, cudaStream_t st);
+
 template <class real>
 struct ParamGradArgs {
   DynView<real> dv;
@@ -252,6 +269,8 @@ struct ParamGradArgs {
   real* ds0;           // [B][d] or nullptr
 };
 
+template <class real>
+cudaError_t launch_adj_ds0(const ParamGradArgs<real>& a, cudaStream_t st);
 template <class real>
 cudaError_t launch_param_grad(const ParamGradArgs<real>& a, cudaStream_t st);
 
