@@ -114,7 +114,7 @@ struct Layout {
   size_t offsets, chunk_first, win_chunk, act_seq, act_row_off, act_chunk_off, acc, info, flags,
       ma, gru_M,
       A, b, aggP, aggv, cin, mob, pin, sprev, lb_ticket, lb_flags, lb_agg, lb_pre, xproj,
-      adj_off, adj_e, slo, sprev_lo, sbound, fastsel, cov_agg, cov_in, total;
+      adj_off, adj_e, slo, sprev_lo, sbound, fastsel, cov_agg, cov_in, segP, segv, segin, total;
   bool cs;         // compensated float32 state
   bool mixed_rc;   // mixed precision without stored Jacobians
   int64_t n_chunks_max;
@@ -228,6 +228,14 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   if (o->jac == DEER_JAC_FULL) ly.aggP = take((size_t)C * d * d * ars);
   ly.aggv = take((size_t)C * d * ars);
   ly.cin = take((size_t)C * d * ars);
+  ly.segP = ly.segv = ly.segin = p;
+  if (o->jac == DEER_JAC_FULL && d > 1) {
+    // segments of at least 8 chunks (two-level carry)
+    const size_t S = (size_t)(C / 8 + B + 1);
+    ly.segP = take(S * d * d * ars);
+    ly.segv = take(S * d * ars);
+    ly.segin = take(S * d * ars);
+  }
   // diag family also needs a second aggregate array; reuse aggP slot for it
   if (o->jac != DEER_JAC_FULL) ly.aggP = take((size_t)C * d * rs);
   if (o->damp == DEER_DAMP_ELK) {
@@ -550,6 +558,12 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
     dsa.reset_thr = reset_thr;
     dsa.slo = slo;
     dsa.tensor_cores = g_tensor_cores.load();
+    if (d > 1) {
+      dsa.segP = reinterpret_cast<real*>(ws + ly.segP);
+      dsa.segv = reinterpret_cast<real*>(ws + ly.segv);
+      dsa.segin = reinterpret_cast<real*>(ws + ly.segin);
+      dsa.max_chunks = (maxT + ly.L - 1) / ly.L;
+    }
   } else {
     gsa.bt = bt;
     gsa.d = d;
@@ -616,6 +630,10 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
       msa.reset_thr = 1e18;  // the scan and the Jacobians are float32
       msa.tc_mode = g_tensor_cores.load() >= 2 ? 2 : 1;
       msa.status = flags;
+      msa.segP = reinterpret_cast<float*>(ws + ly.segP);
+      msa.segv = reinterpret_cast<float*>(ws + ly.segv);
+      msa.segin = reinterpret_cast<float*>(ws + ly.segin);
+      msa.max_chunks = (maxT + ly.L - 1) / ly.L;
       if (ly.mixed_rc) {
         rca.lin = mla;
         rca.lin.E = nullptr;

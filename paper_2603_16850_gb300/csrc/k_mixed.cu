@@ -333,27 +333,20 @@ __global__ void __launch_bounds__(128) k_mixed_chunk(MixedScanArgs a) {
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(128) k_mixed_carry(MixedScanArgs a) {
-  constexpr int G = 128 / D;
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
-  const unsigned gm = gmask_mixed<D>();
-  const int64_t kq = blockIdx.x * (int64_t)G + grp;
-  const bool valid = kq < a.bt.n_act();
-  const int64_t seq = valid ? a.bt.act_seq[kq] : 0;
-  const int64_t c0 = valid ? win_first(a.bt, seq) : 0;
-  const int64_t c1 = valid ? a.bt.chunk_first[seq + 1] : 0;
-  float x = 0.f;
-  for (int64_t c = c0; c < c1; ++c) {
-    a.cin[c * D + lane] = x;
-    const float* P = a.aggP + c * (int64_t)(D * D);
-    float y = a.aggv[c * D + lane];
-    if (c > c0) {
-#pragma unroll
-      for (int k = 0; k < D; ++k) y += P[lane * D + k] * __shfl_sync(gm, x, k, D);
-    }
-    x = y;
-  }
+// The aggregates are float32: the carry is the dense scans' (one or two levels).
+static cudaError_t mixed_carry(const MixedScanArgs& m, cudaStream_t st) {
+  DenseScanArgs<float> a{};
+  a.bt = m.bt;
+  a.d = m.d;
+  a.aggP = m.aggP;
+  a.aggv = m.aggv;
+  a.cin = m.cin;
+  a.tensor_cores = 1;
+  a.segP = m.segP;
+  a.segv = m.segv;
+  a.segin = m.segin;
+  a.max_chunks = m.max_chunks;
+  return launch_dense_carry(a, st);
 }
 
 template <int D>
@@ -756,11 +749,12 @@ cudaError_t launch_mixed_apply_rc(const MixedRcArgs& a, const MixedScanArgs& car
                                   cudaStream_t st) {
   if (a.lin.bt.act_chunks() == 0) return cudaSuccess;
   if (a.lin.dv.d != 16) return cudaErrorInvalidValue;
-  k_mixed_carry<16><<<grid_for(carry.bt.n_act(), 128 / 16), 128, 0, st>>>(carry);
+  const cudaError_t e = mixed_carry(carry, st);
+  if (e != cudaSuccess) return e;
   const unsigned g = grid_for(a.lin.bt.act_chunks(), kRcWarps);
   if (a.lin.dv.kind == DEER_F_MASSACTION_RK4) k_mixed_apply_rc16<true><<<g, 32 * kRcWarps, 0, st>>>(a);
   else k_mixed_apply_rc16<false><<<g, 32 * kRcWarps, 0, st>>>(a);
-  note_launch(2);
+  note_launch();
   return cudaGetLastError();
 }
 
@@ -783,33 +777,34 @@ cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st) {
 }
 
 template <int D>
-static void mixed_launch(const MixedScanArgs& a, cudaStream_t st) {
-  constexpr int G = 128 / D;
-  const unsigned gs = grid_for(a.bt.n_act(), G);
+static cudaError_t mixed_launch(const MixedScanArgs& a, cudaStream_t st) {
   if constexpr (D == 16) {
     const unsigned gw = grid_for(a.bt.act_chunks(), 4);  // one warp per chunk
     if (a.tc_mode == 2) {
-      if (launch_mixed_chunk_tcgen05(a, st) != cudaSuccess) return;
+      const cudaError_t e = launch_mixed_chunk_tcgen05(a, st);
+      if (e != cudaSuccess) return e;
     } else {
       k_mixed_chunk_tc16<<<gw, 128, 0, st>>>(a);
     }
-    k_mixed_carry<D><<<gs, 128, 0, st>>>(a);
+    const cudaError_t e = mixed_carry(a, st);
+    if (e != cudaSuccess) return e;
     k_mixed_apply_tc16<<<gw, 128, 0, st>>>(a);
   } else {
-    const unsigned gc = grid_for(a.bt.act_chunks(), G);
+    const unsigned gc = grid_for(a.bt.act_chunks(), 128 / D);
     k_mixed_chunk<D><<<gc, 128, 0, st>>>(a);
-    k_mixed_carry<D><<<gs, 128, 0, st>>>(a);
+    const cudaError_t e = mixed_carry(a, st);
+    if (e != cudaSuccess) return e;
     k_mixed_apply<D><<<gc, 128, 0, st>>>(a);
   }
-  note_launch(3);
+  note_launch(2);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dense_scan_mixed(const MixedScanArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
-  if (a.d == 16) mixed_launch<16>(a, st);
-  else if (a.d == 32) mixed_launch<32>(a, st);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (a.d == 16) return mixed_launch<16>(a, st);
+  if (a.d == 32) return mixed_launch<32>(a, st);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace deer

@@ -525,11 +525,52 @@ struct RowRing {
   }
 };
 
+// What one group folds: rows r0 .. r0 + n - 1 of (A, b) into aggregate `out`. SEG = false: a
+// chunk of rows into the chunk aggregates; SEG = true: a segment of consecutive chunk
+// aggregates of one active sequence (blockIdx.y) into the segment aggregates.
+struct Span {
+  int64_t r0, out;
+  int n;
+  bool need_P;
+};
+
+template <bool SEG, class real>
+__device__ __forceinline__ bool get_span(const DenseScanArgs<real>& a, int64_t idx, Span& p) {
+  if constexpr (!SEG) {
+    if (idx >= a.bt.act_chunks()) return false;
+    int64_t seq;
+    act_chunk(a.bt, idx, seq, p.out, p.r0, p.n);
+    p.need_P = p.out != win_first(a.bt, seq);
+  } else {
+    if ((int64_t)blockIdx.y >= a.bt.n_act()) return false;
+    const int64_t seq = __ldg(a.bt.act_seq + blockIdx.y);
+    const int64_t c1 = __ldg(a.bt.chunk_first + seq + 1);
+    p.r0 = win_first(a.bt, seq) + (idx << a.log2M);
+    if (p.r0 >= c1) return false;
+    p.n = (int)(c1 - p.r0 < (1 << a.log2M) ? c1 - p.r0 : (1 << a.log2M));
+    p.need_P = idx > 0;
+    // sequence b's segments start at chunk_first[b] / M + b: disjoint, since
+    // floor(x + y) + 1 >= floor(x) + ceil(y)
+    p.out = (__ldg(a.bt.chunk_first + seq) >> a.log2M) + seq + idx;
+  }
+  return true;
+}
+
+template <bool SEG, class real, int D>
+__device__ __forceinline__ void span_ptrs(const DenseScanArgs<real>& a, const Span& p,
+                                          const real*& A0, const real*& b0, real*& Po,
+                                          real*& vo) {
+  A0 = (SEG ? a.aggP : a.A) + p.r0 * (int64_t)(D * D);
+  b0 = (SEG ? a.aggv : a.b) + p.r0 * D;
+  Po = (SEG ? a.segP : a.aggP) + p.out * (int64_t)(D * D);
+  vo = (SEG ? a.segv : a.aggv) + p.out * D;
+}
+
 // Chunk pass: one group of D lanes per chunk (one warp per block), lane j owns
 // column j of the chunk product P and entry j of the vector part. Row t's Jacobian is
 // staged in the ring; every lane reads all of its rows (broadcast) for P <- A_t P and
 // its own row for v <- A_t v + b_t.
-template <class real, int D>
+template <class real, int D, bool SEG>
 __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) {
   constexpr int W = group_lanes<D>(), G = 32 / W;
   using Ring = RowRing<real, D>;
@@ -539,15 +580,15 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
   const int grp = threadIdx.x / W, lane = threadIdx.x % W;
   const int li = lane < D ? lane : 0;  // this lane's row / column
   const unsigned gm = group_mask<D>();
-  const int64_t ac = blockIdx.x * (int64_t)G + grp;
-  if (ac >= a.bt.act_chunks()) return;  // whole groups; groups never synchronise with each other
-  int64_t seq, c, r0;
-  int n;
-  act_chunk(a.bt, ac, seq, c, r0, n);
-  const bool need_P = c != win_first(a.bt, seq);
+  Span p;
+  if (!get_span<SEG>(a, blockIdx.x * (int64_t)G + grp, p))
+    return;  // whole groups; groups never synchronise with each other
+  const real *A0, *b0;
+  real *Po, *vo;
+  span_ptrs<SEG, real, D>(a, p, A0, b0, Po, vo);
+  const int n = p.n;
+  const bool need_P = p.need_P;
   Ring& R = ring[grp];
-  const real* A0 = a.A + r0 * (int64_t)(D * D);
-  const real* b0 = a.b + r0 * D;
 #pragma unroll
   for (int s = 0; s < K; ++s) {
     if (s < n) R.issue(s, lane, A0 + s * (int64_t)(D * D), b0 + s * D);
@@ -592,10 +633,9 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
   }
   cp_async_wait<0>();
   if (lane >= D) return;
-  real* Po = a.aggP + c * (int64_t)(D * D);
 #pragma unroll
   for (int i = 0; i < D; ++i) Po[i * D + lane] = Pc[i];
-  a.aggv[c * D + lane] = v;
+  vo[lane] = v;
 }
 
 // Chunk pass, d = 32: one chunk per block of four warps. The staged rows of A_t are shared
@@ -605,7 +645,7 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
 // v <- A_t v + b_t is formed redundantly by every warp (lane i, row i). A quarter of the
 // dependent work per warp compared with one warp per chunk, and four times the warps:
 // the single long sequences that leave few chunks stay busy.
-template <class real>
+template <class real, bool SEG>
 __global__ void __launch_bounds__(128) k_dense_chunk_ring4(DenseScanArgs<real> a) {
   constexpr int D = 32;
   constexpr int W = 4;                       // warps per chunk
@@ -618,19 +658,18 @@ __global__ void __launch_bounds__(128) k_dense_chunk_ring4(DenseScanArgs<real> a
   __shared__ __align__(16) real sB[K][D];
   __shared__ real sP[D][D + 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t ac = blockIdx.x;
-  if (ac >= a.bt.act_chunks()) return;  // uniform over the block
-  int64_t seq, c, r0;
-  int n;
-  act_chunk(a.bt, ac, seq, c, r0, n);
-  const bool need_P = c != win_first(a.bt, seq);
-  const real* A0 = a.A + r0 * (int64_t)(D * D);
-  const real* b0 = a.b + r0 * D;
+  Span p;
+  if (!get_span<SEG>(a, blockIdx.x, p)) return;  // uniform over the block
+  const real *A0, *b0;
+  real *Po, *vo;
+  span_ptrs<SEG, real, D>(a, p, A0, b0, Po, vo);
+  const int n = p.n;
+  const bool need_P = p.need_P;
   auto issue = [&](int slot, int t) {
     if (t < n) {
       const real* src = A0 + t * (int64_t)(D * D);
-      for (int p = tid; p < PIECES; p += 128)
-        cp_async16(&sA[slot][p / (D / VW)][(p % (D / VW)) * VW], src + p * VW);
+      for (int q = tid; q < PIECES; q += 128)
+        cp_async16(&sA[slot][q / (D / VW)][(q % (D / VW)) * VW], src + q * VW);
       if (tid < D / VW) cp_async16(&sB[slot][tid * VW], b0 + t * D + tid * VW);
     }
     cp_async_commit();
@@ -681,10 +720,9 @@ __global__ void __launch_bounds__(128) k_dense_chunk_ring4(DenseScanArgs<real> a
   }
   cp_async_wait<0>();
   if (warp == 0) {
-    real* Po = a.aggP + c * (int64_t)(D * D);
 #pragma unroll
     for (int i = 0; i < D; ++i) Po[i * D + lane] = Pc[i];
-    a.aggv[c * D + lane] = v;
+    vo[lane] = v;
   }
 }
 
@@ -701,6 +739,7 @@ __global__ void __launch_bounds__(128) k_dense_chunk_ring4(DenseScanArgs<real> a
 // the 32 lanes' words fall in distinct banks). The vector part v <- A_t v + b_t is formed
 // by lane i (row i) of warp 0. Rows are staged through the same cp.async ring as
 // k_dense_chunk_ring4.
+template <bool SEG>
 __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a) {
   constexpr int D = 32;
   constexpr int K = ring_depth<float>();
@@ -710,19 +749,18 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
   __shared__ __align__(16) float sB[K][D];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tq = lane & 3;
-  const int64_t ac = blockIdx.x;
-  if (ac >= a.bt.act_chunks()) return;  // uniform over the block
-  int64_t seq, c, r0;
-  int n;
-  act_chunk(a.bt, ac, seq, c, r0, n);
-  const bool need_P = c != win_first(a.bt, seq);
-  const float* A0 = a.A + r0 * (int64_t)(D * D);
-  const float* b0 = a.b + r0 * D;
+  Span p;
+  if (!get_span<SEG>(a, blockIdx.x, p)) return;  // uniform over the block
+  const float *A0, *b0;
+  float *Po, *vo;
+  span_ptrs<SEG, float, D>(a, p, A0, b0, Po, vo);
+  const int n = p.n;
+  const bool need_P = p.need_P;
   auto issue = [&](int slot, int t) {
     if (t < n) {
       const float* src = A0 + t * (int64_t)(D * D);
-      for (int p = tid; p < PIECES; p += 64)
-        cp_async16(&sA[slot][p / (D / 4)][(p % (D / 4)) * 4], src + p * 4);
+      for (int q = tid; q < PIECES; q += 64)
+        cp_async16(&sA[slot][q / (D / 4)][(q % (D / 4)) * 4], src + q * 4);
       if (tid < D / 4) cp_async16(&sB[slot][tid * 4], b0 + t * D + tid * 4);
     }
     cp_async_commit();
@@ -807,7 +845,6 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
   }
   cp_async_wait<0>();
   // P[i][j] = P^T[j][i]
-  float* Po = a.aggP + c * (int64_t)(D * D);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int n0 = 8 * j + 2 * tq;
@@ -816,12 +853,18 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
     Po[n0 * D + m0 + 8] = acc[j][2];
     Po[(n0 + 1) * D + m0 + 8] = acc[j][3];
   }
-  if (warp == 0) a.aggv[c * D + lane] = v;
+  if (warp == 0) vo[lane] = v;
 }
 
-// Carry pass: x_c = P_c x_{c-1} + v_c along each active sequence's chunks (one group per
-// sequence); the aggregates do not depend on x and stream through the ring.
-template <class real, int D>
+// Carry pass: x_c = P_c x_{c-1} + v_c along each active sequence's chunks; the aggregates do
+// not depend on x and stream through the ring. MODE 0: one group per sequence, over its
+// chunks. Few sequences of many chunks make that the longest chain of the iteration (3125
+// chunks of the mean-field RNN, d = 32, T = 100000: 580 us); the chunks are then folded into
+// segments of M (the chunk pass again, over the aggregates), MODE 1 walks a sequence's
+// segments, MODE 2 the chunks of each segment from the value entering it: 39 + 20 + 10 us
+// there. (Mixed-precision ragged batch, d = 16, up to 3125 chunks a sequence: 134 -> 27 ms of
+// scans per solve, against a carry that loaded each aggregate when it needed it.)
+template <class real, int D, int MODE>
 __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) {
   constexpr int W = group_lanes<D>(), G = 32 / W;
   using Ring = RowRing<real, D>;
@@ -831,16 +874,36 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
   const int li = lane < D ? lane : 0;  // this lane's row
   const unsigned gm = group_mask<D>();
   const int64_t kq = blockIdx.x * (int64_t)G + grp;
-  if (kq >= a.bt.n_act()) return;
-  const int64_t seq = a.bt.act_seq[kq];
-  const int64_t c0 = win_first(a.bt, seq), c1 = a.bt.chunk_first[seq + 1];
+  const real* P = MODE == 1 ? a.segP : a.aggP;
+  const real* v = MODE == 1 ? a.segv : a.aggv;
+  real* in = MODE == 1 ? a.segin : a.cin;
+  int64_t c0, c1;
+  real x = real(0);
+  bool first = true;  // c0 starts from Delta = 0: its aggregate has no P
+  if constexpr (MODE == 2) {
+    Span p;
+    if (!get_span<true>(a, kq, p)) return;
+    c0 = p.r0;
+    c1 = p.r0 + p.n;
+    first = !p.need_P;
+    x = a.segin[p.out * D + li];
+  } else {
+    if (kq >= a.bt.n_act()) return;
+    const int64_t seq = a.bt.act_seq[kq];
+    c0 = win_first(a.bt, seq);
+    c1 = a.bt.chunk_first[seq + 1];
+    if constexpr (MODE == 1) {
+      const int64_t nseg = (c1 - c0 + (1 << a.log2M) - 1) >> a.log2M;
+      c0 = (a.bt.chunk_first[seq] >> a.log2M) + seq;
+      c1 = c0 + nseg;
+    }
+  }
   Ring& R = ring[grp];
 #pragma unroll
   for (int s = 0; s < K; ++s) {
-    if (c0 + s < c1) R.issue(s, lane, a.aggP + (c0 + s) * (int64_t)(D * D), a.aggv + (c0 + s) * D);
+    if (c0 + s < c1) R.issue(s, lane, P + (c0 + s) * (int64_t)(D * D), v + (c0 + s) * D);
     cp_async_commit();
   }
-  real x = real(0);
   for (int64_t cb = c0; cb < c1; cb += K) {
 #pragma unroll
     for (int s = 0; s < K; ++s) {
@@ -848,9 +911,9 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
       cp_async_wait<K - 1>();
       __syncwarp(gm);  // the other lanes' pieces of this slot have landed
       if (c < c1) {
-        if (lane < D) a.cin[c * D + lane] = x;
+        if (lane < D) in[c * D + lane] = x;
         real y = R.v[s][li];
-        if (c > c0) {
+        if (!first || c > c0) {
           real pr[D];
           R.row(s, li, pr);
 #pragma unroll
@@ -859,7 +922,8 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
         x = y;
       }
       __syncwarp(gm);  // every lane is done with the slot before it is refilled
-      if (c + K < c1) R.issue(s, lane, a.aggP + (c + K) * (int64_t)(D * D), a.aggv + (c + K) * D);
+      if (c + K < c1)
+        R.issue(s, lane, P + (c + K) * (int64_t)(D * D), v + (c + K) * D);
       cp_async_commit();
     }
   }
@@ -874,6 +938,7 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
   using Ring = RowRing<real, D>;
   constexpr int K = Ring::K;
   __shared__ __align__(16) Ring ring[G];
+  __shared__ real st[G][K][2][W];  // the rows' states (and compensation), staged with them
   const int grp = threadIdx.x / W, lane = threadIdx.x % W;
   const int li = lane < D ? lane : 0;  // this lane's row
   const unsigned gm = group_mask<D>();
@@ -885,11 +950,18 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
   const real* A0 = a.A + r0 * (int64_t)(D * D);
   const real* b0 = a.b + r0 * D;
   Ring& R = ring[grp];
-#pragma unroll
-  for (int s = 0; s < K; ++s) {
-    if (s < n) R.issue(s, lane, A0 + s * (int64_t)(D * D), b0 + s * D);
+  real* s0 = a.s + r0 * D + li;
+  real* l0 = a.slo ? a.slo + r0 * D + li : nullptr;
+  auto issue = [&](int s, int t) {
+    if (t < n) {
+      R.issue(s, lane, A0 + t * (int64_t)(D * D), b0 + t * D);
+      cp_async_small<sizeof(real)>(&st[grp][s][0][lane], s0 + t * D);
+      if (l0) cp_async_small<sizeof(real)>(&st[grp][s][1][lane], l0 + t * D);
+    }
     cp_async_commit();
-  }
+  };
+#pragma unroll
+  for (int s = 0; s < K; ++s) issue(s, s);
   real x = a.cin[c * D + li];
   for (int t0 = 0; t0 < n; t0 += K) {
 #pragma unroll
@@ -904,26 +976,25 @@ __global__ void __launch_bounds__(32) k_dense_apply_ring(DenseScanArgs<real> a) 
 #pragma unroll
         for (int k = 0; k < D; ++k) y += ar[k] * __shfl_sync(gm, x, k, W);
         x = y;
-        real* sp = a.s + (r0 + t) * D + li;
+        const real so = st[grp][s][0][lane];
         if (lane >= D) {
           // idle lane (d = 5)
-        } else if (a.slo) {
+        } else if (l0) {
           // compensated state: (s, slo) += Delta with error-free transformations
-          real hi = *sp, lo = a.slo[(r0 + t) * D + lane];
+          real hi = so, lo = st[grp][s][1][lane];
           cs_add(hi, lo, y);
           if (a.reset && !(hi <= a.reset_thr && hi >= -a.reset_thr)) {
             hi = real(0);
             lo = real(0);
           }
-          *sp = hi;
-          a.slo[(r0 + t) * D + lane] = lo;
+          s0[t * D] = hi;
+          l0[t * D] = lo;
         } else {
-          *sp = reset_val(*sp + y, a.reset_thr, a.reset);
+          s0[t * D] = reset_val(so + y, a.reset_thr, a.reset);
         }
       }
       __syncwarp(gm);
-      if (t + K < n) R.issue(s, lane, A0 + (t + K) * (int64_t)(D * D), b0 + (t + K) * D);
-      cp_async_commit();
+      issue(s, t + K);
     }
   }
   cp_async_wait<0>();
@@ -975,33 +1046,77 @@ __global__ void __launch_bounds__(128) k_scalar_apply(DenseScanArgs<real> a) {
   }
 }
 
+// Segments shorten the carry when few sequences have many chunks: a chain of n steps becomes
+// M + n / M + M with M about sqrt(n), at the price of folding the aggregates once more. At
+// 157 chunks (Langevin, d = 4, float64) 28 us against 40 in one level; below 128 the two
+// extra launches cost what is saved. More sequences than SM sub-partitions x groups per warp
+// hide the chain by themselves.
+template <class real, int D>
+static void set_segments(DenseScanArgs<real>& a) {
+  a.log2M = 0;
+  const int64_t n = a.max_chunks;
+  if (!a.segP || n < 128 || a.bt.n_act() > 608 * (32 / group_lanes<D>())) return;
+  a.log2M = 3;
+  while (a.log2M < 6 && ((int64_t)1 << (2 * a.log2M + 2)) <= n) ++a.log2M;
+}
+
+template <class real, int D, bool SEG>
+static void dense_chunk_launch(const DenseScanArgs<real>& a, int64_t spans, unsigned ny,
+                               cudaStream_t st) {
+  constexpr int G = D == 32 ? 1 : 32 / group_lanes<D>();
+  const dim3 g(grid_for(spans, G), ny);
+  if constexpr (D == 32) {
+    if constexpr (sizeof(real) == 4) {
+      if (a.tensor_cores) {
+        k_dense_chunk_mma32<SEG><<<g, 64, 0, st>>>(a);
+        return;
+      }
+    }
+    k_dense_chunk_ring4<real, SEG><<<g, 128, 0, st>>>(a);
+  } else {
+    k_dense_chunk_ring<real, D, SEG><<<g, 32, 0, st>>>(a);
+  }
+}
+
+template <class real, int D>
+static void dense_carry(DenseScanArgs<real> a, cudaStream_t st) {
+  constexpr int G = 32 / group_lanes<D>();
+  set_segments<real, D>(a);
+  if (a.log2M == 0) {
+    k_dense_carry_ring<real, D, 0><<<grid_for(a.bt.n_act(), G), 32, 0, st>>>(a);
+    note_launch();
+    return;
+  }
+  const int64_t segs = (a.max_chunks + (1 << a.log2M) - 1) >> a.log2M;
+  const unsigned ny = (unsigned)a.bt.n_act();
+  dense_chunk_launch<real, D, true>(a, segs, ny, st);
+  k_dense_carry_ring<real, D, 1><<<grid_for(a.bt.n_act(), G), 32, 0, st>>>(a);
+  k_dense_carry_ring<real, D, 2><<<dim3(grid_for(segs, G), ny), 32, 0, st>>>(a);
+  note_launch(3);
+}
+
+cudaError_t launch_dense_carry(const DenseScanArgs<float>& a, cudaStream_t st) {
+  if (a.bt.n_act() == 0) return cudaSuccess;
+  if (a.d == 16) dense_carry<float, 16>(a, st);
+  else if (a.d == 32) dense_carry<float, 32>(a, st);
+  else return cudaErrorInvalidValue;
+  return cudaGetLastError();
+}
+
 template <class real, int D>
 static void dense_launch(const DenseScanArgs<real>& a, cudaStream_t st) {
-  constexpr int G = D == 1 ? 128 : 32 / group_lanes<D>();
-  const unsigned gc = grid_for(a.bt.act_chunks(), G);
-  const unsigned gs = grid_for(a.bt.n_act(), G);
   if constexpr (D == 1) {
+    const unsigned gc = grid_for(a.bt.act_chunks(), 128);
     k_scalar_chunk<real><<<gc, 128, 0, st>>>(a);
-    k_scalar_carry<real><<<gs, 128, 0, st>>>(a);
+    k_scalar_carry<real><<<grid_for(a.bt.n_act(), 128), 128, 0, st>>>(a);
     k_scalar_apply<real><<<gc, 128, 0, st>>>(a);
     note_launch(3);
-    return;
-  } else if constexpr (D == 32) {
-    if constexpr (sizeof(real) == 4) {
-      if (a.tensor_cores)
-        k_dense_chunk_mma32<<<grid_for(a.bt.act_chunks(), 1), 64, 0, st>>>(a);
-      else
-        k_dense_chunk_ring4<real><<<grid_for(a.bt.act_chunks(), 1), 128, 0, st>>>(a);
-    } else {
-      k_dense_chunk_ring4<real><<<grid_for(a.bt.act_chunks(), 1), 128, 0, st>>>(a);
-    }
   } else {
-    k_dense_chunk_ring<real, D><<<gc, 32, 0, st>>>(a);
-  }
-  if constexpr (D > 1) {
-    k_dense_carry_ring<real, D><<<gs, 32, 0, st>>>(a);
-    k_dense_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
-    note_launch(3);
+    dense_chunk_launch<real, D, false>(a, a.bt.act_chunks(), 1, st);
+    dense_carry<real, D>(a, st);
+    k_dense_apply_ring<real, D>
+        <<<grid_for(a.bt.act_chunks(), 32 / group_lanes<D>()), 32, 0, st>>>(a);
+    note_launch(2);
   }
 }
 

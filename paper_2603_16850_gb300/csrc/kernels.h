@@ -137,6 +137,13 @@ struct DenseScanArgs {
   real reset_thr;
   real* slo = nullptr;  // compensation of s ([N][d]): s + slo += Delta exactly; nullptr = off
   int tensor_cores = 0;  // d = 32 float32: chunk products on the tensor cores
+  // two-level carry of few sequences with many chunks: aggregates of segments of M chunks
+  // and the carry into each ([n_chunks / 8 + B + 1] each); nullptr = one level
+  real* segP = nullptr;
+  real* segv = nullptr;
+  real* segin = nullptr;
+  int64_t max_chunks = 0;  // chunks of the longest sequence
+  int log2M = 0;           // segment length (set by the launcher)
 };
 
 // Diagonal-family scan in standard form: s_t = a_t s_{t-1} + b_t from s_0, where a_t is
@@ -442,6 +449,11 @@ struct MixedScanArgs {
   int tc_mode = 1;          // d = 16 chunk pass: 1 warp-level bf16 MMAs, 2 tcgen05
                             // block-diagonal MMAs (8 chunks per CTA)
   Flags* status = nullptr;  // timeout flag of the bounded waits (tcgen05 variant)
+  // two-level carry, as in DenseScanArgs
+  float* segP = nullptr;
+  float* segv = nullptr;
+  float* segin = nullptr;
+  int64_t max_chunks = 0;
 };
 
 // Mixed-precision iteration without stored Jacobians (d = 16): the linearisation of each
@@ -461,6 +473,9 @@ struct MixedRcArgs {
 };
 
 cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st);
+// carry pass of the dense scans alone (d = 16, 32), over aggregates formed elsewhere
+cudaError_t launch_dense_carry(const DenseScanArgs<float>& a, cudaStream_t st);
+
 cudaError_t launch_mixed_lin_agg(const MixedRcArgs& a, cudaStream_t st);
 cudaError_t launch_mixed_apply_rc(const MixedRcArgs& a, const MixedScanArgs& carry,
                                   cudaStream_t st);
