@@ -10,13 +10,26 @@
 // relative error about 2^-21 per product, so the residual the Newton iteration is refined
 // against keeps float32 accuracy.
 //
-// One persistent CTA per SM (192 KB of shared memory): the weights are split and staged
-// once in the canonical no-swizzle K-major layout; each tile stages its activations
-// (h, then r o h, then h o r o (1 - r)) into the same layout and one thread issues the
-// MMAs; the 16 warps read the accumulators with tcgen05.ld (warp w reads tensor-memory
-// lanes 32 (w % 4) .. + 31 = tile rows, a quarter w / 4 of the columns) for the gates, the
-// diagonal Jacobian and the residual; h and r stay in registers across the three stages. Every mbarrier wait is bounded; a wait that gives up sets the
-// timeout flag and the kernel winds down, freeing its tensor memory.
+// One persistent CTA of 16 warps per SM. Shared memory (224 KB) holds the weights, split and
+// staged once in the canonical no-swizzle K-major layout, and three 32 KB row buffers; the
+// activations (h, then r o h and h o r o (1 - r)) are split straight into tensor memory, where
+// the MMAs read their A operand, beside the accumulators (all 512 columns). Warp w works on
+// tensor-memory lanes 32 (w % 4) .. + 31 = tile rows and a quarter w / 4 of the columns.
+//
+// What bounds a tile of 128 rows is its 196 KB of rows (s twice, three input projections, a
+// and b written: about 9100 clocks of HBM time per SM) and the gates' arithmetic (about 8000
+// issue slots per scheduler), not the MMAs (3300 clocks). So a warp's part of the row buffers
+// (its 32 rows x 16 columns of each) is its own: it is filled by cp.async in 64-byte row
+// segments ahead of use and emptied without a barrier (pieces swizzled by row),
+//   buffer 0: h, then s; the next tile's h while this tile's gates are formed
+//   buffer 1: r's projection, then h~'s; the next tile's r
+//   buffer 2: z's projection, then a, then b on their way out; the next tile's z
+// and only the two hand-overs of operands to the tensor core are block-wide. Two threads of
+// different warps issue half of the products each. Per pass over 4.19 M rows: 3.76 ms with
+// every thread reading its own row (32 rows per instruction) and the three products back to
+// back, 2.42 ms so (39 % of issue slots: four warps per scheduler, dependent gate arithmetic).
+// Every mbarrier wait is bounded; a wait that gives up sets the timeout flag and the kernel
+// winds down, freeing its tensor memory.
 #include "kernels.h"
 #include "tc.cuh"
 
@@ -29,7 +42,11 @@ constexpr int kD = 64;        // state size = input size
 constexpr int kTM = 128;      // rows per tile = MMA M
 constexpr int kThreads = 512;  // 16 warps: lane quadrant w % 4, column quarter w / 4
 constexpr int kCols = kD / 4;   // columns of each 64-wide block per thread
-constexpr uint32_t kTmemCols = 256;  // D1: 128 columns, D2: 64, D3: 64
+// tensor memory: D1 (z, r) 128 columns, D2 64, D3 64, operands h / r o h (hi, lo) 128 and
+// h o r o (1 - r) (hi, lo) 128
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kColA = 256, kColA3 = 384;
+constexpr uint32_t kNoRow = 0xffffffffu;
 constexpr unsigned kWaitLimit = 1u << 24;
 
 // Canonical no-swizzle K-major layout of an R x 64 float32 operand: core matrices of
@@ -44,7 +61,7 @@ struct TcSmem {
   float B1h[128 * kD], B1l[128 * kD];  // [Uz; Ur]
   float B2h[kD * kD], B2l[kD * kD];    // Uh
   float B3h[kD * kD], B3l[kD * kD];    // M
-  float Ah[kTM * kD], Al[kTM * kD];    // activations
+  float buf[3][16][32 * kCols];        // row buffers by warp, 16-byte pieces swizzled by row
 };
 
 __device__ __forceinline__ float tf32_hi(float x) {
@@ -63,20 +80,38 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   return tc::bar_wait(bar, parity, kWaitLimit);
 }
 
-// D (+)= A B^T over K = 64 with the three-term split: 8 K-steps of 8 (two core matrices)
-__device__ __forceinline__ void gemm3(uint32_t dtmem, const float* Ah, const float* Al,
-                                      const float* Bh, const float* Bl, int N) {
-  const uint32_t idesc = idesc_tf32(N, kTM);
-  const uint32_t lboA = (kTM / 8) * 128, lboB = (uint32_t)(N / 8) * 128, sbo = 128;
-  const uint32_t ah = su32(Ah), al = su32(Al), bh = su32(Bh), bl = su32(Bl);
+// D (+)= A B^T (64 outputs) over K = 64 with the three-term split: 8 K-steps of 8 (two core
+// matrices of B, whose operand has R rows and whose row `r0` is the first output; eight
+// tensor-memory columns of A, hi at `a`, lo 64 columns on)
+__device__ __forceinline__ void gemm3(uint32_t dtmem, uint32_t a, const float* Bh,
+                                      const float* Bl, int R, int r0) {
+  const uint32_t idesc = idesc_tf32(kD, kTM);
+  const uint32_t lboB = (uint32_t)(R / 8) * 128, sbo = 128;
+  const uint32_t bh = su32(Bh) + r0 / 8 * 128, bl = su32(Bl) + r0 / 8 * 128;
 #pragma unroll
   for (int s = 0; s < kD / 8; ++s) {
-    const uint32_t ao = (uint32_t)s * 2 * lboA, bo = (uint32_t)s * 2 * lboB;
-    mma_tf32(dtmem, sdesc(ah + ao, lboA, sbo), sdesc(bh + bo, lboB, sbo), idesc, s > 0);
-    mma_tf32(dtmem, sdesc(ah + ao, lboA, sbo), sdesc(bl + bo, lboB, sbo), idesc, 1u);
-    mma_tf32(dtmem, sdesc(al + ao, lboA, sbo), sdesc(bh + bo, lboB, sbo), idesc, 1u);
+    const uint32_t bo = (uint32_t)s * 2 * lboB;
+    mma_tf32_ts(dtmem, a + 8 * s, sdesc(bh + bo, lboB, sbo), idesc, s > 0);
+    mma_tf32_ts(dtmem, a + 8 * s, sdesc(bl + bo, lboB, sbo), idesc, 1u);
+    mma_tf32_ts(dtmem, a + kD + 8 * s, sdesc(bh + bo, lboB, sbo), idesc, 1u);
   }
 }
+
+// the split of 16 values into an operand's hi and lo columns of this thread's lane
+__device__ __forceinline__ void split_tmem(uint32_t taddr, const float (&v)[kCols]) {
+  float h[kCols], l[kCols];
+#pragma unroll
+  for (int j = 0; j < kCols; ++j) {
+    h[j] = tf32_hi(v[j]);
+    l[j] = v[j] - h[j];
+  }
+  tmem_st16(taddr, h);
+  tmem_st16(taddr + kD, l);
+}
+
+// float offset of piece p (four columns) of row r in a warp's part of a row buffer: eight
+// rows' equal pieces fall in distinct banks
+__device__ __forceinline__ int piece(int r, int p) { return r * kCols + ((p ^ ((r >> 1) & 3)) << 2); }
 
 __device__ __forceinline__ float fsig(float v) { return 1.f / (1.f + __expf(-v)); }
 
@@ -89,11 +124,10 @@ __device__ __forceinline__ float4 ldg4(const float* p) {
 __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>(smraw);
-  __shared__ float diag_z[kD], diag_h[kD];
-  __shared__ float rmx[kTM], rsq[kTM];
+  __shared__ float2 s_diag[kD];  // diagonals of Uz and Uh
   __shared__ __align__(8) unsigned long long mbar;
   __shared__ uint32_t tmem_base_sh;
-  __shared__ int s_ok;
+  __shared__ int s_ok1, s_ok2;  // the waits for the first / the other two products succeeded
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int qd = warp & 3, qc = warp >> 2;
   const int rl = 32 * qd + lane;  // tile row = tensor-memory lane
@@ -109,14 +143,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
     split_store4(S.B2h, S.B2l, core_off(kD, i, k), ldg4(Uh + i * kD + k));
     split_store4(S.B3h, S.B3l, core_off(kD, i, k), ldg4(a.dv.gru_M + i * kD + k));
   }
-  if (tid < kD) {
-    diag_z[tid] = Uz[tid * kD + tid];
-    diag_h[tid] = Uh[tid * kD + tid];
-  }
+  if (tid < kD) s_diag[tid] = make_float2(Uz[tid * kD + tid], Uh[tid * kD + tid]);
   const uint32_t bar = su32(&mbar);
   if (tid == 0) {
-    s_ok = 1;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    s_ok1 = s_ok2 = 1;
+    // two issuing threads commit per phase
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -126,6 +158,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  const int64_t act_rows = a.bt.act_rows();
+  const int64_t n_tiles = (act_rows + kTM - 1) / kTM;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   fence_before();
   __syncthreads();
@@ -134,92 +168,152 @@ __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
   const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16);  // this warp's lanes, column 0
   uint32_t phase = 0, last = 0;
   const float kk = a.dparam;
-
-  // make this thread's staged activations visible to the tensor core, let one thread
-  // issue the products of a stage, and wait (bounded) for them
-  auto run_stage = [&](int which) -> bool {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  float* B0 = S.buf[0][warp];
+  float* B1 = S.buf[1][warp];
+  float* B2 = S.buf[2][warp];
+  // this lane's row of a tile: 2 row + (1 if the first of its sequence), kNoRow past the end
+  auto find_row = [&](int64_t tile, uint32_t& code, int64_t& seq) {
+    const int64_t ar = tile * kTM + rl;
+    code = kNoRow;
+    seq = 0;
+    if (tile < n_tiles && ar < act_rows) {
+      int64_t row;
+      act_row(a.bt, ar, seq, row);
+      code = 2 * (uint32_t)row + (row == __ldg(a.bt.offsets + seq) ? 1u : 0u);
+    }
+  };
+  // copy the warp's rows (16 columns each, four lanes per row) into its part of a buffer
+  enum { SRC_H, SRC_S, SRC_XZ, SRC_XR, SRC_XH };
+  auto copy_rows = [&](float* B, int src, uint32_t code, int64_t seq) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = 8 * q + (lane >> 2), p = lane & 3;
+      const uint32_t cr = __shfl_sync(0xffffffffu, code, r);
+      const int64_t row = cr >> 1;
+      const float* g;
+      if (src == SRC_H) {
+        const int64_t sr = __shfl_sync(0xffffffffu, (long long)seq, r);
+        g = (cr & 1u) ? a.s0 + sr * kD : a.s + (row - 1) * kD;
+      } else if (src == SRC_S) {
+        g = a.s + row * kD;
+      } else {
+        g = a.xproj + row * (3 * kD) + (src == SRC_XZ ? 0 : src == SRC_XR ? kD : 2 * kD);
+      }
+      if (cr != kNoRow) cp_async16(B + piece(r, p), g + c0 + 4 * p);
+    }
+  };
+  auto read16 = [&](const float* B, float (&v)[kCols]) {
+#pragma unroll
+    for (int p = 0; p < kCols / 4; ++p) {
+      const float4 x = *reinterpret_cast<const float4*>(B + piece(lane, p));
+      v[4 * p] = x.x; v[4 * p + 1] = x.y; v[4 * p + 2] = x.z; v[4 * p + 3] = x.w;
+    }
+  };
+  // the warp's part of buffer 2, filled with this lane's 16 values, to its rows of `dst`
+  auto rows_out = [&](const float (&v)[kCols], float* dst, uint32_t code) {
+    __syncwarp();
+#pragma unroll
+    for (int p = 0; p < kCols / 4; ++p)
+      *reinterpret_cast<float4*>(B2 + piece(lane, p)) =
+          make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = 8 * q + (lane >> 2), p = lane & 3;
+      const uint32_t cr = __shfl_sync(0xffffffffu, code, r);
+      if (cr != kNoRow)
+        *reinterpret_cast<float4*>(dst + (int64_t)(cr >> 1) * kD + c0 + 4 * p) =
+            *reinterpret_cast<const float4*>(B2 + piece(r, p));
+    }
+  };
+  // wait (bounded) for the products committed last
+  auto wait_mma = [&](int& flag) {
+    last = phase;
+    if (!bar_wait(bar, last)) flag = 0;
+    phase ^= 1u;
+    fence_after();
+  };
+  // operands complete in tensor memory: hand over to the issuing threads
+  auto hand_over = [&]() {
+    tmem_wait_st();
     fence_before();
     __syncthreads();
     fence_after();
-    if (tid == 0) {
-      if (which == 1) gemm3(tmem, S.Ah, S.Al, S.B1h, S.B1l, 128);
-      else if (which == 2) gemm3(tmem + 128, S.Ah, S.Al, S.B2h, S.B2l, kD);
-      else gemm3(tmem + 192, S.Ah, S.Al, S.B3h, S.B3l, kD);
+  };
+  const bool issuer = tid == 0 || tid == 128;
+
+  uint32_t code;
+  int64_t seq;
+  find_row(blockIdx.x, code, seq);
+  copy_rows(B0, SRC_H, code, seq);
+  copy_rows(B1, SRC_XR, code, seq);
+  cp_async_commit();
+  copy_rows(B2, SRC_XZ, code, seq);
+  cp_async_commit();
+  bool ok = true;
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const bool v = code != kNoRow;
+    // stage 1: h into tensor memory, [z; r] products
+    float h[kCols], r[kCols];
+    cp_async_wait<1>();
+    __syncwarp();  // the warp's h and r rows have landed
+    read16(B0, h);
+    read16(B1, r);
+    if (!v) {
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) h[j] = 0.f;
+    }
+    split_tmem(tl + kColA + c0, h);
+    hand_over();
+    if (!(ok = s_ok2 != 0)) break;  // (of the tile before; written before the barrier)
+    if (issuer) {
+      if (tid == 0) gemm3(tmem + kD, tmem + kColA, S.B1h, S.B1l, 128, kD);
+      else gemm3(tmem, tmem + kColA, S.B1h, S.B1l, 128, 0);
       mma_commit(bar);
     }
-    last = phase;
-    const bool ok = bar_wait(bar, last);
-    phase ^= 1u;
-    fence_after();
-    if (!ok) s_ok = 0;
-    __syncthreads();
-    return s_ok != 0;
-  };
-
-  const int64_t n_tiles = (a.bt.act_rows() + kTM - 1) / kTM;
-  bool ok = true;
-  for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-    const int64_t ar = tile * kTM + rl;
-    const bool v = ar < a.bt.act_rows();
-    int64_t seq = 0, row = 0;
-    if (v) act_row(a.bt, ar, seq, row);
-    const float* hp = a.s0;
-    const float* xp = a.xproj;
-    if (v) {
-      hp = row == __ldg(a.bt.offsets + seq) ? a.s0 + seq * kD : a.s + (row - 1) * kD;
-      xp = a.xproj + row * (3 * kD);
-    }
-    if (qc == 0) { rmx[rl] = 0.f; rsq[rl] = 0.f; }
-    // stage 1: h (kept in registers for the later stages)
-    float h[kCols], xr[kCols];
-#pragma unroll
-    for (int j = 0; j < kCols; j += 4) {
-      const float4 h4 = v ? ldg4(hp + c0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 x4 = v ? ldg4(xp + kD + c0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      h[j] = h4.x; h[j + 1] = h4.y; h[j + 2] = h4.z; h[j + 3] = h4.w;
-      xr[j] = x4.x; xr[j + 1] = x4.y; xr[j + 2] = x4.z; xr[j + 3] = x4.w;
-      split_store4(S.Ah, S.Al, core_off(kTM, rl, c0 + j), h4);
-    }
-    if (!(ok = run_stage(1))) break;
-    // stage 2: r = sig(Wr x + Ur h) (kept), then r o h
-    float r[kCols];
+    __syncwarp();
+    copy_rows(B0, SRC_S, code, seq);
+    copy_rows(B1, SRC_XH, code, seq);
+    cp_async_commit();
+    uint32_t ncode;
+    int64_t nseq;
+    find_row(tile + gridDim.x, ncode, nseq);
+    // stage 2: r = sig(Wr x + Ur h), then the operands of the two remaining products
+    wait_mma(s_ok1);
     {
       float rp[kCols];
       tmem_ld16(tl + kD + c0, rp);
       tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) r[j] = fsig(rp[j] + xr[j]);
+      for (int j = 0; j < kCols; ++j) r[j] = fsig(rp[j] + r[j]);
 #pragma unroll
-      for (int j = 0; j < kCols; j += 4)
-        split_store4(S.Ah, S.Al, core_off(kTM, rl, c0 + j),
-                     make_float4(r[j] * h[j], r[j + 1] * h[j + 1], r[j + 2] * h[j + 2],
-                                 r[j + 3] * h[j + 3]));
+      for (int j = 0; j < kCols; ++j) rp[j] = r[j] * h[j];
+      split_tmem(tl + kColA + c0, rp);
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) rp[j] = h[j] * r[j] * (1.f - r[j]);
+      split_tmem(tl + kColA3 + c0, rp);
     }
-    // the epilogue's row inputs, loaded now so that they arrive while the products run
-    float xz[kCols], xh[kCols], sc[kCols];
-#pragma unroll
-    for (int j = 0; j < kCols; j += 4) {
-      float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a4, c4 = a4;
-      if (v) {
-        a4 = ldg4(xp + c0 + j);
-        b4 = ldg4(xp + 2 * kD + c0 + j);
-        c4 = *reinterpret_cast<const float4*>(a.s + row * kD + c0 + j);
-      }
-      xz[j] = a4.x; xz[j + 1] = a4.y; xz[j + 2] = a4.z; xz[j + 3] = a4.w;
-      xh[j] = b4.x; xh[j + 1] = b4.y; xh[j + 2] = b4.z; xh[j + 3] = b4.w;
-      sc[j] = c4.x; sc[j + 1] = c4.y; sc[j + 2] = c4.z; sc[j + 3] = c4.w;
+    hand_over();
+    if (!(ok = s_ok1 != 0)) break;
+    if (issuer) {
+      if (tid == 0) gemm3(tmem + 128, tmem + kColA, S.B2h, S.B2l, kD, 0);
+      else gemm3(tmem + 192, tmem + kColA3, S.B3h, S.B3l, kD, 0);
+      mma_commit(bar);
     }
-    if (!(ok = run_stage(2))) break;
-    // stage 3: h o r o (1 - r)
-#pragma unroll
-    for (int j = 0; j < kCols; j += 4)
-      split_store4(S.Ah, S.Al, core_off(kTM, rl, c0 + j),
-                   make_float4(h[j] * r[j] * (1.f - r[j]), h[j + 1] * r[j + 1] * (1.f - r[j + 1]),
-                               h[j + 2] * r[j + 2] * (1.f - r[j + 2]),
-                               h[j + 3] * r[j + 3] * (1.f - r[j + 3])));
-    if (!(ok = run_stage(3))) break;
-    // gates, F, diagonal Jacobian, residual (two halves of 8 columns)
+    __syncwarp();
+    float sc[kCols], xz[kCols], xh[kCols];
+    cp_async_wait<0>();
+    __syncwarp();  // the warp's s, z and h~ rows have landed
+    read16(B0, sc);
+    read16(B1, xh);
+    read16(B2, xz);
+    __syncwarp();
+    copy_rows(B0, SRC_H, ncode, nseq);
+    copy_rows(B1, SRC_XR, ncode, nseq);
+    cp_async_commit();
+    wait_mma(s_ok2);
+    // gates, F, diagonal Jacobian, residual (two halves of 8 columns); a and b replace the z
+    // and h~ projections
     float mx = 0.f, sq = 0.f;
 #pragma unroll
     for (int hh = 0; hh < kCols; hh += 8) {
@@ -228,55 +322,48 @@ __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
       tmem_ld8(tl + 128 + c0 + hh, hq);
       tmem_ld8(tl + 192 + c0 + hh, mc);
       tmem_wait_ld();
-      if (v) {
 #pragma unroll
-        for (int jj = 0; jj < 8; jj += 4) {
-          const int j = hh + jj, k = c0 + j;
-          float bo[4], ao[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int o = k + e;
-            const float zi = fsig(zp[jj + e] + xz[j + e]);
-            const float ri = r[j + e];
-            const float ht = tanhf(hq[jj + e] + xh[j + e]);
-            const float hv = h[j + e];
-            const float F = (1.f - zi) * hv + zi * ht;
-            float ai;
-            if (a.jac == DEER_JAC_DIAG) {
-              ai = (1.f - zi) + (ht - hv) * zi * (1.f - zi) * diag_z[o] +
-                   zi * (1.f - ht * ht) * (diag_h[o] * ri + mc[jj + e]);
-            } else {
-              ai = a.jac == DEER_JAC_IDENTITY ? 1.f : 0.f;
-            }
-            if (a.damp == DEER_DAMP_SCALE) ai *= (1.f - kk);
-            else if (a.damp == DEER_DAMP_CLIP) ai = fminf(fmaxf(ai, -kk), kk);
-            ao[e] = ai;
-            bo[e] = F - ai * hv;
-            const float res = sc[j + e] - F;
-            const float sa = fabsf(sc[j + e]);
-            const float m = fabsf(res) / (sa > 1.f ? sa : 1.f);
-            mx = (m > mx || m != m) ? m : mx;
-            sq += res * res;
-          }
-          *reinterpret_cast<float4*>(a.b + row * kD + k) = make_float4(bo[0], bo[1], bo[2], bo[3]);
-          if (a.jac == DEER_JAC_DIAG)
-            *reinterpret_cast<float4*>(a.A + row * kD + k) =
-                make_float4(ao[0], ao[1], ao[2], ao[3]);
+      for (int e = 0; e < 8; ++e) {
+        const int j = hh + e;
+        const float zi = fsig(zp[e] + xz[j]);
+        const float ri = r[j];
+        const float ht = tanhf(hq[e] + xh[j]);
+        const float hv = h[j];
+        const float F = (1.f - zi) * hv + zi * ht;
+        float ai;
+        if (a.jac == DEER_JAC_DIAG) {
+          const float2 dg = s_diag[c0 + j];
+          ai = (1.f - zi) + (ht - hv) * zi * (1.f - zi) * dg.x +
+               zi * (1.f - ht * ht) * (dg.y * ri + mc[e]);
+        } else {
+          ai = a.jac == DEER_JAC_IDENTITY ? 1.f : 0.f;
         }
+        if (a.damp == DEER_DAMP_SCALE) ai *= (1.f - kk);
+        else if (a.damp == DEER_DAMP_CLIP) ai = fminf(fmaxf(ai, -kk), kk);
+        xz[j] = ai;
+        xh[j] = F - ai * hv;
+        const float res = sc[j] - F;
+        const float sa = fabsf(sc[j]);
+        const float m = sa > 1.f ? fabsf(res) / sa : fabsf(res);
+        mx = (m > mx || m != m) ? m : mx;
+        sq += res * res;
       }
     }
-    if (v) {
-      // non-negative floats order like their bit patterns
-      atomicMax(reinterpret_cast<int*>(&rmx[rl]), __float_as_int(mx));
-      atomicAdd(&rsq[rl], sq);
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (qc == 0)
-      acc_resid_f(a.acc, seq, v, rmx[rl], rsq[rl],
-                  bad_key(!(rmx[rl] <= a.tol_f), row - (v ? __ldg(a.bt.offsets + seq) : 0)));
+    fence_before();  // (the next hand-over orders these reads before the products after it)
+    if (a.jac == DEER_JAC_DIAG) rows_out(xz, a.A, code);
+    rows_out(xh, a.b, code);
+    acc_resid_f(a.acc, seq, v, mx, sq,
+                bad_key(v && !(mx <= a.tol_f),
+                        (int64_t)(code >> 1) - (v ? __ldg(a.bt.offsets + seq) : 0)));
+    __syncwarp();
+    code = ncode;
+    seq = nseq;
+    copy_rows(B2, SRC_XZ, code, seq);
+    cp_async_commit();
   }
+  __syncthreads();
+  if (s_ok2 == 0) ok = false;
+  cp_async_wait<0>();
   if (!ok) {
     if (tid == 0) atomicExch(&a.status->timeout, 1);
     // products may still be in flight: give them (bounded) time before tensor memory is

@@ -411,6 +411,8 @@ __global__ void __launch_bounds__(256) k_init_randn(real* __restrict__ s, int64_
 template <class real>
 cudaError_t launch_init(const InitArgs<real>& a, cudaStream_t st) {
   if (a.bt.N == 0) return cudaSuccess;
+  if (a.init == DEER_INIT_ZEROS)  // (a kernel of row-per-thread stores: 600 us for 1.07 GB)
+    return cudaMemsetAsync(a.s, 0, (size_t)a.bt.N * a.dv.d * sizeof(real), st);
   if (a.init == DEER_INIT_RANDN) {
     const int64_t n = a.bt.N * a.dv.d;
     int64_t g = (n + 255) / 256;
