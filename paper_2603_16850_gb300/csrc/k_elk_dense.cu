@@ -6,131 +6,247 @@
 // (s_0, or the frozen state under a sliding window, is known). This kernel runs the
 // covariance recursion and rewrites A_t <- Gamma_t A_t, b_t <- Gamma_t b_t in place; the
 // dense scan then solves the mean in parallel over t. The covariance recursion does not
-// depend on the emissions, only on A_t; it is a dependent chain over t, run by a group of
-// d lanes per sequence (lane i owns row i of every d x d matrix) with the rows exchanged
-// through shared memory, and the inverse by Gauss-Jordan elimination (I + lambda P^- is
-// symmetric positive definite, so no pivoting). For few, long sequences the covariance
-// recursion runs in parallel over time instead (chunk elements, carry, then this
-// recursion per chunk from the carried covariance; see below).
+// depend on the emissions, only on A_t; it is a dependent chain over t, run per sequence, or,
+// for few, long sequences, in parallel over time (chunk elements, carry, then this recursion
+// per chunk from the carried covariance; see below).
+//
+// What bounds these kernels is the chain of small dense products and inverses per row: in
+// float64 a warp issues one FP64 instruction per 64 clocks whatever the number of active
+// lanes, so a row costs its FP64 instruction count. Each chunk (or sequence) gets a group of
+// min(32, d^2) lanes, or more in the carry, and every d x d product is spread over all of
+// them, one or a few entries per lane (16 instructions per product at d = 8 against 64 with a
+// row per lane); inverses are in place (half the entries of an augmented elimination) and
+// their reciprocals take four FP64 instructions instead of a division's 23. Mass action d = 8,
+// float64, 4 sequences of 4096 rows, per iteration (d lanes per chunk, a row per lane, blocks
+// of 16 chunks before): chunk elements 2626 -> 300 us, carry 1696 (64 steps) -> 536 (128
+// steps, 4.2 us each: pivots in order), restart 1538 -> 194 us.
 #include "kernels.h"
 
 namespace deer {
+namespace {
 
-// One group of D lanes per sequence (CHUNKED = false: the covariance starts at zero at the
-// sequence's first row) or per chunk (CHUNKED = true: it starts from the filtered
-// covariance the carry pass computed for the chunk).
-// lanes per block: 128, or 64 for d >= 16 (the shared buffers of the float64 kernels)
+// Lanes of the group that owns one chunk (or sequence): a warp or part of one; in the carry
+// pass of d >= 8 a block of several warps (one block per sequence).
 template <int D>
-constexpr int elk_block() { return D >= 16 ? 64 : 128; }
+constexpr int elk_lanes() { return D * D < 32 ? D * D : 32; }
+template <int D>
+constexpr int elk_carry_lanes() { return D == 8 ? 64 : D == 16 ? 128 : elk_lanes<D>(); }
 
+// 1 / x by Newton's iteration y <- y + y (1 - x y) from a float32 reciprocal of the mantissa
+// (relative error 2^-22, squared twice): four FP64 instructions, within two ulp. Non-finite,
+// zero and subnormal x, and results near the subnormal range, take the division.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  if (e == 0 || e >= 2044) return 1.0 / x;
+  // mantissa m in [1, 2), as double and truncated to float
+  const double m = __hiloint2double((int)(0x3ff00000u | (hi & 0xfffffu)), (int)lo);
+  const unsigned yb =
+      __float_as_uint(1.f / __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29)));
+  double y = __hiloint2double(((int)(yb >> 23) - 127 + 1023) << 20 | (int)((yb & 0x7fffffu) >> 3),
+                              (int)(yb << 29));
+  y = fma(y, fma(-m, y, 1.0), y);
+  y = fma(y, fma(-m, y, 1.0), y);
+  // times 2^(1023 - e), with the sign of x
+  return __hiloint2double((__double2hiint(y) + ((1023 - e) << 20)) | (int)(hi & 0x80000000u),
+                          __double2loint(y));
+}
+__device__ __forceinline__ float recip(float x) { return 1.f / x; }
+
+// larger magnitude = larger key, from the bit pattern (no FP64 comparison)
+__device__ __forceinline__ int mag_key(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int mag_key(float x) { return __float_as_int(x) & 0x7fffffff; }
+
+// d x d matrices of a group: entry e = lane + m GW (row e / D, column e % D) is slot m of a
+// lane; operands are read from shared memory (rows padded against bank conflicts).
+template <class real, int D, int GW>
+struct Grp {
+  static constexpr int EPL = D * D / GW;
+  static constexpr int RS = D + (D >= 4 ? 16 / (int)sizeof(real) : 1);
+  static constexpr int SZ = D * RS;
+  int lane;
+  unsigned mask;
+
+  __device__ __forceinline__ Grp() {
+    lane = threadIdx.x % GW;
+    mask = GW >= 32 ? 0xffffffffu : ((1u << (GW & 31)) - 1u) << (threadIdx.x & 31 & ~(GW - 1));
+  }
+  __device__ __forceinline__ void sync() const {
+    if constexpr (GW > 32) __syncthreads();  // the block is the group
+    else __syncwarp(mask);
+  }
+  __device__ __forceinline__ int row(int m) const { return (lane + m * GW) / D; }
+  __device__ __forceinline__ int col(int m) const { return (lane + m * GW) % D; }
+  __device__ __forceinline__ real eye(int m) const { return row(m) == col(m) ? real(1) : real(0); }
+  __device__ __forceinline__ void store(real* M, const real (&v)[EPL]) const {
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) M[row(m) * RS + col(m)] = v[m];
+  }
+  // row-major dense blocks in global memory
+  __device__ __forceinline__ void gload(const real* g, real (&v)[EPL]) const {
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) v[m] = g[lane + m * GW];
+  }
+  __device__ __forceinline__ void gstore(real* g, const real (&v)[EPL]) const {
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) g[lane + m * GW] = v[m];
+  }
+  __device__ __forceinline__ void fetch(real* M, const real* g) const {
+#pragma unroll
+    for (int m = 0; m < EPL; ++m)
+      cp_async_small<sizeof(real)>(M + row(m) * RS + col(m), g + lane + m * GW);
+  }
+  // entries of op(X) op(Y), op = transpose where TX / TY
+  template <bool TX, bool TY>
+  __device__ __forceinline__ void mul(const real* X, const real* Y, real (&v)[EPL]) const {
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) v[m] = real(0);
+#pragma unroll(D <= 8 ? D : 2)
+    for (int k = 0; k < D; ++k)
+#pragma unroll
+      for (int m = 0; m < EPL; ++m)
+        v[m] += X[TX ? k * RS + row(m) : row(m) * RS + k] *
+                Y[TY ? col(m) * RS + k : k * RS + col(m)];
+  }
+  // Gauss-Jordan inverse of the matrix in M0, in place (M1: scratch of the same size). With
+  // PIVOT, the pivot of column c is the unused row w_c of largest magnitude; rows stay where
+  // they are, and at the end row w_c holds row c of the inverse, its stored column k belonging
+  // to right-hand side w_k. The result is left in `out` (not M0 or M1).
+  template <bool PIVOT>
+  __device__ __forceinline__ void inverse(real* M0, real* M1, real* out) const {
+    unsigned long long where = 0ull;  // 4 bits per column: w_c
+    unsigned used = 0u;
+    real v[EPL];
+#pragma unroll(D <= 8 ? D : 1)
+    for (int c = 0; c < D; ++c) {
+      const real* src = c & 1 ? M1 : M0;
+      real* dst = c & 1 ? M0 : M1;
+      int w = c;
+      if constexpr (PIVOT) {
+        int best = -2;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          const int key = (used >> i) & 1u ? -1 : mag_key(src[i * RS + c]);
+          if (key > best) { best = key; w = i; }
+        }
+        used |= 1u << w;
+        where |= (unsigned long long)w << (4 * c);
+      }
+      const real ip = recip(src[w * RS + c]);
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) {
+        const int i = row(m), j = col(m);
+        // the pivot row is scaled (its pivot entry becomes 1 / p); the others lose their
+        // pivot-column entry f times it (that entry itself becomes -f / p)
+        const real q = (j == c ? real(1) : src[w * RS + j]) * ip;
+        const real o = j == c ? real(0) : src[i * RS + j];
+        v[m] = i == w ? q : o - src[i * RS + c] * q;
+        if (c < D - 1) dst[i * RS + j] = v[m];
+      }
+      if (c < D - 1) sync();
+    }
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) {
+      int i = row(m), j = col(m);
+      if constexpr (PIVOT) {
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < D; ++k)
+          if ((int)((where >> (4 * k)) & 15ull) == i) c = k;
+        i = c;
+        j = (int)((where >> (4 * j)) & 15ull);
+      }
+      out[i * RS + j] = v[m];
+    }
+    sync();
+  }
+};
+
+}  // namespace
+
+// One group per sequence (CHUNKED = false: the covariance starts at zero at the sequence's
+// first row) or per chunk (CHUNKED = true: it starts from the filtered covariance the carry
+// pass computed for the chunk).
 template <class real, int D, bool CHUNKED>
-__global__ void __launch_bounds__(128) k_elk_dense(ElkDenseArgs<real> a) {
-  constexpr int G = elk_block<D>() / D;
-  constexpr int RS = D + (D >= 4 ? 16 / (int)sizeof(real) : 1);  // padded row stride
-  __shared__ real sP[G][D][RS];   // covariance P_{t-1}, then P^-_t
-  __shared__ real sA[G][D][RS];   // A_t
-  __shared__ real sS[G][2][RS];   // pivot row of the elimination (S and the inverse)
-  const int grp = threadIdx.x / D, i = threadIdx.x % D;
-  const unsigned gm = D >= 32 ? 0xffffffffu
-                              : (((1u << D) - 1u) << ((threadIdx.x & 31) & ~(D - 1)));
-  const int64_t k = blockIdx.x * (int64_t)G + grp;
-  int64_t r_begin, r_end;
-  const real lam = a.lambda;
-  real (*P)[RS] = sP[grp];
-  real (*Am)[RS] = sA[grp];
-  real (*Sp)[RS] = sS[grp];
+__global__ void __launch_bounds__(32) k_elk_dense(ElkDenseArgs<real> a) {
+  constexpr int GW = elk_lanes<D>();
+  using G = Grp<real, D, GW>;
+  constexpr int EPL = G::EPL, SZ = G::SZ;
+  __shared__ real sm[32 / GW][8 * SZ];
+  __shared__ real sb[32 / GW][2][D];
+  const G g;
+  const int grp = threadIdx.x / GW;
+  real* F[2] = {sm[grp], sm[grp] + SZ};
+  real *P = sm[grp] + 2 * SZ, *T = sm[grp] + 3 * SZ, *Pm = sm[grp] + 4 * SZ;
+  real *S0 = sm[grp] + 5 * SZ, *S1 = sm[grp] + 6 * SZ, *N = sm[grp] + 7 * SZ;
+  const int64_t k = blockIdx.x * (int64_t)(32 / GW) + grp;
+  int64_t r0, r1;
+  real v[EPL], u[EPL];
+#pragma unroll
+  for (int m = 0; m < EPL; ++m) v[m] = real(0);
   if constexpr (CHUNKED) {
     if (k >= a.bt.act_chunks()) return;  // whole groups
     int64_t seq, c;
     int n;
-    act_chunk(a.bt, k, seq, c, r_begin, n);
-    r_end = r_begin + n;
-    const real* Pin = a.cov_in + c * (int64_t)(D * D);
-#pragma unroll
-    for (int j = 0; j < D; ++j) P[i][j] = Pin[i * D + j];
+    act_chunk(a.bt, k, seq, c, r0, n);
+    r1 = r0 + n;
+    g.gload(a.cov_in + c * (int64_t)(D * D), v);
   } else {
     if (k >= a.bt.n_act()) return;  // whole groups
     const int64_t seq = a.bt.act_seq[k];
     const int64_t cf = a.bt.chunk_first[seq];
-    r_begin = a.bt.offsets[seq] + ((win_first(a.bt, seq) - cf) << a.bt.log2L);
-    r_end = a.bt.offsets[seq + 1];
-#pragma unroll
-    for (int j = 0; j < D; ++j) P[i][j] = real(0);
+    r0 = a.bt.offsets[seq] + ((win_first(a.bt, seq) - cf) << a.bt.log2L);
+    r1 = a.bt.offsets[seq + 1];
   }
-  __syncwarp(gm);
-  for (int64_t row = r_begin; row < r_end; ++row) {
-    real* Ar = a.A + row * (int64_t)(D * D) + i * D;
-    real arow[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      arow[j] = Ar[j];
-      Am[i][j] = arow[j];
+  g.store(P, v);
+  auto fetch = [&](int64_t row) {
+    if (row < r1) {
+      const int s = (int)((row - r0) & 1);
+      g.fetch(s ? F[1] : F[0], a.A + row * (int64_t)(D * D));
+      if (g.lane < D) cp_async_small<sizeof(real)>(&sb[grp][s][g.lane], a.b + row * D + g.lane);
     }
-    __syncwarp(gm);
-    // (A P)_i = sum_m A_im P_m
-    real ap[D];
+    cp_async_commit();
+  };
+  fetch(r0);
+  for (int64_t row = r0; row < r1; ++row) {
+    const int s = (int)((row - r0) & 1);
+    real* Ft = s ? F[1] : F[0];
+    cp_async_wait<0>();
+    g.sync();
+    fetch(row + 1);
+    // P^- = F P F^T + I, S = I + lambda P^-
+    g.template mul<false, false>(Ft, P, v);
+    g.store(T, v);
+    g.sync();
+    g.template mul<false, true>(T, Ft, v);
 #pragma unroll
-    for (int j = 0; j < D; ++j) ap[j] = real(0);
-#pragma unroll
-    for (int m = 0; m < D; ++m)
-#pragma unroll
-      for (int j = 0; j < D; ++j) ap[j] += arow[m] * P[m][j];
-    // P^-_ij = sum_m (A P)_im A_jm + delta_ij; S = I + lambda P^-, augmented with I
-    real pm[D], s[D], e[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      real x = j == i ? real(1) : real(0);
-#pragma unroll
-      for (int m = 0; m < D; ++m) x += ap[m] * Am[j][m];
-      pm[j] = x;
-      s[j] = (j == i ? real(1) : real(0)) + lam * x;
-      e[j] = j == i ? real(1) : real(0);
+    for (int m = 0; m < EPL; ++m) {
+      v[m] += g.eye(m);
+      u[m] = g.eye(m) + a.lambda * v[m];
     }
-    __syncwarp(gm);
+    g.store(Pm, v);
+    g.store(S0, u);
+    g.sync();
+    // Gamma = S^{-1} (symmetric positive definite: no pivoting)
+    g.template inverse<false>(S0, S1, N);
+    // P = Gamma P^-, A <- Gamma A, b <- Gamma b (the lanes of a row share its sum)
+    g.template mul<false, false>(N, Pm, v);
+    g.store(P, v);
+    g.template mul<false, false>(N, Ft, u);
+    g.gstore(a.A + row * (int64_t)(D * D), u);
+    constexpr int PARTS = GW / D;
+    const int i = g.lane / PARTS;
+    real x = real(0);
 #pragma unroll
-    for (int j = 0; j < D; ++j) P[i][j] = pm[j];  // P^- rows for the update below
-    // Gauss-Jordan: S e = I row by row; pivot row c is broadcast through shared memory
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-      if (i == c) {
-        const real inv = real(1) / s[c];
-#pragma unroll
-        for (int j = 0; j < D; ++j) { s[j] *= inv; e[j] *= inv; Sp[0][j] = s[j]; Sp[1][j] = e[j]; }
-      }
-      __syncwarp(gm);
-      if (i != c) {
-        const real fct = s[c];
-#pragma unroll
-        for (int j = 0; j < D; ++j) { s[j] -= fct * Sp[0][j]; e[j] -= fct * Sp[1][j]; }
-      }
-      __syncwarp(gm);
+    for (int q = 0; q < D / PARTS; ++q) {
+      const int kk = q * PARTS + g.lane % PARTS;
+      x += N[i * G::RS + kk] * sb[grp][s][kk];
     }
-    // e = row i of Gamma = S^{-1}; P_t = Gamma P^-; A <- Gamma A; b <- Gamma b
-    real np[D], na[D];
 #pragma unroll
-    for (int j = 0; j < D; ++j) { np[j] = real(0); na[j] = real(0); }
-#pragma unroll
-    for (int m = 0; m < D; ++m) {
-      const real g = e[m];
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        np[j] += g * P[m][j];
-        na[j] += g * Am[m][j];
-      }
-    }
-    const real bi = a.b[row * D + i];
-    real nb = real(0);
-#pragma unroll
-    for (int m = 0; m < D; ++m) nb += e[m] * __shfl_sync(gm, bi, m, D);
-    __syncwarp(gm);
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      P[i][j] = np[j];
-      Ar[j] = na[j];
-    }
-    a.b[row * D + i] = nb;
-    __syncwarp(gm);
+    for (int o = 1; o < PARTS; o <<= 1) x += __shfl_xor_sync(g.mask, x, o, GW);
+    if (g.lane % PARTS == 0) a.b[row * D + i] = x;
   }
+  cp_async_wait<0>();
 }
 
 // ---------------------------------------------------------------------------
@@ -138,277 +254,165 @@ __global__ void __launch_bounds__(128) k_elk_dense(ElkDenseArgs<real> a) {
 // covariance P to A (I + P J)^{-1} P A^T + C with the step's element
 // (A, C, J) = (c F_t, c I, lambda c F_t^T F_t), c = 1 / (1 + lambda) (process noise I,
 // emission variance 1/lambda); elements combine associatively, e_i then e_j giving
-// (A_j N A_i, A_j N C_i A_j^T + C_j, A_i^T N^T J_j A_i + J_i) with N = (I + C_i J_j)^{-1}
-// (Sarkka and Garcia-Fernandez's parallel Kalman filter). The chunk pass folds each
-// chunk's elements in order; the carry pass walks a sequence's chunks applying their
-// aggregates to the covariance (one short chain per sequence: T / L steps instead of T);
-// the per-chunk recursion above then rewrites (A_t, b_t) from the carried covariance.
-// Lane i of a group owns row i of every d x d matrix; products read the other operand's
-// rows from the group's shared buffers; inverses by Gauss-Jordan elimination with partial
-// pivoting (I + C J is not symmetric).
+// (A_j N A_i, A_j N C_i A_j^T + C_j, A_i^T J_j N A_i + J_i) with N = (I + C_i J_j)^{-1}
+// (Sarkka and Garcia-Fernandez's parallel Kalman filter; N^T J_j = J_j N). The chunk pass
+// folds each chunk's elements in order; the carry pass walks a sequence's chunks applying
+// their aggregates to the covariance (one short chain per sequence: T / L steps instead of
+// T); the per-chunk recursion above then rewrites (A_t, b_t) from the carried covariance.
+// Inverses with partial pivoting (I + C J is not symmetric).
 // ---------------------------------------------------------------------------
-
-// row i of Y = X M for X's row x (registers) and M's rows in shared memory
-template <class real, int D, int RS>
-__device__ __forceinline__ void row_times(const real (&x)[D], const real (*M)[RS], real (&y)[D]) {
-#pragma unroll
-  for (int j = 0; j < D; ++j) y[j] = real(0);
-#pragma unroll
-  for (int m = 0; m < D; ++m)
-#pragma unroll
-    for (int j = 0; j < D; ++j) y[j] += x[m] * M[m][j];
-}
-
-// row i of S^{-1} for S's row s (destroyed); piv: two shared rows, out: D shared rows
-template <class real, int D, int RS>
-__device__ __forceinline__ void gj_inverse(real (&s)[D], real (&inv)[D], int i, unsigned gm,
-                                           real (*piv)[RS], real (*out)[RS]) {
-  real e[D];
-#pragma unroll
-  for (int j = 0; j < D; ++j) e[j] = j == i ? real(1) : real(0);
-  bool used = false;
-  int mycol = 0;
-#pragma unroll
-  for (int c = 0; c < D; ++c) {
-    // pivot: the unused row with the largest |s_c| (ties to the lower lane)
-    real key = used ? real(-1) : (s[c] < real(0) ? -s[c] : s[c]);
-    int who = i;
-#pragma unroll
-    for (int o = D / 2; o > 0; o >>= 1) {
-      const real ok = __shfl_xor_sync(gm, key, o, D);
-      const int ow = __shfl_xor_sync(gm, who, o, D);
-      if (ok > key || (ok == key && ow < who)) { key = ok; who = ow; }
-    }
-    if (i == who) {
-      const real ip = real(1) / s[c];
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        s[j] *= ip;
-        e[j] *= ip;
-        piv[0][j] = s[j];
-        piv[1][j] = e[j];
-      }
-      used = true;
-      mycol = c;
-    }
-    __syncwarp(gm);
-    if (i != who) {
-      const real f = s[c];
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        s[j] -= f * piv[0][j];
-        e[j] -= f * piv[1][j];
-      }
-    }
-    __syncwarp(gm);
-  }
-  // the lane that pivoted on column c holds row c of the inverse
-#pragma unroll
-  for (int j = 0; j < D; ++j) out[mycol][j] = e[j];
-  __syncwarp(gm);
-#pragma unroll
-  for (int j = 0; j < D; ++j) inv[j] = out[i][j];
-  __syncwarp(gm);
-}
-
 template <class real, int D>
-__global__ void __launch_bounds__(128) k_elk_cov_chunk(ElkDenseArgs<real> a) {
-  constexpr int G = elk_block<D>() / D;
-  constexpr int RS = D + (D >= 4 ? 16 / (int)sizeof(real) : 1);
-  __shared__ real sM[G][4][D][RS];  // exchange buffers
-  __shared__ real sV[G][2][RS];
-  const int grp = threadIdx.x / D, i = threadIdx.x % D;
-  const unsigned gm = D >= 32 ? 0xffffffffu
-                              : (((1u << D) - 1u) << ((threadIdx.x & 31) & ~(D - 1)));
-  const int64_t k = blockIdx.x * (int64_t)G + grp;
+__global__ void __launch_bounds__(32) k_elk_cov_chunk(ElkDenseArgs<real> a) {
+  constexpr int GW = elk_lanes<D>();
+  using G = Grp<real, D, GW>;
+  constexpr int EPL = G::EPL, SZ = G::SZ;
+  __shared__ real sm[32 / GW][9 * SZ];
+  const G g;
+  const int grp = threadIdx.x / GW;
+  const int64_t k = blockIdx.x * (int64_t)(32 / GW) + grp;
   if (k >= a.bt.act_chunks()) return;  // whole groups
   int64_t seq, c, r0;
   int n;
   act_chunk(a.bt, k, seq, c, r0, n);
-  const real lam = a.lambda;
-  const real cc = real(1) / (real(1) + lam);
-  real (*F)[RS] = sM[grp][0];
-  real (*B1)[RS] = sM[grp][1];
-  real (*B2)[RS] = sM[grp][2];
-  real (*B3)[RS] = sM[grp][3];
-  real Aa[D], Ca[D], Ja[D];  // rows i of the chunk's aggregate element
+  real* F0 = sm[grp];
+  real *F1 = F0 + SZ, *A = F0 + 2 * SZ, *C = F0 + 3 * SZ, *J = F0 + 4 * SZ;
+  real *S0 = F0 + 5 * SZ, *S1 = F0 + 6 * SZ, *N = F0 + 7 * SZ, *X = F0 + 8 * SZ;
+  const real lam = a.lambda, cc = real(1) / (real(1) + lam);
+  real ca[EPL], aa[EPL], ja[EPL], v[EPL], w[EPL];
+  auto fetch = [&](int t) {
+    if (t < n) g.fetch(t & 1 ? F1 : F0, a.A + (r0 + t) * (int64_t)(D * D));
+    cp_async_commit();
+  };
+  fetch(0);
   for (int t = 0; t < n; ++t) {
-    const real* Fr = a.A + (r0 + t) * (int64_t)(D * D) + i * D;
-    real f[D];
+    real* F = t & 1 ? F1 : F0;
+    cp_async_wait<0>();
+    g.sync();
+    fetch(t + 1);
+    g.template mul<true, false>(F, F, v);
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      f[j] = Fr[j];
-      F[i][j] = f[j];
-    }
-    __syncwarp(gm);
-    // J_e row i = lambda c sum_m F_mi F_m
-    real je[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) je[j] = real(0);
-#pragma unroll
-    for (int m = 0; m < D; ++m)
-#pragma unroll
-      for (int j = 0; j < D; ++j) je[j] += F[m][i] * F[m][j];
-#pragma unroll
-    for (int j = 0; j < D; ++j) je[j] *= lam * cc;
+    for (int m = 0; m < EPL; ++m) v[m] *= lam * cc;
     if (t == 0) {
 #pragma unroll
-      for (int j = 0; j < D; ++j) {
-        Aa[j] = cc * f[j];
-        Ca[j] = j == i ? cc : real(0);
-        Ja[j] = je[j];
+      for (int m = 0; m < EPL; ++m) {
+        aa[m] = cc * F[g.row(m) * G::RS + g.col(m)];
+        ca[m] = cc * g.eye(m);
+        ja[m] = v[m];
       }
-      __syncwarp(gm);
-      continue;
+    } else {
+      g.store(J, v);  // the row's J
+      g.sync();
+      // N = (I + C_a J)^{-1}
+      g.template mul<false, false>(C, J, v);
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) v[m] += g.eye(m);
+      g.store(S0, v);
+      g.sync();
+      g.template inverse<true>(S0, S1, N);
+      // X = N A_a, Y = N C_a, V = J A_a
+      g.template mul<false, false>(N, A, v);
+      g.store(X, v);
+      g.template mul<false, false>(N, C, v);
+      g.store(S0, v);
+      g.template mul<false, false>(J, A, v);
+      g.store(S1, v);
+      g.sync();
+      // A = c F X, Z = F Y, J = J_a + V^T X, C = c^2 Z F^T + c I
+      g.template mul<false, false>(F, X, aa);
+      g.template mul<false, false>(F, S0, v);
+      g.store(N, v);
+      g.template mul<true, false>(S1, X, w);
+      g.sync();
+      g.template mul<false, true>(N, F, ca);
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) {
+        aa[m] *= cc;
+        ca[m] = cc * cc * ca[m] + cc * g.eye(m);
+        ja[m] += w[m];
+      }
     }
-    // N = (I + C_a J_e)^{-1}
-#pragma unroll
-    for (int j = 0; j < D; ++j) B1[i][j] = je[j];
-    __syncwarp(gm);
-    real sr[D], nr[D];
-    row_times<real, D, RS>(Ca, B1, sr);
-#pragma unroll
-    for (int j = 0; j < D; ++j) sr[j] += j == i ? real(1) : real(0);
-    __syncwarp(gm);
-    gj_inverse<real, D, RS>(sr, nr, i, gm, sV[grp], B2);
-    // X = N A_a, Y = N C_a (rows i)
-#pragma unroll
-    for (int j = 0; j < D; ++j) { B2[i][j] = Aa[j]; B3[i][j] = Ca[j]; }
-    __syncwarp(gm);
-    real xr[D], yr[D];
-    row_times<real, D, RS>(nr, B2, xr);
-    row_times<real, D, RS>(nr, B3, yr);
-    // V = J_e A_a (row i; B1 holds J_e, B2 holds A_a)
-    real vr[D];
-    row_times<real, D, RS>(je, B2, vr);
-    __syncwarp(gm);
-    // A_new = c F X; Z = F Y; C_new = c^2 Z F^T + c I
-#pragma unroll
-    for (int j = 0; j < D; ++j) { B1[i][j] = xr[j]; B3[i][j] = yr[j]; }
-    __syncwarp(gm);
-    real an[D], zr[D];
-    row_times<real, D, RS>(f, B1, an);
-    row_times<real, D, RS>(f, B3, zr);
-    real cn[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      real x = real(0);
-#pragma unroll
-      for (int m = 0; m < D; ++m) x += zr[m] * F[j][m];
-      cn[j] = cc * cc * x + (j == i ? cc : real(0));
-    }
-    // J_new = A_a^T (N^T V) + J_a: W = N^T V (row i = sum_m N_mi V_m), then rows
-    // sum_m A_a[m][i] W[m]
-    __syncwarp(gm);
-#pragma unroll
-    for (int j = 0; j < D; ++j) { B1[i][j] = nr[j]; B3[i][j] = vr[j]; }
-    __syncwarp(gm);
-    real wr[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) wr[j] = real(0);
-#pragma unroll
-    for (int m = 0; m < D; ++m)
-#pragma unroll
-      for (int j = 0; j < D; ++j) wr[j] += B1[m][i] * B3[m][j];
-    __syncwarp(gm);
-#pragma unroll
-    for (int j = 0; j < D; ++j) B3[i][j] = wr[j];
-    __syncwarp(gm);
-    real jn[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) jn[j] = Ja[j];
-#pragma unroll
-    for (int m = 0; m < D; ++m)
-#pragma unroll
-      for (int j = 0; j < D; ++j) jn[j] += B2[m][i] * B3[m][j];
-    __syncwarp(gm);
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      Aa[j] = cc * an[j];
-      Ca[j] = cn[j];
-      Ja[j] = jn[j];
-    }
+    g.store(A, aa);
+    g.store(C, ca);
   }
+  cp_async_wait<0>();
   real* out = a.cov_agg + c * (int64_t)(3 * D * D);
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    out[i * D + j] = Aa[j];
-    out[D * D + i * D + j] = Ca[j];
-    out[2 * D * D + i * D + j] = Ja[j];
-  }
+  g.gstore(out, aa);
+  g.gstore(out + D * D, ca);
+  g.gstore(out + 2 * D * D, ja);
 }
 
 template <class real, int D>
-__global__ void __launch_bounds__(128) k_elk_cov_carry(ElkDenseArgs<real> a) {
-  constexpr int G = elk_block<D>() / D;
-  constexpr int RS = D + (D >= 4 ? 16 / (int)sizeof(real) : 1);
-  __shared__ real sM[G][3][D][RS];
-  __shared__ real sV[G][2][RS];
-  const int grp = threadIdx.x / D, i = threadIdx.x % D;
-  const unsigned gm = D >= 32 ? 0xffffffffu
-                              : (((1u << D) - 1u) << ((threadIdx.x & 31) & ~(D - 1)));
-  const int64_t kq = blockIdx.x * (int64_t)G + grp;
+__global__ void __launch_bounds__(elk_carry_lanes<D>() < 32 ? 32 : elk_carry_lanes<D>())
+    k_elk_cov_carry(ElkDenseArgs<real> a) {
+  constexpr int GW = elk_carry_lanes<D>();
+  constexpr int GPB = GW < 32 ? 32 / GW : 1;
+  using G = Grp<real, D, GW>;
+  constexpr int EPL = G::EPL, SZ = G::SZ;
+  __shared__ real sm[GPB][6 * SZ];
+  const G g;
+  const int grp = GPB == 1 ? 0 : threadIdx.x / GW;
+  const int64_t kq = blockIdx.x * (int64_t)GPB + grp;
   if (kq >= a.bt.n_act()) return;  // whole groups
   const int64_t seq = a.bt.act_seq[kq];
   const int64_t c0 = win_first(a.bt, seq), c1 = a.bt.chunk_first[seq + 1];
-  real (*Pm)[RS] = sM[grp][0];
-  real (*B1)[RS] = sM[grp][1];
-  real (*B2)[RS] = sM[grp][2];
-  real p[D];
+  real *P = sm[grp], *A = P + SZ, *J = P + 2 * SZ, *S0 = P + 3 * SZ, *S1 = P + 4 * SZ,
+       *N = P + 5 * SZ;
+  // the next chunk's element is loaded ahead
+  real p[EPL], an[EPL], cn[EPL], jn[EPL];
+  auto next = [&](int64_t c) {
+    if (c < c1) {
+      const real* e = a.cov_agg + c * (int64_t)(3 * D * D);
+      g.gload(e, an);
+      g.gload(e + D * D, cn);
+      g.gload(e + 2 * D * D, jn);
+    }
+  };
+  next(c0);
 #pragma unroll
-  for (int j = 0; j < D; ++j) p[j] = real(0);
+  for (int m = 0; m < EPL; ++m) p[m] = real(0);
   for (int64_t c = c0; c < c1; ++c) {
-    real* pin = a.cov_in + c * (int64_t)(D * D);
+    g.gstore(a.cov_in + c * (int64_t)(D * D), p);
+    g.store(P, p);
+    g.store(A, an);
+    g.store(J, jn);
+    real ca[EPL], v[EPL];
 #pragma unroll
-    for (int j = 0; j < D; ++j) pin[i * D + j] = p[j];
-    const real* e = a.cov_agg + c * (int64_t)(3 * D * D);
-    real ar[D], cr[D];
+    for (int m = 0; m < EPL; ++m) ca[m] = cn[m];
+    g.sync();
+    next(c + 1);
+    // N = (I + P J)^{-1}; P <- A N P A^T + C
+    g.template mul<false, false>(P, J, v);
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      ar[j] = e[i * D + j];
-      cr[j] = e[D * D + i * D + j];
-      B1[i][j] = e[2 * D * D + i * D + j];  // J
-      Pm[i][j] = p[j];
-    }
-    __syncwarp(gm);
-    // N = (I + P J)^{-1}; P_out = A N P A^T + C
-    real sr[D], nr[D];
-    row_times<real, D, RS>(p, B1, sr);
+    for (int m = 0; m < EPL; ++m) v[m] += g.eye(m);
+    g.store(S0, v);
+    g.sync();
+    g.template inverse<true>(S0, S1, N);
+    g.template mul<false, false>(N, P, v);
+    g.store(S0, v);
+    g.sync();
+    g.template mul<false, false>(A, S0, v);
+    g.store(S1, v);
+    g.sync();
+    g.template mul<false, true>(S1, A, p);
 #pragma unroll
-    for (int j = 0; j < D; ++j) sr[j] += j == i ? real(1) : real(0);
-    __syncwarp(gm);
-    gj_inverse<real, D, RS>(sr, nr, i, gm, sV[grp], B2);
-    real yr[D];
-    row_times<real, D, RS>(nr, Pm, yr);  // (N P)_i
-    __syncwarp(gm);
-#pragma unroll
-    for (int j = 0; j < D; ++j) { B1[i][j] = yr[j]; B2[i][j] = ar[j]; }
-    __syncwarp(gm);
-    real zr[D];
-    row_times<real, D, RS>(ar, B1, zr);  // (A N P)_i
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      real x = cr[j];
-#pragma unroll
-      for (int m = 0; m < D; ++m) x += zr[m] * B2[j][m];
-      p[j] = x;
-    }
-    __syncwarp(gm);
+    for (int m = 0; m < EPL; ++m) p[m] += ca[m];
+    g.sync();  // every read of this chunk's matrices done
   }
 }
 
 template <class real, int D>
 static void elk_dense_launch(const ElkDenseArgs<real>& a, cudaStream_t st) {
-  constexpr int NT = elk_block<D>();
-  constexpr int G = NT / D;
+  constexpr int GPB = 32 / elk_lanes<D>();
   if (a.cov_agg) {
-    const unsigned gc = grid_for(a.bt.act_chunks(), G);
-    k_elk_cov_chunk<real, D><<<gc, NT, 0, st>>>(a);
-    k_elk_cov_carry<real, D><<<grid_for(a.bt.n_act(), G), NT, 0, st>>>(a);
-    k_elk_dense<real, D, true><<<gc, NT, 0, st>>>(a);
+    constexpr int CW = elk_carry_lanes<D>();
+    const unsigned gc = grid_for(a.bt.act_chunks(), GPB);
+    k_elk_cov_chunk<real, D><<<gc, 32, 0, st>>>(a);
+    k_elk_cov_carry<real, D>
+        <<<grid_for(a.bt.n_act(), CW < 32 ? 32 / CW : 1), CW < 32 ? 32 : CW, 0, st>>>(a);
+    k_elk_dense<real, D, true><<<gc, 32, 0, st>>>(a);
     note_launch(3);
   } else {
-    k_elk_dense<real, D, false><<<grid_for(a.bt.n_act(), G), NT, 0, st>>>(a);
+    k_elk_dense<real, D, false><<<grid_for(a.bt.n_act(), GPB), 32, 0, st>>>(a);
     note_launch();
   }
 }
