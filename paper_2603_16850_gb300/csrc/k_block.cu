@@ -5,22 +5,30 @@
 // batch of short sequences is one launch in which every cluster stops on its own
 // convergence.
 //
-// The cluster's threads own contiguous rows of the sequence in (block rank, thread)
+// The cluster's threads own contiguous rows of the sequence in (block rank, warp, lane)
 // order, R rows each. One iteration:
 //   1. each thread evaluates F_t = f_t(s_{t-1}) and A_t on its rows (the row before its
 //      first comes from the previous thread through shared memory, from the previous
-//      block's shared memory for thread 0, s_0 at the start), forms the residual
+//      block's shared memory for the first thread, s_0 at the start), tests the residual
 //      r_t = s_t - F_t and composes its rows' affine steps Delta -> A_t Delta - r_t into
 //      one element (P, v);
-//   2. a reduction over the cluster gives the largest scaled residual max |r| / max(1, |s|)
-//      and sum r^2, and, behind the same cluster barrier, an exclusive scan of the
-//      elements (warp shuffles, the warp totals, then the blocks' totals read across the
-//      cluster) gives the correction Delta entering each thread's rows;
+//   2. the elements are reduced by trees (lanes of a warp, the block's warps, then the
+//      blocks' totals read across the cluster behind one barrier) and the correction Delta
+//      entering each thread's rows comes back down them;
 //   3. the test and the iteration count follow the library's convergence check, taken
 //      identically by every block; unless it stops, each thread propagates Delta through
 //      its rows with the A_t and F_t it kept, adding it to the iterate with the reset
-//      heuristic.
-// Two cluster barriers per iteration: the boundary rows, then statistics and scan totals.
+//      heuristic. The largest scaled residual and sum r^2 are formed once, at the end: the
+//      decisions need only votes.
+// Two cluster barriers per iteration: the boundary rows, then votes and totals.
+//
+// What bounds an iteration is its chain of FP64 instructions: a warp issues one per 64 clocks,
+// whatever its active lanes. So a composition is spread over lanes, one entry of (P, v) each,
+// and only vectors come down (44 instructions at d = 2, 1024 rows, against 150 for an
+// inclusive scan of whole elements per lane), the rows spread over all four warps of a
+// block, and comparisons work on the bit patterns. Brusselator,
+// float64, T = 1024: 13.0 -> 7.2 us per iteration (start 376, now 278 us a call, of which
+// about 150 is the host); 64 x 2048 rows 3.24 -> 1.77 ms.
 #include <cooperative_groups.h>
 
 #include <cfloat>
@@ -61,18 +69,6 @@ __device__ __forceinline__ Aff<real, D> compose(const Aff<real, D>& l, const Aff
 }
 
 template <class real, int D>
-__device__ __forceinline__ Aff<real, D> shfl_up_aff(const Aff<real, D>& a, int off) {
-  Aff<real, D> o;
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    o.v[i] = __shfl_up_sync(0xffffffffu, a.v[i], off);
-#pragma unroll
-    for (int j = 0; j < D; ++j) o.P[i][j] = __shfl_up_sync(0xffffffffu, a.P[i][j], off);
-  }
-  return o;
-}
-
-template <class real, int D>
 __device__ __forceinline__ Aff<real, D> aff_identity() {
   Aff<real, D> o;
 #pragma unroll
@@ -84,31 +80,83 @@ __device__ __forceinline__ Aff<real, D> aff_identity() {
   return o;
 }
 
-// inclusive scan over the first n lanes of a warp (lane order = time order; n <= 32, the
-// steps stop at the first power of two >= n: every float64 product counts on this GPU)
+// Trees of affine maps in shared memory: n leaves (a power of two), the level of m nodes at
+// offset 2 n - 2 m, an element as D rows of (P[i][0..D), v[i]).
+template <int D>
+constexpr int kEl = D * (D + 1);
+
+// every node = later child o earlier child; one warp, one entry per lane and step
 template <class real, int D>
-__device__ __forceinline__ Aff<real, D> warp_scan_aff(Aff<real, D> x, int lane, int n = 32) {
+__device__ __forceinline__ void tree_up(real* tree, int n, int lane) {
+  constexpr int E = kEl<D>;
+  for (int m = n >> 1; m >= 1; m >>= 1) {
+    const real* child = tree + (2 * n - 4 * m) * E;
+    real* node = tree + (2 * n - 2 * m) * E;
+    for (int t = lane; t < m * E; t += 32) {
+      const int q = t / E, e = t % E, i = e / (D + 1), j = e % (D + 1);
+      const real* early = child + 2 * q * E;
+      const real* late = early + E + i * (D + 1);
+      real x = j == D ? late[D] : real(0);
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    if (off >= n) break;  // uniform over the warp
-    const Aff<real, D> y = shfl_up_aff<real, D>(x, off);
-    if (lane >= off) x = compose<real, D>(x, y);
+      for (int k = 0; k < D; ++k) x += late[k] * early[k * (D + 1) + j];
+      node[t] = x;
+    }
+    __syncwarp();
   }
-  return x;
 }
+
+// Delta entering every node from the one entering the root (x: D values per node, the tree's
+// numbering)
+template <class real, int D>
+__device__ __forceinline__ void tree_down(const real* tree, real* x, int n, int lane) {
+  constexpr int E = kEl<D>;
+  for (int m = 1; m < n; m <<= 1) {
+    const real* xp = x + (2 * n - 2 * m) * D;
+    real* xc = x + (2 * n - 4 * m) * D;
+    const real* child = tree + (2 * n - 4 * m) * E;
+    for (int t = lane; t < m * D; t += 32) {
+      const int q = t / D, i = t % D;
+      const real* early = child + 2 * q * E + i * (D + 1);
+      real y = early[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) y += early[k] * xp[q * D + k];
+      xc[2 * q * D + i] = xp[t];
+      xc[(2 * q + 1) * D + i] = y;
+    }
+    __syncwarp();
+  }
+}
+
+__device__ __forceinline__ int pow2_at_least(int n) {
+  int p = 1;
+  while (p < n) p <<= 1;
+  return p;
+}
+
+// bit pattern of |x|: orders like the value, NaN above everything
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 
 template <class real, int D, int KIND, int NT, int RPT>
 __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
   namespace cg = cooperative_groups;
-  constexpr int NW = NT / 32;
-  __shared__ real s_last[NT][D];       // each thread's last row of the iterate
-  __shared__ Aff<real, D> s_warp[NW];  // inclusive warp totals, then their prefixes
-  __shared__ Aff<real, D> s_tot;       // this block's element (read by later blocks)
+  constexpr int NW = NT / 32, E = kEl<D>, MAXB = 16;
+  // each warp's tree over its threads, and the Delta entering its nodes
+  extern __shared__ __align__(16) unsigned char block_smem[];
+  real (*s_tree)[63 * E] = reinterpret_cast<real (*)[63 * E]>(block_smem);
+  real (*s_x)[63 * D] = reinterpret_cast<real (*)[63 * D]>(block_smem + sizeof(real) * NW * 63 * E);
+  __shared__ real s_wtree[(2 * NW - 1) * E];  // the block's warps (root: the block's element)
+  __shared__ real s_wx[(2 * NW - 1) * D];
+  __shared__ real s_btree[(2 * MAXB - 1) * E];  // the blocks before this one
+  __shared__ real s_last[NT][D];  // each thread's last row of the iterate
+  __shared__ int s_votes[NW];     // 1: a row fails the test, 2: a non-finite entry
+  __shared__ int s_vote;          // this block's (read across the cluster)
+  __shared__ int s_all;           // the cluster's
   __shared__ real s_mx[NW];
   __shared__ double s_sq[NW];
-  __shared__ double s_part[2];         // this block's max scaled residual and sum r^2
-  __shared__ double s_stat[2];         // the cluster's
-  __shared__ real s_din[D];            // Delta entering this block's rows
+  __shared__ double s_part[2];  // this block's max scaled residual and sum r^2
   cg::cluster_group cl = cg::this_cluster();
   const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int64_t seq = blockIdx.x / CL;
@@ -116,19 +164,25 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
   const int64_t r0 = a.offsets[seq];
   const int64_t T = a.offsets[seq + 1] - r0;
   // rows spread evenly over the cluster's blocks (rpc each, in rank order), then over a
-  // block's threads (rpt each, <= RPT: the host sizes the cluster); the threads with rows
-  // are a prefix of each block, and whole warps without rows skip the float64 scans
+  // block's warps (rpt rows for each of a warp's first `per` lanes; the host sizes the
+  // cluster so that rpt <= RPT); the threads with rows are a prefix in (block, warp, lane)
+  // order
   const int64_t rpc = (T + CL - 1) / CL;
   const int rpt = (int)((rpc + NT - 1) / NT);
+  const int threads = rpt > 0 ? (int)((rpc + rpt - 1) / rpt) : 0;  // with rows, full block
+  const int per = (threads + NW - 1) / NW;
+  const int n = pow2_at_least(per);  // leaves of a warp's tree
   const int64_t cbeg = (int64_t)rank * rpc;
   const int64_t cend = cbeg + rpc < T ? cbeg + rpc : T;
-  const int64_t k0 = cbeg + (int64_t)tid * rpt;
-  const int nmine = cend - k0 <= 0 ? 0 : (cend - k0 < rpt ? (int)(cend - k0) : rpt);
-  const bool warp_rows = cbeg + (int64_t)(warp * 32) * rpt < cend;  // uniform over the warp
-  // the previous block (full whenever this one has rows) ends with thread (rpc - 1) / rpt
-  // (an empty sequence has rpt = 0 and no thread with rows: nothing is read)
-  const int prev_last = rpt > 0 ? (int)((rpc - 1) / rpt) : 0;
+  const int q = warp * per + lane;  // thread index among those with rows
+  const int64_t k0 = cbeg + (int64_t)q * rpt;
+  const int nmine = lane >= per || cend - k0 <= 0 ? 0 : (cend - k0 < rpt ? (int)(cend - k0) : rpt);
+  // the last thread of the previous block (full whenever this one has rows)
+  const int prev_last = threads - 1;
   const real scale = a.damp == DEER_DAMP_SCALE ? real(1) - a.dparam : real(1);
+  // the test in the kernel's precision: the largest value not above tol
+  const real tol = sizeof(real) == 8 ? (real)a.tol : (real)__double2float_rd(a.tol);
+  const auto thr_bits = mag_bits(a.reset_thr);
   real s[RPT][D];
   real s0[D];
 #pragma unroll
@@ -137,156 +191,118 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
   for (int k = 0; k < RPT; ++k)
 #pragma unroll
     for (int i = 0; i < D; ++i) s[k][i] = k < nmine ? a.s[(r0 + k0 + k) * D + i] : real(0);
+  real last[D];  // this thread's last row
+#pragma unroll
+  for (int i = 0; i < D; ++i) last[i] = real(0);
+#pragma unroll
+  for (int k = 0; k < RPT; ++k)
+#pragma unroll
+    for (int i = 0; i < D; ++i) last[i] = k < nmine ? s[k][i] : last[i];
   int passes = 0;
   bool done = false, nonfinite = false;
-  double merit = 0.0, mres = 0.0;
   int iters = 0;
+  real Fk[RPT][D], Ak[RPT][D][D];
   for (int it = 0;; ++it) {
     // the row before this thread's first is the previous thread's last, in this block or
-    // (thread 0) in the previous block of the cluster; a thread without rows is followed
-    // only by threads without rows
+    // in the previous block of the cluster; a thread without rows is followed only by
+    // threads without rows
+    if (nmine > 0) {
 #pragma unroll
-    for (int k = 0; k < RPT; ++k)
-      if (k == nmine - 1) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) s_last[tid][i] = s[k][i];
-      }
+      for (int i = 0; i < D; ++i) s_last[q][i] = last[i];
+    }
     cl.sync();
-    real prev[D];
+    real sp[D];
     if (nmine == 0) {
 #pragma unroll
-      for (int i = 0; i < D; ++i) prev[i] = real(0);  // unused: no rows
-    } else if (tid > 0) {
+      for (int i = 0; i < D; ++i) sp[i] = real(0);  // unused: no rows
+    } else if (q > 0) {
 #pragma unroll
-      for (int i = 0; i < D; ++i) prev[i] = s_last[tid - 1][i];
+      for (int i = 0; i < D; ++i) sp[i] = s_last[q - 1][i];
     } else if (rank > 0) {
       const real* pl = cl.map_shared_rank(&s_last[prev_last][0], rank - 1);
 #pragma unroll
-      for (int i = 0; i < D; ++i) prev[i] = pl[i];
+      for (int i = 0; i < D; ++i) sp[i] = pl[i];
     } else {
 #pragma unroll
-      for (int i = 0; i < D; ++i) prev[i] = s0[i];
+      for (int i = 0; i < D; ++i) sp[i] = s0[i];
     }
-    // 1. linearise, residual statistics, this thread's element; F and A are kept for the
-    //    apply pass
+    // 1. linearise, test, this thread's element; F and A are kept for the apply pass
     Aff<real, D> e = aff_identity<real, D>();
-    real Fk[RPT][D], Ak[RPT][D][D];
-    // largest scaled residual |r| / max(1, |s|) kept as a fraction (fn / fd, compared by
-    // cross-multiplication), so that one division per warp replaces one per entry (the
-    // float64 divide is a long sequence on this GPU); non-finite entries raise fnan
-    real fn = real(0), fd = real(1);
-    bool fnan = false;
-    double sq = 0.0;
-    {
-      real sp[D];
+    bool fail = false, bad = false;
 #pragma unroll
-      for (int i = 0; i < D; ++i) sp[i] = prev[i];
+    for (int k = 0; k < RPT; ++k) {
+      if (k < nmine) {
+        eval_f<real, D, KIND, 1>(a.dv, seq, r0 + k0 + k, sp, Fk[k], Ak[k], nullptr);
+        Aff<real, D> st;
 #pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        if (k < nmine) {
-          eval_f<real, D, KIND, 1>(a.dv, seq, r0 + k0 + k, sp, Fk[k], Ak[k], nullptr);
-          Aff<real, D> st;
+        for (int i = 0; i < D; ++i) {
+          const real r = s[k][i] - Fk[k][i];
+          st.v[i] = -r;
+          const auto rb = mag_bits(r), sb = mag_bits(s[k][i]);
+          const real lim = sb > mag_bits(real(1)) ? tol * rabs(s[k][i]) : tol;
+          fail |= rb > mag_bits(lim);
+          bad |= rb > mag_bits(kRealMax<real>) || sb > mag_bits(kRealMax<real>);
 #pragma unroll
-          for (int i = 0; i < D; ++i) {
-            const real r = s[k][i] - Fk[k][i];
-            st.v[i] = -r;
-            const real sabs = rabs(s[k][i]);
-            const real num = rabs(r), den = sabs > real(1) ? sabs : real(1);
-            if (!(num <= kRealMax<real>) || !(den <= kRealMax<real>)) {
-              fnan = true;
-            } else if (num * fd > fn * den) {
-              fn = num;
-              fd = den;
-            }
-            sq += (double)r * (double)r;
-#pragma unroll
-            for (int j = 0; j < D; ++j) {
-              Ak[k][i][j] *= scale;
-              st.P[i][j] = Ak[k][i][j];
-            }
+          for (int j = 0; j < D; ++j) {
+            if (scale != real(1)) Ak[k][i][j] *= scale;
+            st.P[i][j] = Ak[k][i][j];
           }
-          e = compose<real, D>(st, e);
-#pragma unroll
-          for (int i = 0; i < D; ++i) sp[i] = s[k][i];
         }
+        if (k == 0) e = st;
+        else e = compose<real, D>(st, e);
+#pragma unroll
+        for (int i = 0; i < D; ++i) sp[i] = s[k][i];
       }
     }
-    // 2. statistics and scan totals: per warp, per block, then across the cluster with one
-    //    barrier. Every block reduces the blocks' partials in the same order, so all take
-    //    the same decision; the scan is formed before the test and unused if it stops.
-    if (warp_rows) {
+    // 2. votes and elements up the trees
+    const int vote = (__any_sync(0xffffffffu, fail) ? 1 : 0) | (__any_sync(0xffffffffu, bad) ? 2 : 0);
+    if (lane == 0) s_votes[warp] = vote;
+    real* tree = s_tree[warp];
+    if (lane < n) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const real on = __shfl_xor_sync(0xffffffffu, fn, o);
-        const real od = __shfl_xor_sync(0xffffffffu, fd, o);
-        fnan |= __shfl_xor_sync(0xffffffffu, (int)fnan, o) != 0;
-        if (on * fd > fn * od) {
-          fn = on;
-          fd = od;
-        }
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      for (int i = 0; i < D; ++i) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) tree[lane * E + i * (D + 1) + j] = e.P[i][j];
+        tree[lane * E + i * (D + 1) + D] = e.v[i];
       }
-      if (lane == 0) {
-        s_mx[warp] = fnan ? real(NAN) : fn / fd;
-        s_sq[warp] = sq;
-      }
-    } else if (lane == 0) {
-      s_mx[warp] = real(0);
-      s_sq[warp] = 0.0;
     }
-    // 3. scan of the elements: lanes, warps, then the blocks of the cluster
-    const Aff<real, D> inc = warp_rows ? warp_scan_aff<real, D>(e, lane) : e;  // e = I
-    if (lane == 31) s_warp[warp] = inc;
+    __syncwarp();
+    tree_up<real, D>(tree, n, lane);
+    for (int t = lane; t < E; t += 32) s_wtree[warp * E + t] = tree[(2 * n - 2) * E + t];
     __syncthreads();
     if (warp == 0) {
-      Aff<real, D> wt = lane < NW ? s_warp[lane] : aff_identity<real, D>();
-      wt = warp_scan_aff<real, D>(wt, lane, NW);
-      if (lane < NW) s_warp[lane] = wt;
-      if (lane == NW - 1) s_tot = wt;
-      double bm = lane < NW ? (double)s_mx[lane] : 0.0;
-      double bs = lane < NW ? s_sq[lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        bm = nanmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-        bs += __shfl_xor_sync(0xffffffffu, bs, o);
-      }
+      tree_up<real, D>(s_wtree, NW, lane);
       if (lane == 0) {
-        s_part[0] = bm;
-        s_part[1] = bs;
+        int v = 0;
+        for (int w = 0; w < NW; ++w) v |= s_votes[w];
+        s_vote = v;
       }
     }
     cl.sync();
     if (warp == 0) {
-      double bm = 0.0, bs = 0.0;
-      if (lane < CL) {
-        const double* pp = cl.map_shared_rank(&s_part[0], lane);
-        bm = pp[0];
-        bs = pp[1];
+      // the cluster's vote; the blocks before this one: Delta entering this block
+      const int v = lane < CL ? *cl.map_shared_rank(&s_vote, lane) : 0;
+      const int any = (__any_sync(0xffffffffu, v & 1) ? 1 : 0) |
+                      (__any_sync(0xffffffffu, v & 2) ? 2 : 0);
+      const int nb = pow2_at_least(rank);
+      for (int t = lane; t < nb * E; t += 32) {
+        const int b = t / E, x = t % E;
+        s_btree[t] = b < rank ? *cl.map_shared_rank(&s_wtree[(2 * NW - 2) * E + x], b)
+                              : (x % (D + 1) == x / (D + 1) ? real(1) : real(0));
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        bm = nanmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-        bs += __shfl_xor_sync(0xffffffffu, bs, o);
-      }
-      if (lane == 0) {
-        s_stat[0] = bm;
-        s_stat[1] = bs;
-      }
-      // the blocks before this one, composed in order: Delta entering this block
-      Aff<real, D> bt = lane < CL ? *cl.map_shared_rank(&s_tot, lane) : aff_identity<real, D>();
-      bt = warp_scan_aff<real, D>(bt, lane, CL);
-      const Aff<real, D> ex = shfl_up_aff<real, D>(bt, 1);
-      if (lane == rank) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) s_din[i] = rank > 0 ? ex.v[i] : real(0);
-      }
+      __syncwarp();
+      tree_up<real, D>(s_btree, nb, lane);
+      if (lane < D)
+        s_wx[(2 * NW - 2) * D + lane] =
+            rank > 0 ? s_btree[(2 * nb - 2) * E + lane * (D + 1) + D] : real(0);
+      if (lane == 0) s_all = any;
+      __syncwarp();
+      tree_down<real, D>(s_wtree, s_wx, NW, lane);
     }
     __syncthreads();
-    const double bm = s_stat[0], bs = s_stat[1];
-    merit = 0.5 * bs;
-    mres = bm;
-    nonfinite = !(bm <= DBL_MAX);
-    passes = bm <= a.tol ? passes + 1 : 0;
+    const int all = s_all;
+    nonfinite = (all & 2) != 0;
+    passes = all == 0 ? passes + 1 : 0;
     if (passes >= a.confirm) {
       done = true;
       iters = it;
@@ -294,35 +310,14 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
     }
     iters = it < a.max_iters ? it + 1 : it;
     if ((nonfinite && !a.reset) || it >= a.max_iters) break;
-    real din[D] = {};
-    if (warp_rows) {
-      // then the warps before in this block, then the lanes before in this warp
-      real db[D], dw[D];
+    // 3. Delta down to this thread, then through its rows
+    real* xs = s_x[warp];
+    if (lane < D) xs[(2 * n - 2) * D + lane] = s_wx[warp * D + lane];
+    __syncwarp();
+    tree_down<real, D>(tree, xs, n, lane);
+    real din[D];
 #pragma unroll
-      for (int i = 0; i < D; ++i) db[i] = s_din[i];
-      if (warp > 0) {
-        const Aff<real, D>& wp = s_warp[warp - 1];
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          real x = wp.v[i];
-#pragma unroll
-          for (int k = 0; k < D; ++k) x += wp.P[i][k] * db[k];
-          dw[i] = x;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < D; ++i) dw[i] = db[i];
-      }
-      Aff<real, D> ex = shfl_up_aff<real, D>(inc, 1);
-      if (lane == 0) ex = aff_identity<real, D>();
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        real x = ex.v[i];
-#pragma unroll
-        for (int k = 0; k < D; ++k) x += ex.P[i][k] * dw[k];
-        din[i] = x;
-      }
-    }
+    for (int i = 0; i < D; ++i) din[i] = lane < n ? xs[lane * D + i] : real(0);
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       if (k < nmine) {
@@ -337,7 +332,8 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
 #pragma unroll
         for (int i = 0; i < D; ++i) {
           const real y = s[k][i] + dn[i];
-          s[k][i] = (a.reset && !(y <= a.reset_thr && y >= -a.reset_thr)) ? real(0) : y;
+          s[k][i] = a.reset && mag_bits(y) > thr_bits ? real(0) : y;
+          last[i] = s[k][i];
           din[i] = dn[i];
         }
       }
@@ -345,23 +341,80 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
     // (the next iteration's first cluster barrier orders the rewrites of the shared
     // buffers after every block's reads of them)
   }
-  cl.sync();  // no block leaves while another may still read its shared memory
+  // The statistics of the last iterate: the largest scaled residual |r| / max(1, |s|), kept as
+  // a fraction fn / fd compared by cross-multiplication (one division per warp), and sum r^2.
+  {
+    real fn = real(0), fd = real(1);
+    bool fnan = false;
+    double sq = 0.0;
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+      if (k < nmine) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          const real r = s[k][i] - Fk[k][i];
+          const real sabs = rabs(s[k][i]);
+          const real num = rabs(r), den = sabs > real(1) ? sabs : real(1);
+          if (!(num <= kRealMax<real>) || !(den <= kRealMax<real>)) {
+            fnan = true;
+          } else if (num * fd > fn * den) {
+            fn = num;
+            fd = den;
+          }
+          sq += (double)r * (double)r;
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const real on = __shfl_xor_sync(0xffffffffu, fn, o);
+      const real od = __shfl_xor_sync(0xffffffffu, fd, o);
+      fnan |= __shfl_xor_sync(0xffffffffu, (int)fnan, o) != 0;
+      if (on * fd > fn * od) {
+        fn = on;
+        fd = od;
+      }
+      sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    if (lane == 0) {
+      s_mx[warp] = fnan ? real(NAN) : fn / fd;
+      s_sq[warp] = sq;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double bm = 0.0, bs = 0.0;
+      for (int w = 0; w < NW; ++w) {
+        bm = nanmax(bm, (double)s_mx[w]);
+        bs += s_sq[w];
+      }
+      s_part[0] = bm;
+      s_part[1] = bs;
+    }
+  }
 #pragma unroll
   for (int k = 0; k < RPT; ++k)
     if (k < nmine)
 #pragma unroll
       for (int i = 0; i < D; ++i) a.s[(r0 + k0 + k) * D + i] = s[k][i];
+  cl.sync();
   if (tid == 0 && rank == 0) {
+    double bm = 0.0, bs = 0.0;
+    for (int b = 0; b < CL; ++b) {
+      const double* pp = cl.map_shared_rank(&s_part[0], b);
+      bm = nanmax(bm, pp[0]);
+      bs += pp[1];
+    }
     SeqInfo inf = a.info[seq];
     inf.iters = iters;
     inf.done = done ? 1 : 0;
     inf.passes = passes;
-    inf.merit = merit;
-    inf.max_resid = mres;
+    inf.merit = 0.5 * bs;
+    inf.max_resid = bm;
     a.info[seq] = inf;
     if (nonfinite) atomicAdd(&a.flags->n_nonfinite, 1);
     if (!done) atomicAdd(&a.flags->n_active, 1);
   }
+  cl.sync();  // no block leaves while another may still read its shared memory
 }
 
 // Threads per block and the most rows per thread by state size (each thread keeps its
@@ -411,7 +464,14 @@ static cudaError_t block_launch(const BlockSolveArgs<real>& a, cudaStream_t st) 
   attr[0].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg{};
   cfg.blockDim = dim3(kBlockThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = sizeof(real) * (kBlockThreads / 32) * 63 * (kEl<D> + D);
+  static thread_local bool smem_ok = false;  // per host thread: the attribute took
+  if (!smem_ok) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+    smem_ok = true;
+  }
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
