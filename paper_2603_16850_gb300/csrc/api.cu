@@ -137,18 +137,21 @@ static bool use_compensated(const deer_dynamics* f, const deer_options* o) {
          o->damp != DEER_DAMP_ELK && (f->d == 4 || f->d == 8 || f->d == 16 || f->d == 32);
 }
 
-static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N) {
+static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N, bool lean) {
   if (use_diag_lookback(o, d)) return diag_lb_chunk(d);
   if (o->chunk > 0) return o->chunk;
   if (o->jac == DEER_JAC_FULL && d >= 16) return 32;
   if (o->jac == DEER_JAC_FULL) {
     // Shorter chunks while the chunk passes (d lanes per chunk) leave the GPU short of four
     // warps per SM, as long as the per-sequence carry stays the shorter chain: it walks
-    // T / L chunks at about half the time of the chunk passes' L rows. Mass action d = 8,
+    // T / L chunks at about half the time of the chunk passes' L rows in float32; a float64
+    // row costs several times a carry step, except under dense ELK, whose covariance carry
+    // inverts a matrix per chunk. Mass action d = 8,
     // float64, 37 x 1501 rows: L = 16 solves in 5.5 ms, L = 32 in 8.0, L = 64 in 15.2.
     int L = 64;
     const int64_t T = B > 0 ? N / B : 0;
-    while (L > 16 && N / L * d < 152 * 4 * 32 && T <= 2 * (int64_t)L * L) L /= 2;
+    const int64_t r = o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK ? 8 : 2;
+    while (!lean && L > 16 && N / L * d < 152 * 4 * 32 && T <= r * L * L) L /= 2;
     return L;
   }
   return 128;
@@ -166,15 +169,17 @@ static int grad_chunk(const deer_dynamics* f, const deer_options* o) {
 // far from overflowing 64 bits (d <= 64).
 constexpr int64_t kMaxRows = int64_t(1) << 44;
 
+// `lean` (deer_solve_noalloc, whose scratch is a fixed area): no tables or chunk counts beyond
+// what the plain forms of the kernels need.
 static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer_options* o,
-                        Layout& ly) {
+                        Layout& ly, bool lean = false) {
   if (!f || !o || B < 0 || N < 0) return false;
   if (N > kMaxRows || B > kMaxRows || f->d <= 0 || f->d > 64) return false;
   if (o->prec != DEER_FP64 && o->prec != DEER_FP32 && o->prec != DEER_MIXED_BF16) return false;
   const size_t rs = o->prec == DEER_FP32 ? 4 : 8;
   const bool mixed = o->prec == DEER_MIXED_BF16;
   const int d = f->d;
-  const int L = choose_chunk(o, d, B, N);
+  const int L = choose_chunk(o, d, B, N, lean);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
   ly.n_chunks_max = N / L + B + 1;
@@ -198,6 +203,11 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
     ly.ma_stride = (ly.ma_stride + 3) / 4 * 4;
     const bool shared = f->params_stride == 0 && f->topology_stride == 0;
     ly.n_ma = shared ? 1 : B;
+    ly.ma = take((size_t)(ly.n_ma > 0 ? ly.n_ma : 1) * ly.ma_stride * rs);
+  }
+  if (f->kind == DEER_F_LANGEVIN_2WELL && !lean) {
+    ly.ma_stride = 4 * (int64_t)d + 2;
+    ly.n_ma = f->params_stride == 0 ? 1 : B;
     ly.ma = take((size_t)(ly.n_ma > 0 ? ly.n_ma : 1) * ly.ma_stride * rs);
   }
   if (f->kind == DEER_F_GRU) ly.gru_M = take((size_t)d * d * rs);
@@ -229,7 +239,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   ly.aggv = take((size_t)C * d * ars);
   ly.cin = take((size_t)C * d * ars);
   ly.segP = ly.segv = ly.segin = p;
-  if (o->jac == DEER_JAC_FULL && d > 1) {
+  if (o->jac == DEER_JAC_FULL && d > 1 && !lean) {
     // segments of at least 8 chunks (two-level carry)
     const size_t S = (size_t)(C / 8 + B + 1);
     ly.segP = take(S * d * d * ars);
@@ -332,7 +342,7 @@ static DynView<real> make_view(const deer_dynamics* f, const void* x, char* ws,
   v.topo = f->topology;
   v.tstride = f->topology_stride;
   v.x = static_cast<const real*>(x);
-  v.ma = ws ? reinterpret_cast<const real*>(ws + ly.ma) : nullptr;
+  v.ma = ws && ly.n_ma > 0 ? reinterpret_cast<const real*>(ws + ly.ma) : nullptr;
   v.ma_stride = ly.n_ma == 1 ? 0 : ly.ma_stride;
   v.gru_M = ws ? reinterpret_cast<const real*>(ws + ly.gru_M) : nullptr;
   return v;
@@ -456,7 +466,11 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
   if ((double)tol_f > o->tol) tol_f = std::nextafter(tol_f, 0.f);
 
   DynView<real> dv = make_view<real>(f, x_, ws, ly);
-  if (ly.n_ma > 0) {
+  if (f->kind == DEER_F_LANGEVIN_2WELL) {
+    DEER_CK(launch_langevin_setup<real>(ly.n_ma, d, static_cast<const real*>(f->params),
+                                        f->params_stride, reinterpret_cast<real*>(ws + ly.ma),
+                                        ly.ma_stride, st));
+  } else if (ly.n_ma > 0) {
     DEER_CK(launch_ma_setup<real>(ly.n_ma, d, f->n_reactions, static_cast<const real*>(f->params),
                                   f->params_stride, f->topology, f->topology_stride,
                                   reinterpret_cast<real*>(ws + ly.ma), ly.ma_stride,
@@ -1137,7 +1151,11 @@ static deer_status jacobians_at(const deer_dynamics* f, int64_t B, int64_t T, co
     DEER_CK(launch_check(ca, st));
   }
   dv = make_view<real>(f, x_, ws, ly);
-  if (ly.n_ma > 0) {
+  if (f->kind == DEER_F_LANGEVIN_2WELL) {
+    DEER_CK(launch_langevin_setup<real>(ly.n_ma, d, static_cast<const real*>(f->params),
+                                        f->params_stride, reinterpret_cast<real*>(ws + ly.ma),
+                                        ly.ma_stride, st));
+  } else if (ly.n_ma > 0) {
     DEER_CK(launch_ma_setup<real>(ly.n_ma, d, f->n_reactions, static_cast<const real*>(f->params),
                                   f->params_stride, f->topology, f->topology_stride,
                                   reinterpret_cast<real*>(ws + ly.ma), ly.ma_stride,
@@ -1582,7 +1600,7 @@ static deer_status solve_noalloc_impl(const deer_dynamics* f, int64_t B, int64_t
   if (B > 0 && T > kMaxRows / B) return DEER_ERR_INVALID;
   const int64_t N = B * T;
   Layout ly;
-  if (!make_layout(f, B, N, o, ly)) return DEER_ERR_INVALID;
+  if (!make_layout(f, B, N, o, ly, true)) return DEER_ERR_INVALID;
   const size_t info_bytes = align_up((size_t)B * sizeof(deer_info));
   if (ly.total + info_bytes > kNoAllocScratchBytes) {
     snprintf(g_err, sizeof(g_err),

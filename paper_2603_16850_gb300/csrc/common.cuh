@@ -174,6 +174,33 @@ __device__ __forceinline__ unsigned long long dbits(double v) {
 template <class real>
 __device__ __forceinline__ real rabs(real v) { return v < real(0) ? -v : v; }
 
+// bit pattern of |x|: orders like the value, NaN above everything
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+
+// 1 / x by Newton's iteration y <- y + y (1 - x y) from a float32 reciprocal of the mantissa
+// (relative error 2^-22, squared twice): four FP64 instructions, within two ulp. Non-finite,
+// zero and subnormal x, and results near the subnormal range, take the division.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  if (e == 0 || e >= 2044) return 1.0 / x;
+  // mantissa m in [1, 2), as double and truncated to float
+  const double m = __hiloint2double((int)(0x3ff00000u | (hi & 0xfffffu)), (int)lo);
+  const unsigned yb =
+      __float_as_uint(1.f / __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29)));
+  double y = __hiloint2double(((int)(yb >> 23) - 127 + 1023) << 20 | (int)((yb & 0x7fffffu) >> 3),
+                              (int)(yb << 29));
+  y = fma(y, fma(-m, y, 1.0), y);
+  y = fma(y, fma(-m, y, 1.0), y);
+  // times 2^(1023 - e), with the sign of x
+  return __hiloint2double((__double2hiint(y) + ((1023 - e) << 20)) | (int)(hi & 0x80000000u),
+                          __double2loint(y));
+}
+__device__ __forceinline__ float recip(float x) { return 1.f / x; }
+
 // NaN-propagating maximum of two non-negative doubles.
 __device__ __forceinline__ double nanmax(double a, double b) {
   return (b > a || b != b) ? b : a;

@@ -282,21 +282,26 @@ __device__ __forceinline__ void langevin_eval(const DynView<real>& dv, int64_t s
   const real* m2 = p + D;
   const real* v1 = p + 2 * D;
   const real* v2 = p + 3 * D;
+  // reciprocal variances and logarithms, from the table built once per solve where there is
+  // one (k_langevin_setup): in float64 they were three quarters of a row's instructions
+  // (linearisation of 40000 rows, d = 4: 82 -> 32 us)
+  const real* tab = dv.ma ? dv.ma + seq * dv.ma_stride : nullptr;
   real q1 = real(0), q2 = real(0);
   real z1[D], z2[D];  // (s - m_k) / v_k
 #pragma unroll Unroll<D>::n
   for (int i = 0; i < D; ++i) {
     const real a1 = s[i] - __ldg(m1 + i), a2 = s[i] - __ldg(m2 + i);
-    const real iv1 = real(1) / __ldg(v1 + i), iv2 = real(1) / __ldg(v2 + i);
+    const real iv1 = tab ? __ldg(tab + i) : real(1) / __ldg(v1 + i);
+    const real iv2 = tab ? __ldg(tab + D + i) : real(1) / __ldg(v2 + i);
     z1[i] = a1 * iv1;
     z2[i] = a2 * iv2;
-    q1 += log(__ldg(v1 + i)) + a1 * z1[i];
-    q2 += log(__ldg(v2 + i)) + a2 * z2[i];
+    q1 += (tab ? __ldg(tab + 2 * D + i) : log(__ldg(v1 + i))) + a1 * z1[i];
+    q2 += (tab ? __ldg(tab + 3 * D + i) : log(__ldg(v2 + i))) + a2 * z2[i];
   }
-  const real l1 = log(__ldg(p + 4 * D)) - real(0.5) * q1;
-  const real l2 = log(__ldg(p + 4 * D + 1)) - real(0.5) * q2;
-  const real g1 = real(1) / (real(1) + exp(l2 - l1));
-  const real g2 = real(1) / (real(1) + exp(l1 - l2));
+  const real l1 = (tab ? __ldg(tab + 4 * D) : log(__ldg(p + 4 * D))) - real(0.5) * q1;
+  const real l2 = (tab ? __ldg(tab + 4 * D + 1) : log(__ldg(p + 4 * D + 1))) - real(0.5) * q2;
+  const real g1 = recip(real(1) + exp(l2 - l1));
+  const real g2 = recip(real(1) + exp(l1 - l2));
   const real dt = dv.dt;
   const real amp = sqrt(real(2) * dt);
 #pragma unroll Unroll<D>::n
@@ -310,7 +315,8 @@ __device__ __forceinline__ void langevin_eval(const DynView<real>& dv, int64_t s
 #pragma unroll Unroll<D>::n
     for (int i = 0; i < D; ++i) {
       const real ei = z2[i] - z1[i];
-      const real hii = g1 / __ldg(v1 + i) + g2 / __ldg(v2 + i);
+      const real hii = tab ? g1 * __ldg(tab + i) + g2 * __ldg(tab + D + i)
+                           : g1 / __ldg(v1 + i) + g2 / __ldg(v2 + i);
       if constexpr (JM == 2) {
         Ad[i] = real(1) - dt * (hii - g12 * ei * ei);
       } else {

@@ -133,12 +133,6 @@ __device__ __forceinline__ int pow2_at_least(int n) {
   return p;
 }
 
-// bit pattern of |x|: orders like the value, NaN above everything
-__device__ __forceinline__ unsigned long long mag_bits(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-}
-__device__ __forceinline__ unsigned mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-
 template <class real, int D, int KIND, int NT, int RPT>
 __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
   namespace cg = cooperative_groups;

@@ -32,27 +32,6 @@ constexpr int elk_lanes() { return D * D < 32 ? D * D : 32; }
 template <int D>
 constexpr int elk_carry_lanes() { return D == 8 ? 64 : D == 16 ? 128 : elk_lanes<D>(); }
 
-// 1 / x by Newton's iteration y <- y + y (1 - x y) from a float32 reciprocal of the mantissa
-// (relative error 2^-22, squared twice): four FP64 instructions, within two ulp. Non-finite,
-// zero and subnormal x, and results near the subnormal range, take the division.
-__device__ __forceinline__ double recip(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  if (e == 0 || e >= 2044) return 1.0 / x;
-  // mantissa m in [1, 2), as double and truncated to float
-  const double m = __hiloint2double((int)(0x3ff00000u | (hi & 0xfffffu)), (int)lo);
-  const unsigned yb =
-      __float_as_uint(1.f / __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29)));
-  double y = __hiloint2double(((int)(yb >> 23) - 127 + 1023) << 20 | (int)((yb & 0x7fffffu) >> 3),
-                              (int)(yb << 29));
-  y = fma(y, fma(-m, y, 1.0), y);
-  y = fma(y, fma(-m, y, 1.0), y);
-  // times 2^(1023 - e), with the sign of x
-  return __hiloint2double((__double2hiint(y) + ((1023 - e) << 20)) | (int)(hi & 0x80000000u),
-                          __double2loint(y));
-}
-__device__ __forceinline__ float recip(float x) { return 1.f / x; }
-
 // larger magnitude = larger key, from the bit pattern (no FP64 comparison)
 __device__ __forceinline__ int mag_key(double x) { return __double2hiint(x) & 0x7fffffff; }
 __device__ __forceinline__ int mag_key(float x) { return __float_as_int(x) & 0x7fffffff; }

@@ -5,6 +5,37 @@
 
 namespace deer {
 
+// Two-well Langevin: per sequence (or once when shared) 1/v1 | 1/v2 | log v1 | log v2 |
+// log w1, log w2.
+template <class real>
+__global__ void __launch_bounds__(128) k_langevin_setup(int64_t n_seq, int d,
+                                                        const real* __restrict__ params,
+                                                        int64_t pstride, real* __restrict__ out,
+                                                        int64_t ostride) {
+  const int n = 4 * d + 2;
+  const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (id >= n_seq * n) return;
+  const int64_t seq = id / n;
+  const int e = (int)(id - seq * n);
+  const real* p = params + seq * pstride;
+  out[seq * ostride + e] = e < 2 * d ? real(1) / p[2 * d + e]
+                                     : log(p[e]);
+}
+
+template <class real>
+cudaError_t launch_langevin_setup(int64_t n_seq, int d, const real* params, int64_t pstride,
+                                  real* out, int64_t ostride, cudaStream_t st) {
+  if (n_seq == 0) return cudaSuccess;
+  k_langevin_setup<real><<<grid_for(n_seq * (4 * d + 2), 128), 128, 0, st>>>(
+      n_seq, d, params, pstride, out, ostride);
+  note_launch();
+  return cudaGetLastError();
+}
+template cudaError_t launch_langevin_setup<float>(int64_t, int, const float*, int64_t, float*,
+                                                  int64_t, cudaStream_t);
+template cudaError_t launch_langevin_setup<double>(int64_t, int, const double*, int64_t, double*,
+                                                   int64_t, cudaStream_t);
+
 template <class real>
 cudaError_t launch_init_models(const InitArgs<real>& a, cudaStream_t st) {
   switch (a.dv.kind) {

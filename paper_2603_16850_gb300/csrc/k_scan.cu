@@ -214,8 +214,8 @@ cudaError_t launch_check(const CheckArgs& a, cudaStream_t st) {
 
 template <class real>
 __device__ __forceinline__ real reset_val(real v, real thr, int reset) {
-  if (reset && !(v <= thr && v >= -thr)) return real(0);
-  return v;
+  // (bit patterns: no float64 comparison, NaN orders above every threshold)
+  return reset && mag_bits(v) > mag_bits(thr) ? real(0) : v;
 }
 
 // 16 bytes (four floats or two doubles) from a 16-byte aligned address. Plain (coherent)
@@ -714,6 +714,69 @@ __global__ void __launch_bounds__(32) k_dense_chunk_ring(DenseScanArgs<real> a) 
   vo[lane] = v;
 }
 
+// Chunk pass, float64, few chunks: a warp per chunk with the entries of [P | v] spread over
+// its lanes. A warp issues one FP64 instruction per 64 clocks whatever its active lanes, so
+// while chunks are too few to give every SM sub-partition (608) a warp of whole groups, one
+// entry per lane shortens a row from d^2 + d instructions to d (d = 4, 5) or 3 d (d = 8).
+// Langevin, d = 4, 4 x 10000 rows: 62 us a pass in chunks of 64 rows, 14 us so in chunks of
+// 32. The sums run in the same order.
+template <int D, bool SEG>
+__global__ void __launch_bounds__(32) k_dense_chunk_entry(DenseScanArgs<double> a) {
+  constexpr int K = 8, E = D * (D + 1), EPL = (E + 31) / 32;
+  __shared__ double sA[K][D * D], sB[K][D], sX[2][E];
+  const int lane = threadIdx.x;
+  Span p;
+  if (!get_span<SEG>(a, blockIdx.x, p)) return;
+  const double *A0, *b0;
+  double *Po, *vo;
+  span_ptrs<SEG, double, D>(a, p, A0, b0, Po, vo);
+  auto issue = [&](int t) {
+    if (t < p.n) {
+      const int s = t & (K - 1);
+      for (int e = lane; e < D * D; e += 32)
+        cp_async_small<8>(&sA[s][e], A0 + t * (int64_t)(D * D) + e);
+      if (lane < D) cp_async_small<8>(&sB[s][lane], b0 + t * D + lane);
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int t = 0; t < K - 1; ++t) issue(t);
+  int row[EPL], col[EPL];
+  double x[EPL];
+#pragma unroll
+  for (int m = 0; m < EPL; ++m) {
+    const int e = lane + 32 * m < E ? lane + 32 * m : E - 1;
+    row[m] = e / (D + 1);
+    col[m] = e % (D + 1);
+    x[m] = row[m] == col[m] ? 1.0 : 0.0;
+  }
+  for (int t = 0; t < p.n; ++t) {
+    double* X = sX[t & 1];
+#pragma unroll
+    for (int m = 0; m < EPL; ++m)
+      if (lane + 32 * m < E) X[lane + 32 * m] = x[m];
+    cp_async_wait<K - 2>();
+    __syncwarp();  // row t and every entry of [P | v] in place; row t - 1's slot is free
+    issue(t + K - 1);
+    const double* A = sA[t & (K - 1)];
+#pragma unroll
+    for (int m = 0; m < EPL; ++m) {
+      if (!p.need_P && col[m] != D) continue;
+      double y = col[m] == D ? sB[t & (K - 1)][row[m]] : 0.0;
+#pragma unroll
+      for (int k = 0; k < D; ++k) y += A[row[m] * D + k] * X[k * (D + 1) + col[m]];
+      x[m] = y;
+    }
+  }
+  cp_async_wait<0>();
+#pragma unroll
+  for (int m = 0; m < EPL; ++m)
+    if (lane + 32 * m < E) {
+      if (col[m] == D) vo[row[m]] = x[m];
+      else Po[row[m] * D + col[m]] = x[m];
+    }
+}
+
 // Chunk pass, d = 32: one chunk per block of four warps. The staged rows of A_t are shared
 // by the block (its 128 threads copy the 4 KB block together); warp w forms rows
 // 8w .. 8w+7 of P <- A_t P for all 32 columns (lane j owns column j), the new rows meet
@@ -1150,6 +1213,14 @@ static void dense_chunk_launch(const DenseScanArgs<real>& a, int64_t spans, unsi
     }
     k_dense_chunk_ring4<real, SEG><<<g, 128, 0, st>>>(a);
   } else {
+    if constexpr (sizeof(real) == 8 && D >= 4 && D <= 8) {
+      // warps per sub-partition x instructions per row: entries against whole groups
+      const int64_t warps = (spans * ny + 607) / 608;
+      if (warps * (D == 8 ? 3 : 1) < D + 1) {
+        k_dense_chunk_entry<D, SEG><<<dim3((unsigned)spans, ny), 32, 0, st>>>(a);
+        return;
+      }
+    }
     k_dense_chunk_ring<real, D, SEG><<<g, 32, 0, st>>>(a);
   }
 }

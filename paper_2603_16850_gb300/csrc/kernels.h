@@ -181,6 +181,10 @@ template <class real>
 cudaError_t launch_linearize(const LinArgs<real>& a, cudaStream_t st);
 template <class real>
 cudaError_t launch_rollout(const RolloutArgs<real>& a, cudaStream_t st);
+// two-well Langevin: reciprocal variances and logarithms of each parameter set
+template <class real>
+cudaError_t launch_langevin_setup(int64_t n_seq, int d, const real* params, int64_t pstride,
+                                  real* out, int64_t ostride, cudaStream_t st);
 template <class real>
 cudaError_t launch_gru_setup(int d, const real* params, int d_in, real* M, cudaStream_t st);
 // Input gradient of the adjoint: dx[row] = lambda_row^T d f_row / d x_row at s_{row-1}.

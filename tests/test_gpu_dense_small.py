@@ -70,3 +70,25 @@ def test_default_chunk_of_small_batches(B, T, d):
     s, _ = deer.deer_solve(dyn, _t(p["s0"]), T, **o)
     s64, _ = deer.deer_solve(dyn, _t(p["s0"]), T, chunk=64, **o)
     assert _relerr(s.cpu().numpy(), s64.cpu().numpy()) <= 1e-11
+
+
+@pytest.mark.parametrize("d", [4, 5, 8])
+def test_entry_and_group_forms_agree(d):
+    """Float64: 5000 chunks take a group of lanes per chunk, an eighth of them a warp per
+    chunk with its entries spread over the lanes; every sum runs in the same order, so one
+    Newton step is the same bit for bit."""
+    import paper_2603_16850_gb300 as deer
+    B, T = 40, 1000
+    if d == 5:
+        p = synth.word_problem(B, T, seed=7, d=d)
+        dyn = deer.Dynamics.permute(d, torch.float64, DEV)
+    else:
+        p = synth.mean_field_rnn(B, T, d, 0.9, seed=7)
+        dyn = deer.Dynamics.rnn_tanh(_t(p["W"]))
+    x, s0 = _t(p["x"]), _t(p["s0"])
+    o = dict(jac="full", tol=0.0, max_iters=1, init="s0", chunk=8, block_solve=False)
+    whole, _ = deer.deer_solve(dyn, s0, T, x.reshape(-1, d), **o)
+    for b in range(0, B, 5):
+        part, _ = deer.deer_solve(dyn, s0[b:b + 5].contiguous(), T,
+                                  x[b:b + 5].reshape(-1, d).contiguous(), **o)
+        assert torch.equal(part, whole[b * T:(b + 5) * T]), b
