@@ -536,6 +536,11 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
     la.adj_e = reinterpret_cast<const int32_t*>(ws + ly.adj_e);
     la.adj_stride = f->topology_stride ? 4 * (int64_t)f->n_reactions : 0;
   }
+  // mean-field RNN, d = 32, float32: the Jacobians as their column factors (tensor-core mode)
+  const bool rnn_factored = sizeof(real) == 4 && f->kind == DEER_F_RNN_TANH && d == 32 &&
+                            o->jac == DEER_JAC_FULL && o->damp != DEER_DAMP_ELK &&
+                            g_tensor_cores.load() != 0;
+  la.factored = rnn_factored;
   real* slo = ly.cs ? reinterpret_cast<real*>(ws + ly.slo) : nullptr;
   if (slo) {
     // the compensation terms start at zero (the initial guess is a plain float32 state)
@@ -781,6 +786,9 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
         }
         const cudaError_t e = launch_elk_dense<real>(ea, lst);
         if (e != cudaSuccess) return e;
+      }
+      if constexpr (sizeof(real) == 4) {
+        if (rnn_factored) return launch_rnn_scan(dsa, dv, lst);
       }
       return launch_dense_scan<real>(dsa, lst);
     }

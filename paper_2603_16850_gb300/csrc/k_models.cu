@@ -54,11 +54,13 @@ constexpr int kRnnRows = 16;  // consecutive rows per lane group in k_lin_rnn_wi
 // entry i of s_{t-1}, F_t, r_t, b_t; tanh(s_j) and its derivative arrive by shuffles and
 // lane i writes row i of A_t = W diag(1 - tanh(s_{t-1})^2).
 // ----------------------------------------------------------------------------
+constexpr int kJacFactored = 100;  // full Jacobian as its column factors (LinArgs::factored)
+
 template <class real, int D, int JAC>
 __global__ void __launch_bounds__(128) k_lin_rnn_wide(LinArgs<real> a) {
   constexpr int GROUPS = 128 / D;
   constexpr int VW = 16 / (int)sizeof(real);
-  __shared__ __align__(16) real sT[GROUPS][D * (D + 1)];  // transpose tile of A_t
+  __shared__ __align__(16) real sT[GROUPS][JAC == DEER_JAC_FULL ? D * (D + 1) : 1];  // transpose tile of A_t
   const int grp = threadIdx.x / D, lane = threadIdx.x % D;
   const unsigned gmask = D == 32 ? 0xffffffffu : (0xffffu << (16 * ((threadIdx.x >> 4) & 1)));
   // each group walks kRnnRows consecutive active rows; the residual statistics of a
@@ -66,6 +68,7 @@ __global__ void __launch_bounds__(128) k_lin_rnn_wide(LinArgs<real> a) {
   // of once per row, which keeps the accumulator atomics of a long sequence uncontended
   const int64_t ar0 = (blockIdx.x * (int64_t)GROUPS + grp) * kRnnRows;
   int64_t cur = -1;
+  real w[D];  // this lane's row of W
   real mx = real(0), sq = real(0);
   unsigned long long key = 0ull;  // first failing row (sliding window)
   for (int rr_i = 0; rr_i < kRnnRows; ++rr_i) {
@@ -79,23 +82,22 @@ __global__ void __launch_bounds__(128) k_lin_rnn_wide(LinArgs<real> a) {
       mx = real(0);
       sq = real(0);
       key = 0ull;
+      const real* Wr = a.dv.params + seq * a.dv.pstride + lane * D;
+#pragma unroll
+      for (int k = 0; k < D; k += VW) {
+        if constexpr (sizeof(real) == 4) {
+          const float4 q = __ldg(reinterpret_cast<const float4*>(Wr + k));
+          w[k] = q.x; w[k + 1] = q.y; w[k + 2] = q.z; w[k + 3] = q.w;
+        } else {
+          const double2 q = __ldg(reinterpret_cast<const double2*>(Wr + k));
+          w[k] = q.x; w[k + 1] = q.y;
+        }
+      }
     }
     const int64_t first = __ldg(a.bt.offsets + seq);
     const real sp = row == first ? a.s0[seq * D + lane] : a.s[(row - 1) * D + lane];
     const real th = tanh(sp);
     const real dth = real(1) - th * th;
-    const real* Wr = a.dv.params + seq * a.dv.pstride + lane * D;
-    real w[D];
-#pragma unroll
-    for (int k = 0; k < D; k += VW) {
-      if constexpr (sizeof(real) == 4) {
-        const float4 q = __ldg(reinterpret_cast<const float4*>(Wr + k));
-        w[k] = q.x; w[k + 1] = q.y; w[k + 2] = q.z; w[k + 3] = q.w;
-      } else {
-        const double2 q = __ldg(reinterpret_cast<const double2*>(Wr + k));
-        w[k] = q.x; w[k + 1] = q.y;
-      }
-    }
     real F = a.dv.x ? __ldg(a.dv.x + row * D + lane) : real(0);
 #pragma unroll
     for (int j = 0; j < D; ++j) F += w[j] * __shfl_sync(gmask, th, j, D);
@@ -114,6 +116,9 @@ __global__ void __launch_bounds__(128) k_lin_rnn_wide(LinArgs<real> a) {
 #pragma unroll
       for (int j = 0; j < D; ++j) Arow[j] = scale * w[j] * __shfl_sync(gmask, dth, j, D);
       store_block_rows<real, D>(sT[grp], a.A + row * (int64_t)(D * D), Arow, lane, gmask);
+      a.b[row * D + lane] = -rr;
+    } else if constexpr (JAC == kJacFactored) {
+      a.A[row * D + lane] = (a.damp == DEER_DAMP_SCALE ? real(1) - k : real(1)) * dth;
       a.b[row * D + lane] = -rr;
     } else {
       real ai;
@@ -151,7 +156,9 @@ template <class real>
 cudaError_t launch_linearize_models(const LinArgs<real>& a, cudaStream_t st) {
   if (a.dv.kind == DEER_F_RNN_TANH && (a.dv.d == 16 || a.dv.d == 32)) {
     switch (a.jac) {
-      case DEER_JAC_FULL: return lin_rnn_wide<real, DEER_JAC_FULL>(a, st);
+      case DEER_JAC_FULL:
+        if (a.factored) return lin_rnn_wide<real, kJacFactored>(a, st);
+        return lin_rnn_wide<real, DEER_JAC_FULL>(a, st);
       case DEER_JAC_DIAG: return lin_rnn_wide<real, DEER_JAC_DIAG>(a, st);
       case DEER_JAC_IDENTITY: return lin_rnn_wide<real, DEER_JAC_IDENTITY>(a, st);
       default: return lin_rnn_wide<real, DEER_JAC_ZERO>(a, st);

@@ -32,6 +32,9 @@ struct LinArgs {
                        // above it are reported (first failing row, for the sliding window)
   const real* slo = nullptr;  // compensation of s ([N][d], the state is s + slo); nullptr =
                               // plain state (mass-action kinetics only)
+  // mean-field RNN, d = 32: write the 32 column factors of A_t = W diag(e_t) to A's rows
+  // ([N][d]) instead of the dense Jacobians (see k_rnn.cu)
+  bool factored = false;
   // mass action, d = 16 / 32: per-species lists of the reactions that change the species
   // (launch_ma_adjacency; entry = r | (nu + 4) << 16), so that each lane walks its own
   // reactions rather than all of them; nullptr = walk every reaction
@@ -477,6 +480,10 @@ struct MixedRcArgs {
 };
 
 cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st);
+// dense scan of the mean-field RNN (d = 32) from the column factors of its Jacobians
+cudaError_t launch_rnn_scan(const DenseScanArgs<float>& a, const DynView<float>& dv,
+                            cudaStream_t st);
+
 // carry pass of the dense scans alone (d = 16, 32), over aggregates formed elsewhere
 cudaError_t launch_dense_carry(const DenseScanArgs<float>& a, cudaStream_t st);
 
