@@ -97,6 +97,25 @@ __device__ __forceinline__ double nu_f64(int nu) {
 constexpr double kMixedFastAbove = 1e-4;
 constexpr float kMixedFloor = 1e-6f;
 
+// A species' reactions in shared memory, lane-contiguous (entry e of species i at e D + i):
+// reaction | (nu + 4) << 6 | first reactant << 10 | (second reactant + 1) << 16. The walk over
+// them gathered both from global memory once per entry, stage and row before.
+constexpr int kMixList = 16;
+
+template <int D>
+__device__ __forceinline__ void mixed_list(uint32_t* lst, int lane, const int4* tt,
+                                           const int32_t* ae, int e0, int e1) {
+  for (int e = 0; e < kMixList && e0 + e < e1; ++e) {
+    const int code = __ldg(ae + e0 + e), r = code & 0xffff;
+    const int4 q = __ldg(tt + r);
+    // (a reaction naming no species changes nothing here; the set-up kernel reports it)
+    const bool ok = q.x >= 0 && q.x < D && q.y >= -1 && q.y < D;
+    lst[e * D + lane] = ok ? (uint32_t)r | (uint32_t)(code >> 16) << 6 | (uint32_t)q.x << 10 |
+                                 (uint32_t)(q.y + 1) << 16
+                           : (uint32_t)r | 4u << 6;
+  }
+}
+
 // One row of the mixed linearisation with the dynamics' value path (stage states, reaction
 // rates, slopes, F, residual) in V = float or double; the Jacobian path is float32 either
 // way. Writes E and b for the row and returns its scaled residual and squared residual.
@@ -119,7 +138,7 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
                                           const int4 (&q)[RPL], const double (&kd)[RPL],
                                           const float (&kf)[RPL], int R, const int4* tt,
                                           const int32_t* ae, int e0, int e1,
-                                          float (*sG)[D + 4], float (*sK)[D + 4], V* sRate,
+                                          const uint32_t* lst, float (*sG)[D + 4], float (*sK)[D + 4], V* sRate,
                                           float* sD1, float* sD2, float& mx, float& sq,
                                           int64_t seq, unsigned long long& key,
                                           __nv_bfloat16* Eo, float* bo,
@@ -141,12 +160,19 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
     // every reaction's rate once (reaction r on lane r mod d) and its two partials
 #pragma unroll
     for (int k = 0; k < RPL; ++k) {
+      if (k * D >= R) break;  // uniform over the group
       const int r = k * D + lane;
       const int j2 = q[k].y < 0 ? 0 : q[k].y;
       const V c1 = __shfl_sync(gm, c, q[k].x, D);
       const V c2 = __shfl_sync(gm, c, j2, D);
-      const float c1f = __shfl_sync(gm, cf, q[k].x, D);
-      const float c2f = __shfl_sync(gm, cf, j2, D);
+      float c1f, c2f;
+      if constexpr (F64) {
+        c1f = __shfl_sync(gm, cf, q[k].x, D);
+        c2f = __shfl_sync(gm, cf, j2, D);
+      } else {
+        c1f = (float)c1;  // the value path's own concentrations
+        c2f = (float)c2;
+      }
       if (r < R) {
         const bool bi = q[k].y >= 0;
         const V kr = F64 ? (V)kd[k] : (V)kf[k];
@@ -161,15 +187,22 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
     __syncwarp(gm);
     // this species' slope and its row of the rate Jacobian, from its own reactions
     V g = V(0);
-    for (int e = e0; e < e1; ++e) {
-      const int code = __ldg(ae + e);
-      const int r = code & 0xffff;
-      const int nu = (code >> 16) - 4;
+    const int n1 = e1 - e0 < kMixList ? e1 - e0 : kMixList;
+    auto entry = [&](int r, int nu, int i1, int i2) {
       g += (F64 ? (V)nu_f64(nu) : (V)nu) * sRate[r];
-      const int4 qq = __ldg(tt + r);
       const float nuf = (float)nu;
-      sG[lane][qq.x] += nuf * sD1[r];
-      if (qq.y >= 0) sG[lane][qq.y] += nuf * sD2[r];
+      sG[lane][i1] += nuf * sD1[r];
+      if (i2 >= 0) sG[lane][i2] += nuf * sD2[r];
+    };
+    for (int e = 0; e < n1; ++e) {
+      const uint32_t w = lst[e * D + lane];
+      entry((int)(w & 63u), (int)((w >> 6) & 15u) - 4, (int)((w >> 10) & 63u),
+            (int)(w >> 16) - 1);
+    }
+    for (int e = e0 + kMixList; e < e1; ++e) {  // the rest of a long list
+      const int code = __ldg(ae + e);
+      const int4 qq = __ldg(tt + (code & 0xffff));
+      entry(code & 0xffff, (code >> 16) - 4, qq.x, qq.y);
     }
     __syncwarp(gm);
     float Gi[D], Kn[D];
@@ -234,6 +267,11 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
   }
 }
 
+// Each group of D lanes walks kMixRows consecutive rows: the network's reactions, rate
+// constants and species lists are loaded once per group and sequence, and the residual
+// statistics flushed once: 3.2 M rows, d = 16, 24 reactions, 9.3 -> 8.8 ms.
+constexpr int kMixRows = 8;
+
 template <int D, bool RK4>
 __global__ void __launch_bounds__(128) k_lin_ma_mixed(MixedLinArgs a) {
   constexpr int GROUPS = 128 / D;
@@ -246,47 +284,63 @@ __global__ void __launch_bounds__(128) k_lin_ma_mixed(MixedLinArgs a) {
   __shared__ __align__(16) float sK[GROUPS][D + 1][D + 4];
   __shared__ double sRate[GROUPS][RMAX];  // float rates use the first half in float32 mode
   __shared__ float sD1[GROUPS][RMAX], sD2[GROUPS][RMAX];  // d rate / d c_i1, d c_i2
+  __shared__ uint32_t sList[GROUPS][kMixList * D];
   const int grp = threadIdx.x / D, lane = threadIdx.x % D;
   const unsigned gm = gmask_mixed<D>();
-  const int64_t ar = blockIdx.x * (int64_t)GROUPS + grp;
-  const bool valid = ar < a.bt.act_rows();
-  int64_t seq = 0, row = 0;
-  if (valid) act_row(a.bt, ar, seq, row);
-  const double s_prev = valid ? (row == __ldg(a.bt.offsets + seq) ? a.s0[seq * D + lane]
-                                                                : a.s[(row - 1) * D + lane])
-                              : 0.0;
-  const double* kk = a.dv.params + seq * a.dv.pstride;
-  const int4* tt = reinterpret_cast<const int4*>(a.dv.topo + seq * a.dv.tstride);
-  const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1);
-  const int32_t* ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
-  const int e0 = __ldg(aoff + lane), e1 = __ldg(aoff + lane + 1);
+  const int64_t ar0 = (blockIdx.x * (int64_t)GROUPS + grp) * kMixRows;
+  const int64_t rows = a.bt.act_rows();
   const int R = a.dv.R < RMAX ? a.dv.R : RMAX;
+  int64_t cur = -1;
+  const int4* tt = nullptr;
+  const int32_t* ae = nullptr;
+  int e0 = 0, e1 = 0;
   int4 q[RPL];
   double kd[RPL];
   float kf[RPL];
-#pragma unroll
-  for (int k = 0; k < RPL; ++k) {
-    const int r = k * D + lane;
-    q[k] = __ldg(tt + (r < R ? r : 0));
-    kd[k] = r < R ? __ldg(kk + r) : 0.0;
-    kf[k] = d2f_trunc(kd[k]);
-  }
-  const bool fast = !valid || a.it == 0 || a.info[seq].max_resid > kMixedFastAbove;
+  bool fast = true;
   float mx = 0.f, sq = 0.f;
   unsigned long long key = 0ull;  // first failing row (sliding window)
-  const double sc = valid ? a.s[row * D + lane] : 0.0;
-  __nv_bfloat16* Eo = a.E + (valid ? row : 0) * (int64_t)(D * D);
-  float* bo = a.b + (valid ? row : 0) * D;
-  if (fast)
-    mixed_row<float, D, RK4, RPL>(a, valid, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
-                                  e0, e1, sG[grp], sK[grp],
-                                  reinterpret_cast<float*>(sRate[grp]), sD1[grp], sD2[grp],
-                                  mx, sq, seq, key, Eo, bo);
-  else
-    mixed_row<double, D, RK4, RPL>(a, valid, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
-                                   e0, e1, sG[grp], sK[grp], sRate[grp], sD1[grp], sD2[grp],
-                                   mx, sq, seq, key, Eo, bo);
-  acc_resid_f(a.acc, seq, valid, mx, sq, key);
+  for (int ri = 0; ri < kMixRows && ar0 + ri < rows; ++ri) {  // uniform over the group
+    int64_t seq, row;
+    act_row(a.bt, ar0 + ri, seq, row);
+    if (seq != cur) {
+      if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
+      cur = seq;
+      mx = 0.f;
+      sq = 0.f;
+      key = 0ull;
+      const double* kk = a.dv.params + seq * a.dv.pstride;
+      tt = reinterpret_cast<const int4*>(a.dv.topo + seq * a.dv.tstride);
+      const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1);
+      ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
+      e0 = __ldg(aoff + lane);
+      e1 = __ldg(aoff + lane + 1);
+      mixed_list<D>(sList[grp], lane, tt, ae, e0, e1);
+#pragma unroll
+      for (int k = 0; k < RPL; ++k) {
+        const int r = k * D + lane;
+        q[k] = __ldg(tt + (r < R ? r : 0));
+        kd[k] = r < R ? __ldg(kk + r) : 0.0;
+        kf[k] = d2f_trunc(kd[k]);
+      }
+      fast = a.it == 0 || a.info[seq].max_resid > kMixedFastAbove;
+    }
+    const double s_prev = row == __ldg(a.bt.offsets + seq) ? a.s0[seq * D + lane]
+                                                          : a.s[(row - 1) * D + lane];
+    const double sc = a.s[row * D + lane];
+    __nv_bfloat16* Eo = a.E + row * (int64_t)(D * D);
+    float* bo = a.b + row * D;
+    if (fast)
+      mixed_row<float, D, RK4, RPL>(a, true, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
+                                    e0, e1, sList[grp], sG[grp], sK[grp],
+                                    reinterpret_cast<float*>(sRate[grp]), sD1[grp], sD2[grp],
+                                    mx, sq, seq, key, Eo, bo);
+    else
+      mixed_row<double, D, RK4, RPL>(a, true, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
+                                     e0, e1, sList[grp], sG[grp], sK[grp], sRate[grp],
+                                     sD1[grp], sD2[grp], mx, sq, seq, key, Eo, bo);
+  }
+  if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
 }
 
 // ---- mixed dense scan: lane j owns column j of P and entry j of the vectors ----------
@@ -519,6 +573,7 @@ struct RcSmem {
   float d1[2][kRcRmax], d2[2][kRcRmax];
   float E[2][16 * kRcES];
   float b[2][16];
+  uint32_t list[kMixList * 16];
   double old[16];  // pass 2: old state of the previous pair's second row
 };
 
@@ -561,12 +616,12 @@ __device__ __forceinline__ void rc_row(const MixedLinArgs& a, bool fast, bool va
   if (fast)
     mixed_row<float, 16, RK4, kRcRmax / 16>(
         a, valid, row, lane, gm, sp, sc, n.q, n.kd, n.kf, n.R, n.tt, n.ae, n.e0, n.e1,
-        S.G[half], S.K[half], reinterpret_cast<float*>(S.rate[half]), S.d1[half],
+        S.list, S.G[half], S.K[half], reinterpret_cast<float*>(S.rate[half]), S.d1[half],
         S.d2[half], mx, sq, seq, key, nullptr, S.b[half], S.E[half]);
   else
     mixed_row<double, 16, RK4, kRcRmax / 16>(
         a, valid, row, lane, gm, sp, sc, n.q, n.kd, n.kf, n.R, n.tt, n.ae, n.e0, n.e1,
-        S.G[half], S.K[half], S.rate[half], S.d1[half], S.d2[half], mx, sq, seq, key,
+        S.list, S.G[half], S.K[half], S.rate[half], S.d1[half], S.d2[half], mx, sq, seq, key,
         nullptr, S.b[half], S.E[half]);
 }
 
@@ -639,6 +694,8 @@ __global__ void __launch_bounds__(32 * kRcWarps) k_mixed_lin_agg16(MixedRcArgs r
   const int64_t base = __ldg(a.bt.offsets + seq);
   RcNet net;
   rc_net(a, seq, lane, net);
+  if (half == 0) mixed_list<16>(S.list, lane, net.tt, net.ae, net.e0, net.e1);
+  __syncwarp();
   const bool fast = a.it == 0 || a.info[seq].max_resid > kMixedFastAbove;
   if (l32 == 0) r.fastsel[seq] = fast ? 1 : 0;  // the same value from every chunk
   // the old state before the chunk, kept for the second pass (whose neighbouring chunk may
@@ -703,6 +760,8 @@ __global__ void __launch_bounds__(32 * kRcWarps) k_mixed_apply_rc16(MixedRcArgs 
   const int64_t base = __ldg(a.bt.offsets + seq);
   RcNet net;
   rc_net(a, seq, lane, net);
+  if (half == 0) mixed_list<16>(S.list, lane, net.tt, net.ae, net.e0, net.e1);
+  __syncwarp();
   const bool fast = r.fastsel[seq] != 0;
   const double prev0 = r0 == base ? a.s0[seq * 16 + lane] : r.sbound[c * 16 + lane];
   float x = r.cin[c * 16 + lane];  // Delta entering the chunk, entry lane mod 16
@@ -762,7 +821,7 @@ cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
   const bool rk4 = a.dv.kind == DEER_F_MASSACTION_RK4;
   const int d = a.dv.d;
-  const unsigned g = grid_for(a.bt.act_rows(), 128 / d);
+  const unsigned g = grid_for(a.bt.act_rows(), 128 / d * kMixRows);
   if (d == 16) {
     if (rk4) k_lin_ma_mixed<16, true><<<g, 128, 0, st>>>(a);
     else k_lin_ma_mixed<16, false><<<g, 128, 0, st>>>(a);
