@@ -11,9 +11,11 @@ path a host-side caller uses); CUDA tensors are used in place.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 from dataclasses import dataclass
 from typing import Optional
 
+import numpy as np
 import torch
 
 from . import _native as N
@@ -122,6 +124,27 @@ class SolveInfo:
     max_resid: torch.Tensor   # [B] float64
 
 
+_INFO_DTYPE = np.dtype([("iters", "<i4"), ("converged", "<i4"), ("merit", "<f8"),
+                        ("max_resid", "<f8")])
+
+
+def _solve_info(status: int, infos, B: int) -> SolveInfo:
+    """The library's per-sequence records as tensors, column by column (reading them field by
+    field through ctypes took 5 ms for 4096 sequences)."""
+    a = np.frombuffer(infos, dtype=_INFO_DTYPE, count=B)
+    return SolveInfo(
+        status=status,
+        iters=torch.from_numpy(a["iters"].copy()),
+        converged=torch.from_numpy(a["converged"] != 0),
+        merit=torch.from_numpy(a["merit"].copy()),
+        max_resid=torch.from_numpy(a["max_resid"].copy()))
+
+
+@functools.lru_cache(maxsize=None)
+def _gpu_name(index: int) -> str:
+    return torch.cuda.get_device_name(index)
+
+
 def _check_dev(t: torch.Tensor, name: str):
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
@@ -213,7 +236,8 @@ def _run_solve(dyn, B, T, offsets, s0, x, s_init, opts, stream, workspace, devic
     Tmax = T if offsets is None else max(
         (int(offsets[i + 1]) - int(offsets[i]) for i in range(B)), default=0)
     tuned = autotune.cached_options(dyn, Tmax, opts["jac"], opts["prec"],
-                                    gpu=torch.cuda.get_device_name(device))
+                                    gpu=_gpu_name(torch.cuda.current_device()
+                                                  if device.index is None else device.index))
     if tuned:
         upd = {k: v for k, v in tuned.items()
                if (k == "chunk" and int(opts.get("chunk", 0)) == 0)
@@ -251,12 +275,7 @@ def _run_solve(dyn, B, T, offsets, s0, x, s_init, opts, stream, workspace, devic
                                     C.byref(o), _ptr(workspace), workspace.numel(), sh, infos)
     if st not in (N.DEER_OK, N.DEER_NOT_CONVERGED):
         raise N.DeerError(st, "deer_solve")
-    info = SolveInfo(
-        status=st,
-        iters=torch.tensor([infos[i].iters for i in range(B)], dtype=torch.int32),
-        converged=torch.tensor([bool(infos[i].converged) for i in range(B)]),
-        merit=torch.tensor([infos[i].merit for i in range(B)], dtype=torch.float64),
-        max_resid=torch.tensor([infos[i].max_resid for i in range(B)], dtype=torch.float64))
+    info = _solve_info(st, infos, B)
     return s, info
 
 

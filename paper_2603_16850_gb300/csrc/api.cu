@@ -429,11 +429,8 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
   SeqAcc* acc = reinterpret_cast<SeqAcc*>(ws + ly.acc);
   SeqInfo* info = reinterpret_cast<SeqInfo*>(ws + ly.info);
   Flags* flags = reinterpret_cast<Flags*>(ws + ly.flags);
-  if (B > 0) {
-    DEER_CK(cudaMemsetAsync(acc, 0, B * sizeof(SeqAcc), st));
-    DEER_CK(cudaMemsetAsync(info, 0, B * sizeof(SeqInfo), st));
-  }
-  DEER_CK(cudaMemsetAsync(flags, 0, sizeof(Flags), st));
+  // accumulators, per-sequence records and status word lie one after the other
+  DEER_CK(cudaMemsetAsync(acc, 0, ly.flags + sizeof(Flags) - ly.acc, st));
 
   Batch bt;
   bt.B = B;
@@ -720,6 +717,7 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
 
   deer_status status = DEER_OK;
   Flags hf;
+  std::vector<char> host_info;  // the records, where they have been read already
   PhaseTimer pt(st);
 
   // The steps of one iteration, shared by the host-driven loop and the graph of the
@@ -813,17 +811,18 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
                            !mixed && !ly.cs && !o->history && maxT >= 1 &&
                            maxT <= block_solve_max_T(f->kind, d) && B <= INT32_MAX;
   if (block_solve) {
-    // the initial active-set pass counted every sequence; the block solve counts the
-    // unconverged ones itself
-    DEER_CK(cudaMemsetAsync(&flags->n_active, 0, sizeof(int32_t), st));
     BlockSolveArgs<real> ba{dv, B, maxT, d_off, s0, s, info, flags, o->tol, max_iters,
                             o->confirm > 1 ? o->confirm : 1, o->reset, o->damp,
                             (real)o->damp_param, reset_thr};
     pt.begin(PH_LIN);  // the whole loop is one launch: its time goes to linearisation
     DEER_CK(launch_block_solve<real>(ba, st));
     pt.end(PH_LIN);
-    DEER_CK(cudaMemcpyAsync(&hf, flags, sizeof(Flags), cudaMemcpyDeviceToHost, st));
+    // the records and the status word lie one after the other: one copy brings both
+    host_info.resize(ly.flags + sizeof(Flags) - ly.info);
+    DEER_CK(cudaMemcpyAsync(host_info.data(), info, host_info.size(), cudaMemcpyDeviceToHost,
+                            st));
     DEER_CK(cudaStreamSynchronize(st));
+    std::memcpy(&hf, host_info.data() + (ly.flags - ly.info), sizeof(Flags));
     if (pt.on) {
       const int64_t launches[PH_N] = {0, 1, 0, 0};
       const int64_t rows[PH_N] = {0, N, 0, 0};
@@ -978,15 +977,19 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
 
   if (info_h && B > 0) {
     std::vector<SeqInfo> hi(B);
-    DEER_CK(cudaMemcpyAsync(hi.data(), info, B * sizeof(SeqInfo), cudaMemcpyDeviceToHost, st));
-    DEER_CK(cudaStreamSynchronize(st));
+    if (!host_info.empty()) {
+      std::memcpy(hi.data(), host_info.data(), B * sizeof(SeqInfo));
+    } else {
+      DEER_CK(cudaMemcpyAsync(hi.data(), info, B * sizeof(SeqInfo), cudaMemcpyDeviceToHost, st));
+      DEER_CK(cudaStreamSynchronize(st));
+    }
     for (int64_t b = 0; b < B; ++b) {
       info_h[b].iters = hi[b].iters;
       info_h[b].converged = hi[b].done;
       info_h[b].merit = hi[b].merit;
       info_h[b].max_resid = hi[b].max_resid;
     }
-  } else {
+  } else if (host_info.empty()) {
     DEER_CK(cudaStreamSynchronize(st));
   }
   return status;

@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
     inf.max_resid = bm;
     a.info[seq] = inf;
     if (nonfinite) atomicAdd(&a.flags->n_nonfinite, 1);
-    if (!done) atomicAdd(&a.flags->n_active, 1);
+    if (done) atomicSub(&a.flags->n_active, 1);  // the active-set pass counted every sequence
   }
   cl.sync();  // no block leaves while another may still read its shared memory
 }
@@ -475,10 +475,20 @@ static cudaError_t block_launch(const BlockSolveArgs<real>& a, cudaStream_t st) 
     // a cluster of 16 that cannot be placed: take 8 instead (the longest sequence taken
     // fits 8)
     if (cl > kMaxCluster) {
-      int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess ||
-          nclusters < 1) {
+      // (asked once per host thread, device and cluster size: the query takes longer than the
+      // launch)
+      static thread_local signed char placed[16][kWideCluster + 1] = {};
+      int dev = 0;
+      cudaGetDevice(&dev);
+      signed char unknown = 0;
+      signed char& fits = dev < 16 ? placed[dev][cl] : unknown;
+      if (fits == 0) {
+        int nclusters = 0;
+        fits = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) == cudaSuccess &&
+                       nclusters >= 1 ? 1 : -1;
         (void)cudaGetLastError();
+      }
+      if (fits < 0) {
         cl = kMaxCluster;
         continue;
       }
