@@ -116,9 +116,6 @@ __device__ __forceinline__ void mixed_list(uint32_t* lst, int lane, const int4* 
   }
 }
 
-// One row of the mixed linearisation with the dynamics' value path (stage states, reaction
-// rates, slopes, F, residual) in V = float or double; the Jacobian path is float32 either
-// way. Writes E and b for the row and returns its scaled residual and squared residual.
 // A row of D floats from shared memory in 16-byte pieces (16-byte aligned).
 template <int D>
 __device__ __forceinline__ void ld_row4(const float* p, float (&v)[D]) {
@@ -129,20 +126,24 @@ __device__ __forceinline__ void ld_row4(const float* p, float (&v)[D]) {
   }
 }
 
-// The row's outputs go to Eo (its D x D block of E, row-major bf16) and bo (its entry
-// of b = -r): in global memory for the materialised path, in shared memory for the
-// recomputing one. sc is the row's own state s_t (read by the caller).
+// One row of the mixed linearisation with the dynamics' value path (stage states, reaction
+// rates, slopes, F, residual) in V = float or double; the Jacobian path is float32 either
+// way. Writes E and b for the row and returns its scaled residual and squared residual.
+//
+// A lane per species: the recomputing path's form. The row's outputs go to Eo (its D x D
+// block of E) and bo (its entry of b = -r) in shared memory. sc is the row's own state s_t
+// (read by the caller).
 template <class V, int D, bool RK4, int RPL>
 __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int64_t row,
                                           int lane, unsigned gm, double s_prev_d, double sc,
                                           const int4 (&q)[RPL], const double (&kd)[RPL],
                                           const float (&kf)[RPL], int R, const int4* tt,
                                           const int32_t* ae, int e0, int e1,
-                                          const uint32_t* lst, float (*sG)[D + 4], float (*sK)[D + 4], V* sRate,
-                                          float* sD1, float* sD2, float& mx, float& sq,
+                                          const uint32_t* lst, float (*sG)[D + 4],
+                                          float (*sK)[D + 4], V* sRate, float* sD1,
+                                          float* sD2, float& mx, float& sq,
                                           int64_t seq, unsigned long long& key,
-                                          __nv_bfloat16* Eo, float* bo,
-                                          float* Eo32 = nullptr) {
+                                          float* bo, float* Eo) {
   constexpr bool F64 = sizeof(V) == 8;
   const V s_prev = F64 ? (V)s_prev_d : (V)d2f_trunc(s_prev_d);
   const V h = F64 ? (V)a.dv.dt : (V)a.dt_f;
@@ -243,104 +244,407 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
     if (!(m <= a.tol_f) && key == 0ull) key = bad_key(true, row - __ldg(a.bt.offsets + seq));
     const float scale = a.scale_f;
     const float hwf = RK4 ? hf / 6.f : hf;
-    // E = A - I with A = I + hw Kacc (scaled by (1 - k) under scale-ELK: E = s A - I):
-    // bf16 row-major, or float32 with rows padded to 20 (the recomputing path)
-    if (Eo32) {
-      float* Er = Eo32 + lane * 20;
+    // E = A - I with A = I + hw Kacc (scaled by (1 - k) under scale-ELK: E = s A - I),
+    // float32 with rows padded to 20
+    float* Er = Eo + lane * 20;
 #pragma unroll
-      for (int j = 0; j < D; j += 4)
-        *reinterpret_cast<float4*>(Er + j) =
-            make_float4(scale * hwf * Kacc[j] + (j == lane ? scale - 1.f : 0.f),
-                        scale * hwf * Kacc[j + 1] + (j + 1 == lane ? scale - 1.f : 0.f),
-                        scale * hwf * Kacc[j + 2] + (j + 2 == lane ? scale - 1.f : 0.f),
-                        scale * hwf * Kacc[j + 3] + (j + 3 == lane ? scale - 1.f : 0.f));
-    } else {
-      Eo += lane * D;
-#pragma unroll
-      for (int j = 0; j < D; j += 2) {
-        const float x0 = scale * hwf * Kacc[j] + (j == lane ? scale - 1.f : 0.f);
-        const float x1 = scale * hwf * Kacc[j + 1] + (j + 1 == lane ? scale - 1.f : 0.f);
-        *reinterpret_cast<__nv_bfloat162*>(Eo + j) = __floats2bfloat162_rn(x0, x1);
-      }
-    }
+    for (int j = 0; j < D; j += 4)
+      *reinterpret_cast<float4*>(Er + j) =
+          make_float4(scale * hwf * Kacc[j] + (j == lane ? scale - 1.f : 0.f),
+                      scale * hwf * Kacc[j + 1] + (j + 1 == lane ? scale - 1.f : 0.f),
+                      scale * hwf * Kacc[j + 2] + (j + 2 == lane ? scale - 1.f : 0.f),
+                      scale * hwf * Kacc[j + 3] + (j + 3 == lane ? scale - 1.f : 0.f));
     bo[lane] = -rf;
   }
 }
 
-// Each group of D lanes walks kMixRows consecutive rows: the network's reactions, rate
-// constants and species lists are loaded once per group and sequence, and the residual
-// statistics flushed once: 3.2 M rows, d = 16, 24 reactions, 9.3 -> 8.8 ms.
-constexpr int kMixRows = 8;
+// ---- linearisation: two columns per lane ------------------------------------------------
+// D / 2 lanes share a row: each forms the rate-Jacobian rows of its two species, then takes
+// its two columns of every stage Jacobian K_j = G_j (I + c_j K_{j-1}) with both factors of a
+// column at hand: K_{j-1}'s columns in registers, G's rows broadcast from shared memory, so
+// the products are two-wide FMAs and K is never exchanged. What bounds it is shared-memory
+// wavefronts. With a lane per species (row i of K, K_{j-1} broadcast) 94 % of their rate was
+// in use, the FMA pipe at 17 %: half of them the scatter of every reaction's partials into G
+// (zero, add in place, read back), half the K rows. Here G's entries are sums of products
+// coefficient x concentration, listed once per sequence in the order of their entries, so
+// that each is summed in a register and stored once; entries that no term names stay zero.
+// Sums keep the reactions' order and the products round alike (nu is a power of two up to
+// sign), so the results are those of the scatter. 3.2 M rows, d = 16, 24 reactions:
+// 8.8 -> 6.1 ms, evaluated in float64 9.7 -> 8.6 (then the float64 pipe counts too). Tried and
+// slower: the products as tf32 MMAs with the three-term split (fewer reads of G, but the splits
+// cost more instructions: 7.6 ms), and more rows per warp (128: partly filled last rounds).
+//
+// A warp walks kMixRows consecutive rows, 32 / (D / 2) at a time, all of one sequence, so that
+// it holds one network: lists and rate constants are built once per warp and sequence, and the
+// residual statistics flushed once.
+constexpr int kMixRows = 32;
+constexpr int kMixTerms = 2 * kMixList;  // entries of G named by a species' listed reactions
+constexpr int kMixReact = 64;            // reactions per network (the host checks)
+constexpr int kMixBatch = 4;             // list entries whose loads are issued together
+static_assert(kMixList % kMixBatch == 0, "lists are filled up to whole batches");
+
+template <int D>
+struct MixNet {  // one per warp
+  // term e of species i: coefficient, byte offset in G | last of its entry | byte offset of the
+  // source concentration << 16
+  uint2 term[kMixTerms][D];
+  uint32_t run[kMixList][D];   // reaction e of species i: change (float bits) | reaction
+  uint32_t react[kMixReact];   // first reactant | second << 8 (D, whose concentration is 1)
+  double kd[kMixReact];
+  float kf[kMixReact];
+};
+
+template <int D>
+struct MixRow {  // one per row in flight
+  float G[D * (D + 4) + 4];
+  float c[D + 4];   // c[D] = 1
+  double cd[D + 2];
+  double rate[kMixReact + 2];  // [kMixReact] = 0; floats in float32 mode
+  float pad[D == 16 ? 8 : 4];  // the rows of a warp in different banks
+};
+
+__device__ __forceinline__ float mix_nu(uint32_t w, float) {
+  return __uint_as_float(w & 0xffffff80u);
+}
+__device__ __forceinline__ double mix_nu(uint32_t w, double) {  // +-1 or +-2 (or next to 0)
+  return __hiloint2double(
+      (int)((w & 0x80000000u) | (((w >> 3) & 0x0ff00000u) + 0x38000000u)), 0);
+}
+
+// The sequence's lists, by the whole warp, and the lengths of the longest: most_t entries of G
+// and most_g reactions of a species (shorter lists are filled up with entries of no effect).
+template <int D>
+__device__ __forceinline__ void mix_net(const MixedLinArgs& a, int64_t seq, int R, int l32,
+                                        MixNet<D>& W, int& most_t, int& most_g) {
+  constexpr int RS = D + 4;
+  const double* kk = a.dv.params + seq * a.dv.pstride;
+  const int4* tt = reinterpret_cast<const int4*>(a.dv.topo + seq * a.dv.tstride);
+  const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1);
+  const int32_t* ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
+  int nt = 0, ng = 0;
+  if (l32 < D) {
+    const int e0 = __ldg(aoff + l32), e1 = __ldg(aoff + l32 + 1);
+    auto put = [&](float k, int j, int m) {  // stable insertion by the place in G
+      const uint32_t at = 4u * (uint32_t)(l32 * RS + j);
+      int e = nt++;
+      for (; e > 0 && (W.term[e - 1][l32].y & 0xffffu) > at; --e)
+        W.term[e][l32] = W.term[e - 1][l32];
+      W.term[e][l32] = make_uint2(__float_as_uint(k), at | (uint32_t)m << 18);
+    };
+    for (; ng < kMixList && e0 + ng < e1; ++ng) {
+      const int code = __ldg(ae + e0 + ng), r = code & 0xffff;
+      const int4 q = __ldg(tt + r);
+      // (a reaction naming no species changes nothing here; the set-up kernel reports it)
+      const bool ok = q.x >= 0 && q.x < D && q.y >= -1 && q.y < D;
+      const float nu = ok ? (float)((code >> 16) - 4) : 0.f;
+      W.run[ng][l32] = __float_as_uint(nu) | (uint32_t)(r < kMixReact ? r : kMixReact);
+      if (ok) {
+        const float k = nu * d2f_trunc(__ldg(kk + r));
+        put(k, q.x, q.y < 0 ? D : q.y);      // d rate / d c_i1
+        if (q.y >= 0) put(k, q.y, q.x);      // d rate / d c_i2
+      }
+    }
+    for (int e = 0; e < nt; ++e)
+      if (e + 1 == nt || (W.term[e + 1][l32].y & 0xffffu) != (W.term[e][l32].y & 0xffffu))
+        W.term[e][l32].y |= 1u;
+  }
+  // (whole batches of kMixBatch)
+  most_t = (__reduce_max_sync(0xffffffffu, nt) + kMixBatch - 1) / kMixBatch * kMixBatch;
+  most_g = (__reduce_max_sync(0xffffffffu, ng) + kMixBatch - 1) / kMixBatch * kMixBatch;
+  if (l32 < D) {
+    for (int e = nt; e < most_t; ++e) W.term[e][l32] = make_uint2(0u, (uint32_t)D << 18);
+    for (int e = ng; e < most_g; ++e) W.run[e][l32] = (uint32_t)kMixReact;
+  }
+  for (int r = l32; r < R; r += 32) {
+    const int4 q = __ldg(tt + r);
+    const double k = __ldg(kk + r);
+    W.react[r] = (q.x >= 0 && q.x < D ? (uint32_t)q.x : (uint32_t)D) |
+                 (q.y >= 0 && q.y < D ? (uint32_t)q.y : (uint32_t)D) << 8;
+    W.kd[r] = k;
+    W.kf[r] = d2f_trunc(k);
+  }
+}
+
+// One row, with the dynamics' value path in V = float or double (see mixed_row). `tail`: some
+// species of the network has reactions beyond its list.
+template <class V, int D, bool RK4>
+__device__ __forceinline__ void mixed_row_cols(const MixedLinArgs& a, bool valid, int64_t seq,
+                                               int64_t row, int lane, const MixNet<D>& W,
+                                               MixRow<D>& S, int R, int most_t, int most_g,
+                                               bool tail, const double (&spd)[2],
+                                               const double (&sc)[2], float& mx, float& sq,
+                                               unsigned long long& key) {
+  constexpr bool F64 = sizeof(V) == 8;
+  constexpr int LPR = D / 2, RS = D + 4;  // G's rows padded by 16 bytes
+  V* rate = reinterpret_cast<V*>(S.rate);
+  const V h = F64 ? (V)a.dv.dt : (V)a.dt_f;
+  const float hf = a.dt_f;
+  V prev[2], c[2], acc[2];
+  float2 K[D], Kacc[D];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    prev[x] = F64 ? (V)spd[x] : (V)d2f_trunc(spd[x]);
+    c[x] = prev[x];
+    acc[x] = V(0);
+  }
+#pragma unroll
+  for (int i = 0; i < D; ++i) Kacc[i] = make_float2(0.f, 0.f);
+  constexpr int NST = RK4 ? 4 : 1;
+#pragma unroll 1
+  for (int stage = 0; stage < NST; ++stage) {
+    // RK4 tableau: stage derivative weights (1, 2, 2, 1), stage offsets (h/2, h/2, h)
+    const float cK = stage == 3 ? hf : 0.5f * hf;
+    const V w = (stage == 1 || stage == 2) ? V(2) : V(1);
+    const float wf = (stage == 1 || stage == 2) ? 2.f : 1.f;
+    if constexpr (F64) {
+      *reinterpret_cast<float2*>(&S.c[2 * lane]) =
+          make_float2(d2f_trunc((double)c[0]), d2f_trunc((double)c[1]));
+      *reinterpret_cast<double2*>(&S.cd[2 * lane]) = make_double2((double)c[0], (double)c[1]);
+    } else {
+      *reinterpret_cast<float2*>(&S.c[2 * lane]) = make_float2((float)c[0], (float)c[1]);
+    }
+    if (tail) {  // entries that only unlisted reactions name
+      for (int j = 0; j < RS / 2; ++j)
+        *reinterpret_cast<float4*>(&S.G[2 * lane * RS + 4 * j]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncwarp();
+    // (loads of a batch first: the stores between them could alias)
+    for (int r0 = lane; r0 < R; r0 += 4 * LPR) {
+      V v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u * LPR < R ? r0 + u * LPR : lane;
+        const uint32_t q = W.react[r];
+        if constexpr (F64) v[u] = W.kd[r] * S.cd[q & 0xffu] * S.cd[q >> 8];
+        else v[u] = W.kf[r] * S.c[q & 0xffu] * S.c[q >> 8];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u * LPR < R) rate[r0 + u * LPR] = v[u];
+    }
+    char* Gb = reinterpret_cast<char*>(S.G);
+    const char* cb = reinterpret_cast<const char*>(S.c);
+    float ga = 0.f, gb = 0.f;
+    for (int e = 0; e < most_t; e += kMixBatch) {
+      uint4 q[kMixBatch];
+      float va[kMixBatch], vb[kMixBatch];
+#pragma unroll
+      for (int u = 0; u < kMixBatch; ++u)
+        q[u] = *reinterpret_cast<const uint4*>(&W.term[e + u][2 * lane]);
+#pragma unroll
+      for (int u = 0; u < kMixBatch; ++u) {
+        va[u] = __fmul_rn(__uint_as_float(q[u].x),
+                          *reinterpret_cast<const float*>(cb + (q[u].y >> 16)));
+        vb[u] = __fmul_rn(__uint_as_float(q[u].z),
+                          *reinterpret_cast<const float*>(cb + (q[u].w >> 16)));
+      }
+#pragma unroll
+      for (int u = 0; u < kMixBatch; ++u) {
+        ga = __fadd_rn(ga, va[u]);
+        gb = __fadd_rn(gb, vb[u]);
+        if (q[u].y & 1u) *reinterpret_cast<float*>(Gb + (q[u].y & 0xfffcu)) = ga;
+        if (q[u].w & 1u) *reinterpret_cast<float*>(Gb + (q[u].w & 0xfffcu)) = gb;
+        ga = q[u].y & 1u ? 0.f : ga;
+        gb = q[u].w & 1u ? 0.f : gb;
+      }
+    }
+    __syncwarp();  // the rates
+    V g[2] = {V(0), V(0)};
+    for (int e = 0; e < most_g; e += kMixBatch) {
+      uint2 q[kMixBatch];
+      V ra[kMixBatch], rb[kMixBatch];
+#pragma unroll
+      for (int u = 0; u < kMixBatch; ++u) {
+        q[u] = *reinterpret_cast<const uint2*>(&W.run[e + u][2 * lane]);
+        ra[u] = rate[q[u].x & 0x7fu];
+        rb[u] = rate[q[u].y & 0x7fu];
+      }
+#pragma unroll
+      for (int u = 0; u < kMixBatch; ++u) {
+        g[0] += mix_nu(q[u].x, V(0)) * ra[u];
+        g[1] += mix_nu(q[u].y, V(0)) * rb[u];
+      }
+    }
+    if (tail) {
+      const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1) + 2 * lane;
+      const int32_t* ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        float* Gi = &S.G[(2 * lane + x) * RS];
+        V gx = g[x];
+        const int e1 = __ldg(aoff + x + 1);
+        for (int e = __ldg(aoff + x) + kMixList; e < e1; ++e) {
+          const int code = __ldg(ae + e), r = code & 0xffff;
+          if (r >= R) continue;
+          const uint32_t q = W.react[r];
+          const float nu = (float)((code >> 16) - 4);
+          const uint32_t i1 = q & 0xffu, i2 = q >> 8;
+          gx += mix_nu(__float_as_uint(nu), V(0)) * rate[r];
+          if (i1 < D) Gi[i1] += nu * (W.kf[r] * S.c[i2]);
+          if (i2 < D) Gi[i2] += nu * (W.kf[r] * S.c[i1]);
+        }
+        g[x] = gx;
+      }
+      __syncwarp();
+    }
+    if (stage == 0) {
+#pragma unroll
+      for (int i = 0; i < D; ++i) K[i] = *reinterpret_cast<const float2*>(&S.G[i * RS + 2 * lane]);
+    } else {
+      float2 Y[D];
+      const float2 cK2 = make_float2(cK, cK);
+      constexpr int IB = 4;  // rows in flight: independent chains for the FMA latency
+#pragma unroll
+      for (int i = 0; i < D; i += IB) {
+#pragma unroll
+        for (int x = 0; x < IB; ++x)
+          Y[i + x] = *reinterpret_cast<const float2*>(&S.G[(i + x) * RS + 2 * lane]);
+#pragma unroll
+        for (int m = 0; m < D; m += 4) {
+          float2 q0[IB], q1[IB];
+#pragma unroll
+          for (int x = 0; x < IB; ++x) {
+            const float4 q = *reinterpret_cast<const float4*>(&S.G[(i + x) * RS + m]);
+            q0[x] = __fmul2_rn(make_float2(q.x, q.y), cK2);
+            q1[x] = __fmul2_rn(make_float2(q.z, q.w), cK2);
+          }
+#pragma unroll
+          for (int x = 0; x < IB; ++x)
+            Y[i + x] = __ffma2_rn(make_float2(q0[x].x, q0[x].x), K[m], Y[i + x]);
+#pragma unroll
+          for (int x = 0; x < IB; ++x)
+            Y[i + x] = __ffma2_rn(make_float2(q0[x].y, q0[x].y), K[m + 1], Y[i + x]);
+#pragma unroll
+          for (int x = 0; x < IB; ++x)
+            Y[i + x] = __ffma2_rn(make_float2(q1[x].x, q1[x].x), K[m + 2], Y[i + x]);
+#pragma unroll
+          for (int x = 0; x < IB; ++x)
+            Y[i + x] = __ffma2_rn(make_float2(q1[x].y, q1[x].y), K[m + 3], Y[i + x]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < D; ++i) K[i] = Y[i];
+    }
+    const V cs = stage == 2 ? h : V(0.5) * h;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      acc[x] += w * g[x];
+      c[x] = prev[x] + cs * g[x];
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) Kacc[i] = __ffma2_rn(make_float2(wf, wf), K[i], Kacc[i]);
+    __syncwarp();  // the next stage or row overwrites G, the rates and the concentrations
+  }
+  if (!valid) return;
+  const V hw = RK4 ? h / V(6) : h;
+  float rf[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const V F = prev[x] + hw * acc[x];
+    const float scf = d2f_trunc(sc[x]);
+    if constexpr (F64) rf[x] = d2f_trunc(sc[x] - (double)F);
+    else rf[x] = scf - (float)F;
+    const float sabs = fabsf(scf);
+    float m = fabsf(rf[x]) / (sabs > 1.f ? sabs : 1.f);
+    if (!F64 && !(m != m)) m = m > kMixedFloor ? m : kMixedFloor;
+    mx = nanmaxf(mx, m);
+    sq += rf[x] * rf[x];
+    if (!(m <= a.tol_f) && key == 0ull) key = bad_key(true, row - __ldg(a.bt.offsets + seq));
+  }
+  const float scale = a.scale_f;
+  const float hwf = RK4 ? hf / 6.f : hf;
+  // E = A - I with A = I + hw Kacc (scaled by (1 - k) under scale-ELK: E = s A - I)
+  __nv_bfloat16* Eo = a.E + row * (int64_t)(D * D) + 2 * lane;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const float x0 = scale * hwf * Kacc[i].x + (i == 2 * lane ? scale - 1.f : 0.f);
+    const float x1 = scale * hwf * Kacc[i].y + (i == 2 * lane + 1 ? scale - 1.f : 0.f);
+    *reinterpret_cast<__nv_bfloat162*>(Eo + i * D) = __floats2bfloat162_rn(x0, x1);
+  }
+  *reinterpret_cast<float2*>(a.b + row * D + 2 * lane) = make_float2(-rf[0], -rf[1]);
+}
+
+template <int D>
+constexpr size_t kMixSmem = 4 * sizeof(MixNet<D>) + 256 / D * sizeof(MixRow<D>);
 
 template <int D, bool RK4>
-__global__ void __launch_bounds__(128) k_lin_ma_mixed(MixedLinArgs a) {
-  constexpr int GROUPS = 128 / D;
-  constexpr int RMAX = 64;         // reactions per network held in shared memory
-  constexpr int RPL = RMAX / D;    // reactions per lane
-  // rows padded to D + 4 floats: 16-byte row accesses of eight lanes fall in distinct
-  // banks; one padding row per group of sK: the two groups of a warp read their (common)
-  // K rows from banks 20 apart (same-bank reads of different groups would serialise)
-  __shared__ __align__(16) float sG[GROUPS][D][D + 4];
-  __shared__ __align__(16) float sK[GROUPS][D + 1][D + 4];
-  __shared__ double sRate[GROUPS][RMAX];  // float rates use the first half in float32 mode
-  __shared__ float sD1[GROUPS][RMAX], sD2[GROUPS][RMAX];  // d rate / d c_i1, d c_i2
-  __shared__ uint32_t sList[GROUPS][kMixList * D];
-  const int grp = threadIdx.x / D, lane = threadIdx.x % D;
-  const unsigned gm = gmask_mixed<D>();
-  const int64_t ar0 = (blockIdx.x * (int64_t)GROUPS + grp) * kMixRows;
+__global__ void __launch_bounds__(128, D == 16 ? 3 : 2) k_lin_ma_mixed(MixedLinArgs a) {
+  constexpr int LPR = D / 2;
+  extern __shared__ __align__(16) unsigned char mix_smem[];
+  MixNet<D>& W = reinterpret_cast<MixNet<D>*>(mix_smem)[threadIdx.x >> 5];
+  MixRow<D>& S =
+      reinterpret_cast<MixRow<D>*>(mix_smem + 4 * sizeof(MixNet<D>))[threadIdx.x / LPR];
+  const int l32 = threadIdx.x & 31, lane = l32 % LPR, grp = l32 / LPR;
   const int64_t rows = a.bt.act_rows();
-  const int R = a.dv.R < RMAX ? a.dv.R : RMAX;
+  const int64_t lo = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * kMixRows;
+  const int64_t hi = lo + kMixRows < rows ? lo + kMixRows : rows;
+  const int R = a.dv.R < kMixReact ? a.dv.R : kMixReact;
   int64_t cur = -1;
-  const int4* tt = nullptr;
-  const int32_t* ae = nullptr;
-  int e0 = 0, e1 = 0;
-  int4 q[RPL];
-  double kd[RPL];
-  float kf[RPL];
-  bool fast = true;
+  int most_t = 0, most_g = 0;
+  bool tail = false, fast = true;
   float mx = 0.f, sq = 0.f;
   unsigned long long key = 0ull;  // first failing row (sliding window)
-  for (int ri = 0; ri < kMixRows && ar0 + ri < rows; ++ri) {  // uniform over the group
+  if (lane == 0) {
+    S.c[D] = 1.f;
+    S.cd[D] = 1.0;
+  }
+  for (int64_t pos = lo; pos < hi;) {  // uniform over the warp
     int64_t seq, row;
-    act_row(a.bt, ar0 + ri, seq, row);
-    if (seq != cur) {
-      if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
-      cur = seq;
+    act_row(a.bt, pos + grp < hi ? pos + grp : hi - 1, seq, row);
+    // the step's rows are those of its first row's sequence
+    const int64_t sq0 = __shfl_sync(0xffffffffu, seq, 0);
+    const bool valid = pos + grp < hi && seq == sq0;
+    pos += __popc(__ballot_sync(0xffffffffu, valid)) / LPR;
+    if (sq0 != cur) {
+      if (cur >= 0) acc_resid_group<32>(a.acc, cur, mx, sq, key, l32, 0xffffffffu);
+      cur = sq0;
       mx = 0.f;
       sq = 0.f;
       key = 0ull;
-      const double* kk = a.dv.params + seq * a.dv.pstride;
-      tt = reinterpret_cast<const int4*>(a.dv.topo + seq * a.dv.tstride);
-      const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1);
-      ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
-      e0 = __ldg(aoff + lane);
-      e1 = __ldg(aoff + lane + 1);
-      mixed_list<D>(sList[grp], lane, tt, ae, e0, e1);
-#pragma unroll
-      for (int k = 0; k < RPL; ++k) {
-        const int r = k * D + lane;
-        q[k] = __ldg(tt + (r < R ? r : 0));
-        kd[k] = r < R ? __ldg(kk + r) : 0.0;
-        kf[k] = d2f_trunc(kd[k]);
+      fast = a.it == 0 || a.info[cur].max_resid > kMixedFastAbove;
+      __syncwarp();
+      mix_net<D>(a, cur, R, l32, W, most_t, most_g);
+      const int32_t* aoff = a.adj_off + (a.adj_stride ? cur : 0) * (D + 1);
+      tail = __any_sync(0xffffffffu,
+                        l32 < D && __ldg(aoff + (l32 < D ? l32 : 0) + 1) -
+                                           __ldg(aoff + (l32 < D ? l32 : 0)) > kMixList);
+      for (int j = lane; j < D * (D + 4); j += LPR) S.G[j] = 0.f;
+      if (lane == 0) {
+        if (fast) reinterpret_cast<float*>(S.rate)[kMixReact] = 0.f;
+        else S.rate[kMixReact] = 0.0;
       }
-      fast = a.it == 0 || a.info[seq].max_resid > kMixedFastAbove;
+      __syncwarp();
     }
-    const double s_prev = row == __ldg(a.bt.offsets + seq) ? a.s0[seq * D + lane]
-                                                          : a.s[(row - 1) * D + lane];
-    const double sc = a.s[row * D + lane];
-    __nv_bfloat16* Eo = a.E + row * (int64_t)(D * D);
-    float* bo = a.b + row * D;
+    const bool row_first = row == __ldg(a.bt.offsets + seq);
+    double sp[2], sc[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      sp[x] = row_first ? a.s0[seq * D + 2 * lane + x] : a.s[(row - 1) * D + 2 * lane + x];
+      sc[x] = a.s[row * D + 2 * lane + x];
+    }
     if (fast)
-      mixed_row<float, D, RK4, RPL>(a, true, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
-                                    e0, e1, sList[grp], sG[grp], sK[grp],
-                                    reinterpret_cast<float*>(sRate[grp]), sD1[grp], sD2[grp],
-                                    mx, sq, seq, key, Eo, bo);
+      mixed_row_cols<float, D, RK4>(a, valid, cur, row, lane, W, S, R, most_t, most_g, tail, sp,
+                                    sc, mx, sq, key);
     else
-      mixed_row<double, D, RK4, RPL>(a, true, row, lane, gm, s_prev, sc, q, kd, kf, R, tt, ae,
-                                     e0, e1, sList[grp], sG[grp], sK[grp], sRate[grp],
-                                     sD1[grp], sD2[grp], mx, sq, seq, key, Eo, bo);
+      mixed_row_cols<double, D, RK4>(a, valid, cur, row, lane, W, S, R, most_t, most_g, tail,
+                                     sp, sc, mx, sq, key);
   }
-  if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
+  if (cur >= 0) acc_resid_group<32>(a.acc, cur, mx, sq, key, l32, 0xffffffffu);
+}
+
+template <int D, bool RK4>
+static cudaError_t lin_mixed_launch(const MixedLinArgs& a, cudaStream_t st) {
+  auto kern = k_lin_ma_mixed<D, RK4>;
+  static thread_local bool configured = false;  // per host thread: the attribute took
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem<D>);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  kern<<<grid_for(a.bt.act_rows(), 4 * kMixRows), 128, kMixSmem<D>, st>>>(a);
+  note_launch();
+  return cudaGetLastError();
 }
 
 // ---- mixed dense scan: lane j owns column j of P and entry j of the vectors ----------
@@ -617,12 +921,12 @@ __device__ __forceinline__ void rc_row(const MixedLinArgs& a, bool fast, bool va
     mixed_row<float, 16, RK4, kRcRmax / 16>(
         a, valid, row, lane, gm, sp, sc, n.q, n.kd, n.kf, n.R, n.tt, n.ae, n.e0, n.e1,
         S.list, S.G[half], S.K[half], reinterpret_cast<float*>(S.rate[half]), S.d1[half],
-        S.d2[half], mx, sq, seq, key, nullptr, S.b[half], S.E[half]);
+        S.d2[half], mx, sq, seq, key, S.b[half], S.E[half]);
   else
     mixed_row<double, 16, RK4, kRcRmax / 16>(
         a, valid, row, lane, gm, sp, sc, n.q, n.kd, n.kf, n.R, n.tt, n.ae, n.e0, n.e1,
         S.list, S.G[half], S.K[half], S.rate[half], S.d1[half], S.d2[half], mx, sq, seq, key,
-        nullptr, S.b[half], S.E[half]);
+        S.b[half], S.E[half]);
 }
 
 // P^T <- P^T + P^T E^T for the warp's 16 x 16 accumulator acc[n-tile][4] (lane (g, t):
@@ -821,18 +1125,11 @@ cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
   const bool rk4 = a.dv.kind == DEER_F_MASSACTION_RK4;
   const int d = a.dv.d;
-  const unsigned g = grid_for(a.bt.act_rows(), 128 / d * kMixRows);
-  if (d == 16) {
-    if (rk4) k_lin_ma_mixed<16, true><<<g, 128, 0, st>>>(a);
-    else k_lin_ma_mixed<16, false><<<g, 128, 0, st>>>(a);
-  } else if (d == 32) {
-    if (rk4) k_lin_ma_mixed<32, true><<<g, 128, 0, st>>>(a);
-    else k_lin_ma_mixed<32, false><<<g, 128, 0, st>>>(a);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  note_launch();
-  return cudaGetLastError();
+  if (d == 16)
+    return rk4 ? lin_mixed_launch<16, true>(a, st) : lin_mixed_launch<16, false>(a, st);
+  if (d == 32)
+    return rk4 ? lin_mixed_launch<32, true>(a, st) : lin_mixed_launch<32, false>(a, st);
+  return cudaErrorInvalidValue;
 }
 
 template <int D>
