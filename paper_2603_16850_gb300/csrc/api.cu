@@ -137,7 +137,9 @@ static bool use_compensated(const deer_dynamics* f, const deer_options* o) {
          o->damp != DEER_DAMP_ELK && (f->d == 4 || f->d == 8 || f->d == 16 || f->d == 32);
 }
 
-static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N, bool lean) {
+static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t B, int64_t N,
+                        bool lean) {
+  const int d = f->d;
   if (use_diag_lookback(o, d)) return diag_lb_chunk(d);
   if (o->chunk > 0) return o->chunk;
   if (o->jac == DEER_JAC_FULL && d >= 16) return 32;
@@ -152,6 +154,14 @@ static int choose_chunk(const deer_options* o, int d, int64_t B, int64_t N, bool
     const int64_t T = B > 0 ? N / B : 0;
     const int64_t r = o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK ? 8 : 2;
     while (!lean && L > 16 && N / L * d < 152 * 4 * 32 && T <= r * L * L) L /= 2;
+    // Float64 kinetics issue-bound on a few warps: up to four warps per scheduler (a row more on
+    // one scheduler than on the next is then a smaller part), while the carry's T / 8 steps stay
+    // the shorter chain. L = 8 against 16, ms: 37 x 1501 rows 6.6 / 7.7, 101 x 701 4.7 / 5.3,
+    // 301 x 401 6.9 / 7.4, 7 x 801 2.1 / 3.3; 20 x 3001 6.1 / 5.7, 16 x 16384 25.8 / 21.9.
+    const bool kinetics =
+        f->kind == DEER_F_MASSACTION_EULER || f->kind == DEER_F_MASSACTION_RK4;
+    if (!lean && kinetics && o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK && T <= 2048)
+      while (L > 8 && N / L * d < 608 * 4 * 32) L /= 2;
     return L;
   }
   return 128;
@@ -179,7 +189,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   const size_t rs = o->prec == DEER_FP32 ? 4 : 8;
   const bool mixed = o->prec == DEER_MIXED_BF16;
   const int d = f->d;
-  const int L = choose_chunk(o, d, B, N, lean);
+  const int L = choose_chunk(f, o, B, N, lean);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
   ly.n_chunks_max = N / L + B + 1;
