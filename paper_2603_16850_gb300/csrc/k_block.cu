@@ -41,6 +41,27 @@ namespace deer {
 template <class real>
 constexpr real kRealMax = sizeof(real) == 8 ? real(DBL_MAX) : real(FLT_MAX);
 
+// Half an ulp of a tolerance (0 where that underflows).
+__device__ __forceinline__ double half_ulp(double t) {
+  const int e = (__double2hiint(t) >> 20) & 0x7ff;
+  return e > 53 ? __hiloint2double((e - 53) << 20, 0) : 0.0;
+}
+__device__ __forceinline__ float half_ulp(float t) {
+  const int e = (__float_as_int(t) >> 23) & 0xff;
+  return e > 24 ? __int_as_float((e - 24) << 23) : 0.f;
+}
+
+// !(|r| / |s| <= tol) as the division rounds, for |s| > 1 and tol >= 0, without dividing: the
+// quotient rounds to tol or below exactly when |r| <= |s| (tol + half an ulp) (no quotient lies
+// on that midpoint). More than two ulps from tol |s| the bit patterns decide.
+template <class real>
+__device__ __forceinline__ bool over_tol(real r, real s, real tol) {
+  const real lim = tol * rabs(s);
+  const auto rb = mag_bits(r), lb = mag_bits(lim);
+  if (rb - lb + 2u <= 4u) return fma(-tol, rabs(s), rabs(r)) > rabs(s) * half_ulp(tol);
+  return rb > lb;
+}
+
 template <class real, int D>
 struct Aff {  // the affine map Delta -> P Delta + v
   real P[D][D];
@@ -174,7 +195,9 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
   // the last thread of the previous block (full whenever this one has rows)
   const int prev_last = threads - 1;
   const real scale = a.damp == DEER_DAMP_SCALE ? real(1) - a.dparam : real(1);
-  // the test in the kernel's precision: the largest value not above tol
+  // the test in the kernel's precision: the largest value not above tol. A negative or NaN
+  // tolerance is met by nothing (the comparisons below drop its sign), also with no rows
+  const bool tol_met = a.tol >= 0.0;
   const real tol = sizeof(real) == 8 ? (real)a.tol : (real)__double2float_rd(a.tol);
   const auto thr_bits = mag_bits(a.reset_thr);
   real s[RPT][D];
@@ -222,7 +245,7 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
     }
     // 1. linearise, test, this thread's element; F and A are kept for the apply pass
     Aff<real, D> e = aff_identity<real, D>();
-    bool fail = false, bad = false;
+    bool fail = !tol_met, bad = false;
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       if (k < nmine) {
@@ -233,8 +256,7 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
           const real r = s[k][i] - Fk[k][i];
           st.v[i] = -r;
           const auto rb = mag_bits(r), sb = mag_bits(s[k][i]);
-          const real lim = sb > mag_bits(real(1)) ? tol * rabs(s[k][i]) : tol;
-          fail |= rb > mag_bits(lim);
+          fail |= sb > mag_bits(real(1)) ? over_tol(r, s[k][i], tol) : rb > mag_bits(tol);
           bad |= rb > mag_bits(kRealMax<real>) || sb > mag_bits(kRealMax<real>);
 #pragma unroll
           for (int j = 0; j < D; ++j) {
