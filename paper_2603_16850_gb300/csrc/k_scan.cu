@@ -995,62 +995,31 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
   if (warp == 0) vo[lane] = v;
 }
 
-// Carry pass: x_c = P_c x_{c-1} + v_c along each active sequence's chunks; the aggregates do
-// not depend on x and stream through the ring. MODE 0: one group per sequence, over its
-// chunks. Few sequences of many chunks make that the longest chain of the iteration (3125
-// chunks of the mean-field RNN, d = 32, T = 100000: 580 us); the chunks are then folded into
-// segments of M (the chunk pass again, over the aggregates), MODE 1 walks a sequence's
-// segments, MODE 2 the chunks of each segment from the value entering it: 39 + 20 + 10 us
-// there. (Mixed-precision ragged batch, d = 16, up to 3125 chunks a sequence: 134 -> 27 ms of
-// scans per solve, against a carry that loaded each aggregate when it needed it.)
-template <class real, int D, int MODE>
-__global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) {
-  constexpr int W = group_lanes<D>(), G = 32 / W;
-  using Ring = RowRing<real, D>;
-  constexpr int K = Ring::K;
-  __shared__ __align__(16) Ring ring[G];
-  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
-  const int li = lane < D ? lane : 0;  // this lane's row
+// x <- P_c x + v_c over the aggregates c0 .. c1 - 1, streamed through the ring; the x entering
+// each goes to `in` (if any). `first`: c0 starts from Delta = 0 and its P is not formed. With
+// CHECK, returns the first aggregate that would leave x non-finite, x being the value that
+// enters it; otherwise c1.
+template <bool CHECK, class real, int D>
+__device__ __forceinline__ int64_t carry_walk(RowRing<real, D>& R, const real* P, const real* v,
+                                              real* in, int64_t c0, int64_t c1, bool first,
+                                              real& x) {
+  constexpr int W = group_lanes<D>(), K = RowRing<real, D>::K;
+  const int lane = threadIdx.x % W, li = lane < D ? lane : 0;  // this lane's row
   const unsigned gm = group_mask<D>();
-  const int64_t kq = blockIdx.x * (int64_t)G + grp;
-  const real* P = MODE == 1 ? a.segP : a.aggP;
-  const real* v = MODE == 1 ? a.segv : a.aggv;
-  real* in = MODE == 1 ? a.segin : a.cin;
-  int64_t c0, c1;
-  real x = real(0);
-  bool first = true;  // c0 starts from Delta = 0: its aggregate has no P
-  if constexpr (MODE == 2) {
-    Span p;
-    if (!get_span<true>(a, kq, p)) return;
-    c0 = p.r0;
-    c1 = p.r0 + p.n;
-    first = !p.need_P;
-    x = a.segin[p.out * D + li];
-  } else {
-    if (kq >= a.bt.n_act()) return;
-    const int64_t seq = a.bt.act_seq[kq];
-    c0 = win_first(a.bt, seq);
-    c1 = a.bt.chunk_first[seq + 1];
-    if constexpr (MODE == 1) {
-      const int64_t nseg = (c1 - c0 + (1 << a.log2M) - 1) >> a.log2M;
-      c0 = (a.bt.chunk_first[seq] >> a.log2M) + seq;
-      c1 = c0 + nseg;
-    }
-  }
-  Ring& R = ring[grp];
 #pragma unroll
   for (int s = 0; s < K; ++s) {
     if (c0 + s < c1) R.issue(s, lane, P + (c0 + s) * (int64_t)(D * D), v + (c0 + s) * D);
     cp_async_commit();
   }
-  for (int64_t cb = c0; cb < c1; cb += K) {
+  int64_t stop = c1;
+  for (int64_t cb = c0; cb < c1 && stop == c1; cb += K) {
 #pragma unroll
     for (int s = 0; s < K; ++s) {
       const int64_t c = cb + s;
       cp_async_wait<K - 1>();
       __syncwarp(gm);  // the other lanes' pieces of this slot have landed
-      if (c < c1) {
-        if (lane < D) in[c * D + lane] = x;
+      if (c < stop) {
+        if (in && lane < D) in[c * D + lane] = x;
         real y = R.v[s][li];
         if (!first || c > c0) {
           real pr[D];
@@ -1058,15 +1027,67 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
 #pragma unroll
           for (int k = 0; k < D; ++k) y += pr[k] * __shfl_sync(gm, x, k, W);
         }
-        x = y;
+        if (CHECK && __any_sync(gm, mag_bits(y) >= mag_bits(real(INFINITY)))) stop = c;
+        else x = y;
       }
       __syncwarp(gm);  // every lane is done with the slot before it is refilled
-      if (c + K < c1)
+      if (c + K < stop)
         R.issue(s, lane, P + (c + K) * (int64_t)(D * D), v + (c + K) * D);
       cp_async_commit();
     }
   }
   cp_async_wait<0>();
+  __syncwarp(gm);  // the ring may be refilled
+  return stop;
+}
+
+// Carry pass: x_c = P_c x_{c-1} + v_c along each active sequence's chunks. MODE 0: one group
+// per sequence, over its
+// chunks. Few sequences of many chunks make that the longest chain of the iteration (3125
+// chunks of the mean-field RNN, d = 32, T = 100000: 580 us); the chunks are then folded into
+// segments of M (the chunk pass again, over the aggregates), MODE 1 walks a sequence's
+// segments, MODE 2 the chunks of each segment from the value entering it: 39 + 20 + 10 us
+// there. (Mixed-precision ragged batch, d = 16, up to 3125 chunks a sequence: 134 -> 27 ms of
+// scans per solve, against a carry that loaded each aggregate when it needed it.)
+// A product over a segment (up to 64 chunks) can overflow where those over its chunks do not,
+// and inf times a Delta of zero would then spread NaN over rows that are solved already: MODE
+// 1 walks such a segment's chunks one by one.
+template <class real, int D, int MODE>
+__global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) {
+  constexpr int W = group_lanes<D>(), G = 32 / W;
+  __shared__ __align__(16) RowRing<real, D> ring[G];
+  const int grp = threadIdx.x / W, lane = threadIdx.x % W;
+  const int64_t kq = blockIdx.x * (int64_t)G + grp;
+  RowRing<real, D>& R = ring[grp];
+  real x = real(0);
+  if constexpr (MODE == 2) {
+    Span p;
+    if (!get_span<true>(a, kq, p)) return;
+    x = a.segin[p.out * D + (lane < D ? lane : 0)];
+    carry_walk<false, real, D>(R, a.aggP, a.aggv, a.cin, p.r0, p.r0 + p.n, !p.need_P, x);
+  } else {
+    if (kq >= a.bt.n_act()) return;
+    const int64_t seq = a.bt.act_seq[kq];
+    const int64_t c0 = win_first(a.bt, seq), c1 = a.bt.chunk_first[seq + 1];
+    if constexpr (MODE == 0) {
+      carry_walk<false, real, D>(R, a.aggP, a.aggv, a.cin, c0, c1, true, x);
+    } else {
+      const int64_t M = (int64_t)1 << a.log2M;
+      const int64_t s0 = (a.bt.chunk_first[seq] >> a.log2M) + seq;
+      const int64_t s1 = s0 + ((c1 - c0 + M - 1) >> a.log2M);
+      carry_walk<false, real, D>(R, a.segP, a.segv, a.segin, s0, s1, true, x);
+      // (a non-finite entry makes every entry after it non-finite: only the end is looked at)
+      if (!__any_sync(group_mask<D>(), mag_bits(x) >= mag_bits(real(INFINITY)))) return;
+      x = real(0);
+      for (int64_t k = s0; k < s1; ++k) {
+        k = carry_walk<true, real, D>(R, a.segP, a.segv, a.segin, k, s1, k == s0, x);
+        if (k == s1) break;
+        const int64_t q0 = c0 + (k - s0) * M;
+        carry_walk<false, real, D>(R, a.aggP, a.aggv, nullptr, q0, q0 + M < c1 ? q0 + M : c1,
+                                   k == s0, x);
+      }
+    }
+  }
 }
 
 // Apply pass: Delta_t = A_t Delta_{t-1} + b_t from the chunk's carry, s_t += Delta_t; lane
