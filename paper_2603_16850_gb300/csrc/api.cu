@@ -175,6 +175,10 @@ static int grad_chunk(const deer_dynamics* f, const deer_options* o) {
   return f->d >= 16 ? 32 : 64;
 }
 
+// Most reactions that a species' list can number (16 bits of an entry, launch_ma_adjacency);
+// the linearisation of larger networks walks every reaction.
+constexpr int kMaxListed = 65536;
+
 // Largest row count any layout accepts: keeps every size product below (N + C) d^2 * 8
 // far from overflowing 64 bits (d <= 64).
 constexpr int64_t kMaxRows = int64_t(1) << 44;
@@ -269,7 +273,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   }
   ly.adj_off = ly.adj_e = p;
   const bool ma_kind = f->kind == DEER_F_MASSACTION_EULER || f->kind == DEER_F_MASSACTION_RK4;
-  if (mixed || (ma_kind && (d == 16 || d == 32))) {
+  if (mixed || (ma_kind && (d == 16 || d == 32) && f->n_reactions <= kMaxListed)) {
     // per-species reaction lists (the mixed path's and the wide linearisation's)
     const int64_t nseq = f->topology_stride ? (B > 0 ? B : 1) : 1;
     ly.adj_off = take((size_t)nseq * (d + 1) * 4);
