@@ -467,11 +467,13 @@ static cudaError_t block_launch(const BlockSolveArgs<real>& a, cudaStream_t st) 
   int64_t cl = (a.max_T + kBlockThreads / 2 - 1) / (kBlockThreads / 2);
   cl = cl < 1 ? 1 : (cl > kWideCluster ? kWideCluster : cl);
   if (cl > kMaxCluster) {
-    static thread_local int wide_ok = -1;  // per host thread: 1 if the attribute took
-    if (wide_ok < 0)
-      wide_ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                     1) == cudaSuccess ? 1 : 0;
-    if (!wide_ok) cl = kMaxCluster;
+    static DeviceOnce wide;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (wide.ensure(dev, [&] {
+          return cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        }) != cudaSuccess)
+      cl = kMaxCluster;
     (void)cudaGetLastError();
   }
   cudaLaunchAttribute attr[1];
@@ -481,13 +483,9 @@ static cudaError_t block_launch(const BlockSolveArgs<real>& a, cudaStream_t st) 
   cudaLaunchConfig_t cfg{};
   cfg.blockDim = dim3(kBlockThreads, 1, 1);
   cfg.dynamicSmemBytes = sizeof(real) * (kBlockThreads / 32) * 63 * (kEl<D> + D);
-  static thread_local bool smem_ok = false;  // per host thread: the attribute took
-  if (!smem_ok) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
-    if (e != cudaSuccess) return e;
-    smem_ok = true;
-  }
+  static DeviceOnce smem_ok;
+  const cudaError_t se = allow_smem(smem_ok, kern, cfg.dynamicSmemBytes);
+  if (se != cudaSuccess) return se;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;

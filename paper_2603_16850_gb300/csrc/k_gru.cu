@@ -320,13 +320,9 @@ cudaError_t launch_gru_xproj(const float* W, const float* x, int64_t N, float* o
                              cudaStream_t st) {
   if (N == 0) return cudaSuccess;
   const int smem = (int)sizeof(XprojSmem);
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_gru_xproj, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce configured;
+  const cudaError_t e = allow_smem(configured, k_gru_xproj, smem);
+  if (e != cudaSuccess) return e;
   const int g = persistent_grid((const void*)k_gru_xproj, 256, smem);
   const int64_t tiles = (N + kXR - 1) / kXR;
   k_gru_xproj<<<(unsigned)(tiles < g ? tiles : g), 256, smem, st>>>(
@@ -338,13 +334,9 @@ cudaError_t launch_gru_xproj(const float* W, const float* x, int64_t N, float* o
 cudaError_t launch_gru_lin_tiled(const GruTileArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
   const size_t smem = sizeof(GruSmem);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_gru_lin_tiled,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce configured;
+  const cudaError_t e = allow_smem(configured, k_gru_lin_tiled, smem);
+  if (e != cudaSuccess) return e;
   const int g = persistent_grid((const void*)k_gru_lin_tiled, kGThreads, smem);
   const int64_t tiles = (a.bt.act_rows() + kGT - 1) / kGT;
   k_gru_lin_tiled<<<(unsigned)(tiles < g ? tiles : g), kGThreads, smem, st>>>(a);

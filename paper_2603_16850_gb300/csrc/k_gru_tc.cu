@@ -382,13 +382,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gru_lin_tc(GruTileArgs a) {
 cudaError_t launch_gru_lin_tc(const GruTileArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
   const int smem = (int)sizeof(TcSmem);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_gru_lin_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce configured;
+  const cudaError_t e = allow_smem(configured, k_gru_lin_tc, smem);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

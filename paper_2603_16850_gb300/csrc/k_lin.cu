@@ -1002,14 +1002,10 @@ __global__ void __launch_bounds__(128, (D == 32 && sizeof(real) == 4) ? 4 : 1)
 
 template <class real, int D, bool RK4, int JAC>
 static cudaError_t lin_ma_wide_launch(const LinArgs<real>& a, unsigned g, cudaStream_t st) {
-  const int smem = (int)sizeof(MaListSmem<real, D>);
-  static thread_local bool configured = false;  // per host thread: the attribute took
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_lin_ma_wide<real, D, RK4, JAC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  const size_t smem = sizeof(MaListSmem<real, D>);
+  static DeviceOnce configured;
+  const cudaError_t e = allow_smem(configured, k_lin_ma_wide<real, D, RK4, JAC>, smem);
+  if (e != cudaSuccess) return e;
   k_lin_ma_wide<real, D, RK4, JAC><<<g, 128, smem, st>>>(a);
   note_launch();
   return cudaGetLastError();

@@ -635,13 +635,9 @@ __global__ void __launch_bounds__(128, D == 16 ? 3 : 2) k_lin_ma_mixed(MixedLinA
 template <int D, bool RK4>
 static cudaError_t lin_mixed_launch(const MixedLinArgs& a, cudaStream_t st) {
   auto kern = k_lin_ma_mixed<D, RK4>;
-  static thread_local bool configured = false;  // per host thread: the attribute took
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem<D>);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce configured;
+  const cudaError_t e = allow_smem(configured, kern, kMixSmem<D>);
+  if (e != cudaSuccess) return e;
   kern<<<grid_for(a.bt.act_rows(), 4 * kMixRows), 128, kMixSmem<D>, st>>>(a);
   note_launch();
   return cudaGetLastError();

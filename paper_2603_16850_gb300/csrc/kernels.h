@@ -3,8 +3,20 @@
 #pragma once
 
 #include "common.cuh"
+#include "device_once.h"
 
 namespace deer {
+
+// Lets `kern` use `bytes` of dynamic shared memory on the current device; `once` is the kernel's.
+template <class Kern>
+inline cudaError_t allow_smem(DeviceOnce& once, Kern* kern, size_t bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once.ensure(dev, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
 
 template <class real>
 struct InitArgs {
