@@ -267,7 +267,8 @@ typedef struct {
 void deer_default_options(deer_options* opt);
 
 /* Workspace bytes needed by deer_solve / deer_solve_batched for `batch` sequences
-   holding `total_steps` rows in all. Returns 0 for an invalid configuration. */
+   holding `total_steps` rows in all. Never less for more sequences or rows (jac_bytes_max = 0),
+   so one workspace serves every smaller problem. Returns 0 for an invalid configuration. */
 size_t deer_workspace_bytes(const deer_dynamics* f, int64_t batch, int64_t total_steps,
                             const deer_options* opt);
 

@@ -137,6 +137,23 @@ static bool use_compensated(const deer_dynamics* f, const deer_options* o) {
          o->damp != DEER_DAMP_ELK && (f->d == 4 || f->d == 8 || f->d == 16 || f->d == 32);
 }
 
+// Default chunk of the full Jacobian at d < 16: kLongChunk rows, fewer while the lanes (d per
+// chunk) of a whole problem stay below a bound.
+constexpr int kLongChunk = 64;
+constexpr int64_t kFewLanes = 152 * 4 * 32;       // four warps per SM
+constexpr int64_t kFewLanesF64 = 608 * 4 * 32;    // four warps per scheduler
+
+// The caller leaves the chunk length to the rule on sizes (`lean`: see make_layout).
+static bool chunk_by_size(const deer_options* o, int d, bool lean) {
+  return !lean && o->chunk <= 0 && o->jac == DEER_JAC_FULL && d < 16;
+}
+
+// Float64 kinetics: chunks down to eight rows, up to kFewLanesF64.
+static bool chunk_to_eight(const deer_dynamics* f, const deer_options* o) {
+  return (f->kind == DEER_F_MASSACTION_EULER || f->kind == DEER_F_MASSACTION_RK4) &&
+         o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK;
+}
+
 static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t B, int64_t N,
                         bool lean) {
   const int d = f->d;
@@ -150,21 +167,37 @@ static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t B
     // row costs several times a carry step, except under dense ELK, whose covariance carry
     // inverts a matrix per chunk. Mass action d = 8,
     // float64, 37 x 1501 rows: L = 16 solves in 5.5 ms, L = 32 in 8.0, L = 64 in 15.2.
-    int L = 64;
+    int L = kLongChunk;
+    if (!chunk_by_size(o, d, lean)) return L;
     const int64_t T = B > 0 ? N / B : 0;
     const int64_t r = o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK ? 8 : 2;
-    while (!lean && L > 16 && N / L * d < 152 * 4 * 32 && T <= r * L * L) L /= 2;
+    while (L > 16 && N / L * d < kFewLanes && T <= r * L * L) L /= 2;
     // Float64 kinetics issue-bound on a few warps: up to four warps per scheduler (a row more on
     // one scheduler than on the next is then a smaller part), while the carry's T / 8 steps stay
     // the shorter chain. L = 8 against 16, ms: 37 x 1501 rows 6.6 / 7.7, 101 x 701 4.7 / 5.3,
     // 301 x 401 6.9 / 7.4, 7 x 801 2.1 / 3.3; 20 x 3001 6.1 / 5.7, 16 x 16384 25.8 / 21.9.
-    const bool kinetics =
-        f->kind == DEER_F_MASSACTION_EULER || f->kind == DEER_F_MASSACTION_RK4;
-    if (!lean && kinetics && o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK && T <= 2048)
-      while (L > 8 && N / L * d < 608 * 4 * 32) L /= 2;
+    if (chunk_to_eight(f, o) && T <= 2048)
+      while (L > 8 && N / L * d < kFewLanesF64) L /= 2;
     return L;
   }
   return 128;
+}
+
+// Chunks to make room for: the most that any problem of up to B sequences and N rows in all has,
+// so that a workspace that holds a problem holds every smaller one too (the rule above gives a
+// smaller problem shorter chunks, and more of them). A chunk is halved only while the chunks
+// before number fewer than lanes / d.
+static int64_t chunk_room(const deer_dynamics* f, const deer_options* o, int64_t B, int64_t N,
+                          int L, bool lean) {
+  int64_t n = N / L;
+  if (chunk_by_size(o, f->d, lean)) {
+    const bool eight = chunk_to_eight(f, o);
+    const int64_t most = 2 * (((eight ? kFewLanesF64 : kFewLanes) - 1) / f->d) + 1;
+    const int64_t all = N / (eight ? 8 : 16);  // every chunk at its shortest
+    const int64_t halved = all < most ? all : most;
+    n = N / kLongChunk > halved ? N / kLongChunk : halved;
+  }
+  return n + B + 1;
 }
 
 // Chunk length of the adjoint where the caller leaves it to the library: fixed by d in
@@ -196,7 +229,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   const int L = choose_chunk(f, o, B, N, lean);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
-  ly.n_chunks_max = N / L + B + 1;
+  ly.n_chunks_max = chunk_room(f, o, B, N, L, lean);
   const int64_t C = ly.n_chunks_max;
   size_t p = 0;
   auto take = [&](size_t bytes) { size_t at = p; p = align_up(p + bytes); return at; };
@@ -240,7 +273,9 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
              dense_fused_supported(f->kind, d)) {
     // pending Jacobians / offsets of the fused path (chunk-major or chunk-interleaved),
     // padded to whole chunks and to groups of 32 chunks
-    const size_t rows = (size_t)((C + 31) / 32 * 32) * L;
+    // (at any chunk length of the rule, where the rule chooses it)
+    const size_t rows = chunk_by_size(o, d, lean) ? (size_t)(N + (B + 32) * kLongChunk)
+                                                  : (size_t)((C + 31) / 32 * 32) * L;
     ly.A = take(rows * d * d * rs);
     ly.b = take(rows * d * rs);
   } else {
