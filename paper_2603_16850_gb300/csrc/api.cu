@@ -1,5 +1,6 @@
 // Host side of the C ABI: argument checks, workspace layout and the Newton loop of
 // Algorithm alg:deer (linearise -> convergence test -> parallel scan, repeated).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <mutex>
@@ -154,8 +155,9 @@ static bool chunk_to_eight(const deer_dynamics* f, const deer_options* o) {
          o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK;
 }
 
-static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t B, int64_t N,
-                        bool lean) {
+// `longest`: rows of the longest sequence.
+static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t N,
+                        int64_t longest, bool lean) {
   const int d = f->d;
   if (use_diag_lookback(o, d)) return diag_lb_chunk(d);
   if (o->chunk > 0) return o->chunk;
@@ -165,11 +167,12 @@ static int choose_chunk(const deer_dynamics* f, const deer_options* o, int64_t B
     // warps per SM, as long as the per-sequence carry stays the shorter chain: it walks
     // T / L chunks at about half the time of the chunk passes' L rows in float32; a float64
     // row costs several times a carry step, except under dense ELK, whose covariance carry
-    // inverts a matrix per chunk. Mass action d = 8,
+    // inverts a matrix per chunk. T is the longest sequence's: its carry is the chain that an
+    // iteration waits for. Mass action d = 8,
     // float64, 37 x 1501 rows: L = 16 solves in 5.5 ms, L = 32 in 8.0, L = 64 in 15.2.
     int L = kLongChunk;
     if (!chunk_by_size(o, d, lean)) return L;
-    const int64_t T = B > 0 ? N / B : 0;
+    const int64_t T = longest;
     const int64_t r = o->prec == DEER_FP64 && o->damp != DEER_DAMP_ELK ? 8 : 2;
     while (L > 16 && N / L * d < kFewLanes && T <= r * L * L) L /= 2;
     // Float64 kinetics issue-bound on a few warps: up to four warps per scheduler (a row more on
@@ -217,16 +220,17 @@ constexpr int kMaxListed = 65536;
 constexpr int64_t kMaxRows = int64_t(1) << 44;
 
 // `lean` (deer_solve_noalloc, whose scratch is a fixed area): no tables or chunk counts beyond
-// what the plain forms of the kernels need.
+// what the plain forms of the kernels need. `longest`: rows of the longest sequence, which the
+// chunk length depends on and the sizes do not; -1 = sequences of equal length.
 static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer_options* o,
-                        Layout& ly, bool lean = false) {
+                        Layout& ly, bool lean = false, int64_t longest = -1) {
   if (!f || !o || B < 0 || N < 0) return false;
   if (N > kMaxRows || B > kMaxRows || f->d <= 0 || f->d > 64) return false;
   if (o->prec != DEER_FP64 && o->prec != DEER_FP32 && o->prec != DEER_MIXED_BF16) return false;
   const size_t rs = o->prec == DEER_FP32 ? 4 : 8;
   const bool mixed = o->prec == DEER_MIXED_BF16;
   const int d = f->d;
-  const int L = choose_chunk(f, o, B, N, lean);
+  const int L = choose_chunk(f, o, N, longest >= 0 ? longest : B > 0 ? N / B : 0, lean);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
   ly.n_chunks_max = chunk_room(f, o, B, N, L, lean);
@@ -440,8 +444,11 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
                               const void* s0_, const void* x_, void* s_, const deer_options* o,
                               void* ws_, size_t ws_bytes, cudaStream_t st, deer_info* info_h) {
   const int64_t N = offsets_h[B];
+  int64_t maxT = 0;
+  for (int64_t b = 0; b < B; ++b)
+    maxT = std::max(maxT, offsets_h[b + 1] - offsets_h[b]);
   Layout ly;
-  if (!make_layout(f, B, N, o, ly)) return DEER_ERR_INVALID;
+  if (!make_layout(f, B, N, o, ly, false, maxT)) return DEER_ERR_INVALID;
   if (!ws_ || ws_bytes < ly.total || (reinterpret_cast<uintptr_t>(ws_) & 255u))
     return DEER_ERR_WORKSPACE;
   char* ws = static_cast<char*>(ws_);
@@ -451,13 +458,12 @@ static deer_status solve_impl(const deer_dynamics* f, int64_t B, const int64_t* 
 
   // sequence / chunk tables
   std::vector<int64_t> chunk_first(B + 1);
-  int64_t maxT = 0, nc = 0;
+  int64_t nc = 0;
   for (int64_t b = 0; b < B; ++b) {
     const int64_t len = offsets_h[b + 1] - offsets_h[b];
     if (len < 0) return DEER_ERR_INVALID;
     chunk_first[b] = nc;
     nc += (len + ly.L - 1) / ly.L;
-    if (len > maxT) maxT = len;
   }
   chunk_first[B] = nc;
   if (offsets_h[0] != 0) return DEER_ERR_INVALID;
