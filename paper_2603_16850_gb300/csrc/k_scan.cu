@@ -1210,12 +1210,13 @@ __global__ void __launch_bounds__(128) k_scalar_apply(DenseScanArgs<real> a) {
 // M + n / M + M with M about sqrt(n), at the price of folding the aggregates once more. At
 // 157 chunks (Langevin, d = 4, float64) 28 us against 40 in one level; below 128 the two
 // extra launches cost what is saved. More sequences than SM sub-partitions x groups per warp
-// hide the chain by themselves.
+// hide the chain by themselves. The batch size decides, not the active set: the two forms round
+// differently, and a call keeps one of them, whatever else is still active and whichever loop runs.
 template <class real, int D>
 static void set_segments(DenseScanArgs<real>& a) {
   a.log2M = 0;
   const int64_t n = a.max_chunks;
-  if (!a.segP || n < 128 || a.bt.n_act() > 608 * (32 / group_lanes<D>())) return;
+  if (!a.segP || n < 128 || a.bt.B > 608 * (32 / group_lanes<D>())) return;
   a.log2M = 3;
   while (a.log2M < 6 && ((int64_t)1 << (2 * a.log2M + 2)) <= n) ++a.log2M;
 }
