@@ -230,6 +230,8 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   const size_t rs = o->prec == DEER_FP32 ? 4 : 8;
   const bool mixed = o->prec == DEER_MIXED_BF16;
   const int d = f->d;
+  const bool fused = !mixed && o->jac == DEER_JAC_FULL && o->damp != DEER_DAMP_ELK &&
+                     dense_fused_supported(f->kind, d);
   const int L = choose_chunk(f, o, N, longest >= 0 ? longest : B > 0 ? N / B : 0, lean);
   if (!pow2(L) || L < 8 || L > 1024) return false;
   ly.L = L;
@@ -273,8 +275,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
     // bfloat16 E = A - I, float32 offsets and aggregates
     ly.A = take((size_t)N * d * d * 2);
     ly.b = take((size_t)N * d * 4);
-  } else if (o->jac == DEER_JAC_FULL && o->damp != DEER_DAMP_ELK &&
-             dense_fused_supported(f->kind, d)) {
+  } else if (fused) {
     // pending Jacobians / offsets of the fused path (chunk-major or chunk-interleaved),
     // padded to whole chunks and to groups of 32 chunks
     // (at any chunk length of the rule, where the rule chooses it)
@@ -292,8 +293,8 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   ly.aggv = take((size_t)C * d * ars);
   ly.cin = take((size_t)C * d * ars);
   ly.segP = ly.segv = ly.segin = p;
-  if (o->jac == DEER_JAC_FULL && d > 1 && !lean) {
-    // segments of at least 8 chunks (two-level carry)
+  if (o->jac == DEER_JAC_FULL && d > 1 && !lean && !fused && C >= 128) {
+    // segments of at least 8 chunks (two-level carry of the dense scans, from 128 chunks on)
     const size_t S = (size_t)(C / 8 + B + 1);
     ly.segP = take(S * d * d * ars);
     ly.segv = take(S * d * ars);
@@ -322,9 +323,7 @@ static bool make_layout(const deer_dynamics* f, int64_t B, int64_t N, const deer
   if (gru_tiled_supported(f->kind, d, f->d_in, o->jac, o->prec))
     ly.xproj = take((size_t)N * 3 * d * rs);
   ly.sprev = p;
-  if (!mixed && o->jac == DEER_JAC_FULL && o->damp != DEER_DAMP_ELK &&
-      dense_fused_supported(f->kind, d))
-    ly.sprev = take((size_t)C * d * rs);
+  if (fused) ly.sprev = take((size_t)C * d * rs);
   ly.cs = use_compensated(f, o);
   ly.slo = ly.sprev_lo = p;
   if (ly.cs) {
