@@ -130,10 +130,10 @@ __device__ __forceinline__ void ld_row4(const float* p, float (&v)[D]) {
 // rates, slopes, F, residual) in V = float or double; the Jacobian path is float32 either
 // way. Writes E and b for the row and returns its scaled residual and squared residual.
 //
-// A lane per species: the recomputing path's form. The row's outputs go to Eo (its D x D
-// block of E) and bo (its entry of b = -r) in shared memory. sc is the row's own state s_t
-// (read by the caller).
-template <class V, int D, bool RK4, int RPL>
+// A lane per species: the form of d = 32 and of the recomputing path. The row's outputs go to
+// Eo (its D x D block of E) and bo (its entry of b = -r): bfloat16 in global memory, or float32
+// in shared memory on the recomputing path. sc is the row's own state s_t (read by the caller).
+template <class V, int D, bool RK4, int RPL, class TE>
 __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int64_t row,
                                           int lane, unsigned gm, double s_prev_d, double sc,
                                           const int4 (&q)[RPL], const double (&kd)[RPL],
@@ -143,7 +143,7 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
                                           float (*sK)[D + 4], V* sRate, float* sD1,
                                           float* sD2, float& mx, float& sq,
                                           int64_t seq, unsigned long long& key,
-                                          float* bo, float* Eo) {
+                                          float* bo, TE* Eo) {
   constexpr bool F64 = sizeof(V) == 8;
   const V s_prev = F64 ? (V)s_prev_d : (V)d2f_trunc(s_prev_d);
   const V h = F64 ? (V)a.dv.dt : (V)a.dt_f;
@@ -203,7 +203,8 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
     for (int e = e0 + kMixList; e < e1; ++e) {  // the rest of a long list
       const int code = __ldg(ae + e);
       const int4 qq = __ldg(tt + (code & 0xffff));
-      entry(code & 0xffff, (code >> 16) - 4, qq.x, qq.y);
+      if (qq.x >= 0 && qq.x < D && qq.y >= -1 && qq.y < D)  // (as in mixed_list)
+        entry(code & 0xffff, (code >> 16) - 4, qq.x, qq.y);
     }
     __syncwarp(gm);
     float Gi[D], Kn[D];
@@ -244,21 +245,28 @@ __device__ __forceinline__ void mixed_row(const MixedLinArgs& a, bool valid, int
     if (!(m <= a.tol_f) && key == 0ull) key = bad_key(true, row - __ldg(a.bt.offsets + seq));
     const float scale = a.scale_f;
     const float hwf = RK4 ? hf / 6.f : hf;
-    // E = A - I with A = I + hw Kacc (scaled by (1 - k) under scale-ELK: E = s A - I),
-    // float32 with rows padded to 20
-    float* Er = Eo + lane * 20;
+    // E = A - I with A = I + hw Kacc (scaled by (1 - k) under scale-ELK: E = s A - I):
+    // bfloat16, or float32 with rows padded to 20
+    auto e = [&](int j) { return scale * hwf * Kacc[j] + (j == lane ? scale - 1.f : 0.f); };
+    if constexpr (sizeof(TE) == 4) {
 #pragma unroll
-    for (int j = 0; j < D; j += 4)
-      *reinterpret_cast<float4*>(Er + j) =
-          make_float4(scale * hwf * Kacc[j] + (j == lane ? scale - 1.f : 0.f),
-                      scale * hwf * Kacc[j + 1] + (j + 1 == lane ? scale - 1.f : 0.f),
-                      scale * hwf * Kacc[j + 2] + (j + 2 == lane ? scale - 1.f : 0.f),
-                      scale * hwf * Kacc[j + 3] + (j + 3 == lane ? scale - 1.f : 0.f));
+      for (int j = 0; j < D; j += 4)
+        *reinterpret_cast<float4*>(Eo + lane * 20 + j) =
+            make_float4(e(j), e(j + 1), e(j + 2), e(j + 3));
+    } else {
+#pragma unroll
+      for (int j = 0; j < D; j += 8) {
+        __nv_bfloat162 w[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) w[m] = __floats2bfloat162_rn(e(j + 2 * m), e(j + 2 * m + 1));
+        *reinterpret_cast<uint4*>(Eo + lane * D + j) = *reinterpret_cast<const uint4*>(w);
+      }
+    }
     bo[lane] = -rf;
   }
 }
 
-// ---- linearisation: two columns per lane ------------------------------------------------
+// ---- linearisation, d = 16: two columns per lane ----------------------------------------
 // D / 2 lanes share a row: each forms the rate-Jacobian rows of its two species, then takes
 // its two columns of every stage Jacobian K_j = G_j (I + c_j K_{j-1}) with both factors of a
 // column at hand: K_{j-1}'s columns in registers, G's rows broadcast from shared memory, so
@@ -300,7 +308,7 @@ struct MixRow {  // one per row in flight
   float c[D + 4];   // c[D] = 1
   double cd[D + 2];
   double rate[kMixReact + 2];  // [kMixReact] = 0; floats in float32 mode
-  float pad[D == 16 ? 8 : 4];  // the rows of a warp in different banks
+  float pad[8];  // the rows of a warp in different banks (d = 16)
 };
 
 __device__ __forceinline__ float mix_nu(uint32_t w, float) {
@@ -567,9 +575,9 @@ __device__ __forceinline__ void mixed_row_cols(const MixedLinArgs& a, bool valid
 template <int D>
 constexpr size_t kMixSmem = 4 * sizeof(MixNet<D>) + 256 / D * sizeof(MixRow<D>);
 
-template <int D, bool RK4>
-__global__ void __launch_bounds__(128, D == 16 ? 3 : 2) k_lin_ma_mixed(MixedLinArgs a) {
-  constexpr int LPR = D / 2;
+template <bool RK4>
+__global__ void __launch_bounds__(128, 3) k_lin_ma_mixed_cols(MixedLinArgs a) {
+  constexpr int D = 16, LPR = D / 2;
   extern __shared__ __align__(16) unsigned char mix_smem[];
   MixNet<D>& W = reinterpret_cast<MixNet<D>*>(mix_smem)[threadIdx.x >> 5];
   MixRow<D>& S =
@@ -632,13 +640,103 @@ __global__ void __launch_bounds__(128, D == 16 ? 3 : 2) k_lin_ma_mixed(MixedLinA
   if (cur >= 0) acc_resid_group<32>(a.acc, cur, mx, sq, key, l32, 0xffffffffu);
 }
 
-template <int D, bool RK4>
+// ---- linearisation, d = 32: a lane per species -------------------------------------------
+// Two columns of K and of their sum take 128 registers at d = 32, which spills (255 registers,
+// 1124 bytes): 0.8 M rows, 48 reactions take 7.2 ms that way and 6.7 with a lane per species,
+// evaluated in float64 8.1 and 7.0. A warp walks kMixLaneRows consecutive rows: reactions, rate constants and lists are loaded once
+// per warp and sequence, and the residual statistics flushed once.
+constexpr int kMixLaneRows = 8;
+
+template <int D>
+struct MixLane {  // one per warp
+  // rows padded to D + 4 floats: 16-byte row accesses of eight lanes fall in distinct banks
+  float G[D][D + 4], K[D][D + 4];
+  double rate[kMixReact];               // floats use the first half in float32 mode
+  float d1[kMixReact], d2[kMixReact];   // d rate / d c_i1, d c_i2
+  uint32_t list[kMixList * D];
+};
+
+template <bool RK4>
+__global__ void __launch_bounds__(128) k_lin_ma_mixed_lane(MixedLinArgs a) {
+  constexpr int D = 32, RPL = kMixReact / D;  // reactions per lane
+  extern __shared__ __align__(16) unsigned char mix_smem[];
+  MixLane<D>& S = reinterpret_cast<MixLane<D>*>(mix_smem)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  constexpr unsigned gm = 0xffffffffu;
+  const int64_t rows = a.bt.act_rows();
+  const int64_t lo = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * kMixLaneRows;
+  const int R = a.dv.R < kMixReact ? a.dv.R : kMixReact;
+  int64_t cur = -1;
+  const int4* tt = nullptr;
+  const int32_t* ae = nullptr;
+  int e0 = 0, e1 = 0;
+  int4 q[RPL];
+  double kd[RPL];
+  float kf[RPL];
+  bool fast = true;
+  float mx = 0.f, sq = 0.f;
+  unsigned long long key = 0ull;  // first failing row (sliding window)
+  for (int64_t pos = lo; pos < lo + kMixLaneRows && pos < rows; ++pos) {  // uniform over the warp
+    int64_t seq, row;
+    act_row(a.bt, pos, seq, row);
+    if (seq != cur) {
+      if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
+      cur = seq;
+      mx = 0.f;
+      sq = 0.f;
+      key = 0ull;
+      const double* kk = a.dv.params + seq * a.dv.pstride;
+      tt = reinterpret_cast<const int4*>(a.dv.topo + seq * a.dv.tstride);
+      const int32_t* aoff = a.adj_off + (a.adj_stride ? seq : 0) * (D + 1);
+      ae = a.adj_e + (a.adj_stride ? seq : 0) * a.adj_stride;
+      e0 = __ldg(aoff + lane);
+      e1 = __ldg(aoff + lane + 1);
+      mixed_list<D>(S.list, lane, tt, ae, e0, e1);  // (each lane reads only its own column)
+#pragma unroll
+      for (int k = 0; k < RPL; ++k) {
+        const int r = k * D + lane;
+        q[k] = __ldg(tt + (r < R ? r : 0));
+        kd[k] = r < R ? __ldg(kk + r) : 0.0;
+        kf[k] = d2f_trunc(kd[k]);
+      }
+      fast = a.it == 0 || a.info[seq].max_resid > kMixedFastAbove;
+    }
+    const double sp = row == __ldg(a.bt.offsets + seq) ? a.s0[seq * D + lane]
+                                                      : a.s[(row - 1) * D + lane];
+    const double sc = a.s[row * D + lane];
+    __nv_bfloat16* Eo = a.E + row * (int64_t)(D * D);
+    float* bo = a.b + row * D;
+    if (fast)
+      mixed_row<float, D, RK4, RPL>(a, true, row, lane, gm, sp, sc, q, kd, kf, R, tt, ae, e0, e1,
+                                    S.list, S.G, S.K, reinterpret_cast<float*>(S.rate), S.d1,
+                                    S.d2, mx, sq, seq, key, bo, Eo);
+    else
+      mixed_row<double, D, RK4, RPL>(a, true, row, lane, gm, sp, sc, q, kd, kf, R, tt, ae, e0, e1,
+                                     S.list, S.G, S.K, S.rate, S.d1, S.d2, mx, sq, seq, key, bo,
+                                     Eo);
+  }
+  if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
+}
+
+template <bool RK4>
 static cudaError_t lin_mixed_launch(const MixedLinArgs& a, cudaStream_t st) {
-  auto kern = k_lin_ma_mixed<D, RK4>;
-  static DeviceOnce configured;
-  const cudaError_t e = allow_smem(configured, kern, kMixSmem<D>);
-  if (e != cudaSuccess) return e;
-  kern<<<grid_for(a.bt.act_rows(), 4 * kMixRows), 128, kMixSmem<D>, st>>>(a);
+  static DeviceOnce cols, lanes;
+  cudaError_t e;
+  if (a.dv.d == 16) {
+    constexpr size_t smem = kMixSmem<16>;
+    e = allow_smem(cols, k_lin_ma_mixed_cols<RK4>, smem);
+    if (e != cudaSuccess) return e;
+    k_lin_ma_mixed_cols<RK4>
+        <<<grid_for(a.bt.act_rows(), 4 * kMixRows), 128, smem, st>>>(a);
+  } else if (a.dv.d == 32) {
+    constexpr size_t smem = 4 * sizeof(MixLane<32>);
+    e = allow_smem(lanes, k_lin_ma_mixed_lane<RK4>, smem);
+    if (e != cudaSuccess) return e;
+    k_lin_ma_mixed_lane<RK4>
+        <<<grid_for(a.bt.act_rows(), 4 * kMixLaneRows), 128, smem, st>>>(a);
+  } else {
+    return cudaErrorInvalidValue;
+  }
   note_launch();
   return cudaGetLastError();
 }
@@ -1119,13 +1217,8 @@ cudaError_t launch_mixed_apply_rc(const MixedRcArgs& a, const MixedScanArgs& car
 
 cudaError_t launch_lin_ma_mixed(const MixedLinArgs& a, cudaStream_t st) {
   if (a.bt.act_rows() == 0) return cudaSuccess;
-  const bool rk4 = a.dv.kind == DEER_F_MASSACTION_RK4;
-  const int d = a.dv.d;
-  if (d == 16)
-    return rk4 ? lin_mixed_launch<16, true>(a, st) : lin_mixed_launch<16, false>(a, st);
-  if (d == 32)
-    return rk4 ? lin_mixed_launch<32, true>(a, st) : lin_mixed_launch<32, false>(a, st);
-  return cudaErrorInvalidValue;
+  return a.dv.kind == DEER_F_MASSACTION_RK4 ? lin_mixed_launch<true>(a, st)
+                                            : lin_mixed_launch<false>(a, st);
 }
 
 template <int D>
