@@ -793,7 +793,6 @@ static cudaError_t mixed_carry(const MixedScanArgs& m, cudaStream_t st) {
   a.aggP = m.aggP;
   a.aggv = m.aggv;
   a.cin = m.cin;
-  a.tensor_cores = 1;
   a.segP = m.segP;
   a.segv = m.segv;
   a.segin = m.segin;

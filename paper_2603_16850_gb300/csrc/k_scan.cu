@@ -878,7 +878,6 @@ __global__ void __launch_bounds__(128) k_dense_chunk_ring4(DenseScanArgs<real> a
 // the 32 lanes' words fall in distinct banks). The vector part v <- A_t v + b_t is formed
 // by lane i (row i) of warp 0. Rows are staged through the same cp.async ring as
 // k_dense_chunk_ring4.
-template <bool SEG>
 __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a) {
   constexpr int D = 32;
   constexpr int K = ring_depth<float>();
@@ -889,10 +888,10 @@ __global__ void __launch_bounds__(64) k_dense_chunk_mma32(DenseScanArgs<float> a
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tq = lane & 3;
   Span p;
-  if (!get_span<SEG>(a, blockIdx.x, p)) return;  // uniform over the block
+  if (!get_span<false>(a, blockIdx.x, p)) return;  // uniform over the block
   const float *A0, *b0;
   float *Po, *vo;
-  span_ptrs<SEG, float, D>(a, p, A0, b0, Po, vo);
+  span_ptrs<false, float, D>(a, p, A0, b0, Po, vo);
   const int n = p.n;
   const bool need_P = p.need_P;
   auto issue = [&](int slot, int t) {
@@ -1047,7 +1046,8 @@ __device__ __forceinline__ int64_t carry_walk(RowRing<real, D>& R, const real* P
 // chunks of the mean-field RNN, d = 32, T = 100000: 580 us); the chunks are then folded into
 // segments of M (the chunk pass again, over the aggregates), MODE 1 walks a sequence's
 // segments, MODE 2 the chunks of each segment from the value entering it: 39 + 20 + 10 us
-// there. (Mixed-precision ragged batch, d = 16, up to 3125 chunks a sequence: 134 -> 27 ms of
+// there. The folds are float32 multiply-adds, as the walk over the chunks is, also where the
+// chunk pass uses the tensor cores. (Mixed-precision ragged batch, d = 16, up to 3125 chunks a sequence: 134 -> 27 ms of
 // scans per solve, against a carry that loaded each aggregate when it needed it.)
 // A product over a segment (up to 64 chunks) can overflow where those over its chunks do not,
 // and inf times a Delta of zero would then spread NaN over rows that are solved already: MODE
@@ -1227,9 +1227,9 @@ static void dense_chunk_launch(const DenseScanArgs<real>& a, int64_t spans, unsi
   constexpr int G = D == 32 ? 1 : 32 / group_lanes<D>();
   const dim3 g(grid_for(spans, G), ny);
   if constexpr (D == 32) {
-    if constexpr (sizeof(real) == 4) {
+    if constexpr (sizeof(real) == 4 && !SEG) {
       if (a.tensor_cores) {
-        k_dense_chunk_mma32<SEG><<<g, 64, 0, st>>>(a);
+        k_dense_chunk_mma32<<<g, 64, 0, st>>>(a);
         return;
       }
     }
