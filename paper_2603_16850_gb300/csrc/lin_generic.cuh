@@ -42,7 +42,7 @@ __device__ __forceinline__ void store_row(real* __restrict__ p, const real* v) {
 }
 
 // ----------------------------------------------------------------------------
-// Initial guess
+// Initial guess (zeros are a memset, launch_init)
 // ----------------------------------------------------------------------------
 template <class real, int D, int KIND>
 __global__ void __launch_bounds__(128) k_init(InitArgs<real> a) {
@@ -50,10 +50,7 @@ __global__ void __launch_bounds__(128) k_init(InitArgs<real> a) {
   if (row >= a.bt.N) return;
   const int64_t seq = find_seq(a.bt.offsets, a.bt.B, row);
   real v[D];
-  if (a.init == DEER_INIT_ZEROS) {
-#pragma unroll Unroll<D>::n
-    for (int i = 0; i < D; ++i) v[i] = real(0);
-  } else if (a.init == DEER_INIT_S0) {
+  if (a.init == DEER_INIT_S0) {
 #pragma unroll Unroll<D>::n
     for (int i = 0; i < D; ++i) v[i] = a.s0[seq * D + i];
   } else {  // Jacobi: f_t(0)
