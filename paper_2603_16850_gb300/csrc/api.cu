@@ -141,8 +141,8 @@ static bool use_compensated(const deer_dynamics* f, const deer_options* o) {
 // Default chunk of the full Jacobian at d < 16: kLongChunk rows, fewer while the lanes (d per
 // chunk) of a whole problem stay below a bound.
 constexpr int kLongChunk = 64;
-constexpr int64_t kFewLanes = 152 * 4 * 32;       // four warps per SM
-constexpr int64_t kFewLanesF64 = 608 * 4 * 32;    // four warps per scheduler
+constexpr int64_t kFewLanes = kSMs * 4 * 32;       // four warps per SM
+constexpr int64_t kFewLanesF64 = kSchedulers * 4 * 32;    // four warps per scheduler
 
 // The caller leaves the chunk length to the rule on sizes (`lean`: see make_layout).
 static bool chunk_by_size(const deer_options* o, int d, bool lean) {

@@ -8,6 +8,11 @@
 
 namespace deer {
 
+// The GPU: streaming multiprocessors and warp schedulers (rules of thumb on sizes; a grid that
+// must fit the device asks it)
+constexpr int kSMs = 152;
+constexpr int kSchedulers = 4 * kSMs;
+
 // ---------------------------------------------------------------------------
 // Per-sequence solver state kept in the workspace.
 // ---------------------------------------------------------------------------

@@ -416,7 +416,7 @@ cudaError_t launch_init(const InitArgs<real>& a, cudaStream_t st) {
   if (a.init == DEER_INIT_RANDN) {
     const int64_t n = a.bt.N * a.dv.d;
     int64_t g = (n + 255) / 256;
-    if (g > 152 * 32) g = 152 * 32;
+    if (g > kSMs * 32) g = kSMs * 32;
     k_init_randn<real><<<(unsigned)g, 256, 0, st>>>(a.s, n, a.seed);
     note_launch();
     return cudaGetLastError();

@@ -246,7 +246,7 @@ cudaError_t launch_ma_param_grad(const MaGradArgs<real>& a, cudaStream_t st) {
   // 64 rows per group (the reaction lists are built once per group), fewer while the batch
   // leaves the GPU short of eight warps per SM
   b.rows = 64;
-  while (b.rows > 8 && a.B * a.T / b.rows * a.dv.d < 152 * 8 * 32) b.rows /= 2;
+  while (b.rows > 8 && a.B * a.T / b.rows * a.dv.d < kSMs * 8 * 32) b.rows /= 2;
   switch (a.dv.d) {
     case 16: return param_grad_rounds<real, 16>(b, st);
     case 32: return param_grad_rounds<real, 32>(b, st);

@@ -1216,7 +1216,7 @@ template <class real, int D>
 static void set_segments(DenseScanArgs<real>& a) {
   a.log2M = 0;
   const int64_t n = a.max_chunks;
-  if (!a.segP || n < 128 || a.bt.B > 608 * (32 / group_lanes<D>())) return;
+  if (!a.segP || n < 128 || a.bt.B > kSchedulers * (32 / group_lanes<D>())) return;
   a.log2M = 3;
   while (a.log2M < 6 && ((int64_t)1 << (2 * a.log2M + 2)) <= n) ++a.log2M;
 }
@@ -1237,7 +1237,7 @@ static void dense_chunk_launch(const DenseScanArgs<real>& a, int64_t spans, unsi
   } else {
     if constexpr (sizeof(real) == 8 && D >= 4 && D <= 8) {
       // warps per sub-partition x instructions per row: entries against whole groups
-      const int64_t warps = (spans * ny + 607) / 608;
+      const int64_t warps = (spans * ny + kSchedulers - 1) / kSchedulers;
       if (warps * (D == 8 ? 3 : 1) < D + 1) {
         k_dense_chunk_entry<D, SEG><<<dim3((unsigned)spans, ny), 32, 0, st>>>(a);
         return;
