@@ -1076,15 +1076,29 @@ __global__ void __launch_bounds__(32) k_dense_carry_ring(DenseScanArgs<real> a) 
       const int64_t s0 = (a.bt.chunk_first[seq] >> a.log2M) + seq;
       const int64_t s1 = s0 + ((c1 - c0 + M - 1) >> a.log2M);
       carry_walk<false, real, D>(R, a.segP, a.segv, a.segin, s0, s1, true, x);
-      // (a non-finite entry makes every entry after it non-finite: only the end is looked at)
-      if (!__any_sync(group_mask<D>(), mag_bits(x) >= mag_bits(real(INFINITY)))) return;
-      x = real(0);
-      for (int64_t k = s0; k < s1; ++k) {
-        k = carry_walk<true, real, D>(R, a.segP, a.segv, a.segin, k, s1, k == s0, x);
-        if (k == s1) break;
+      const unsigned gm = group_mask<D>();
+      auto nonfinite = [&](real y) {
+        return __any_sync(gm, mag_bits(y) >= mag_bits(real(INFINITY))) != 0;
+      };
+      // a non-finite entry makes every value after it non-finite: only the end is looked at
+      if (!nonfinite(x)) return;
+      // the first segment that leaves x non-finite, by bisection over the values stored
+      const int li = lane < D ? lane : 0;
+      int64_t k = s0, end = s1;
+      while (end - k > 1) {
+        const int64_t mid = k + (end - k) / 2;
+        if (nonfinite(a.segin[mid * D + li])) end = mid;
+        else k = mid;
+      }
+      x = a.segin[k * D + li];
+      for (;;) {
         const int64_t q0 = c0 + (k - s0) * M;
         carry_walk<false, real, D>(R, a.aggP, a.aggv, nullptr, q0, q0 + M < c1 ? q0 + M : c1,
                                    k == s0, x);
+        // (non-finite chunk by chunk too: the values stored stand)
+        if (++k >= s1 || nonfinite(x)) return;
+        k = carry_walk<true, real, D>(R, a.segP, a.segv, a.segin, k, s1, false, x);
+        if (k == s1) return;
       }
     }
   }

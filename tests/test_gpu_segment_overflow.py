@@ -66,3 +66,32 @@ def test_solution_as_guess(d, prec, growth, reset):
                               init="zeros", reset=reset)
     assert info.iters.tolist() == [1] and bool(info.converged.all()), info
     assert not bool(s.any())
+
+
+@pytest.mark.parametrize("d", [16, 32])
+@pytest.mark.parametrize("prec,limit", [("fp32", 1e18), ("fp64", 1e30)])
+def test_correction_that_overflows_itself(d, prec, limit):
+    """s_t = 2 s_{t-1} from the zero guess: the one step's correction is 2^t, exact until it
+    overflows; entries above the reset threshold, and all from the overflow on, end at zero. A
+    sequence beside it is solved as ever."""
+    import paper_2603_16850_gb300 as deer
+    dt = torch.float32 if prec == "fp32" else torch.float64
+    T = 8192
+    A = torch.diag(torch.tensor([2.0] + [0.5] * (d - 1), dtype=dt, device="cuda"))
+    s0 = torch.zeros(2, d, dtype=dt, device="cuda")
+    s0[0, 0] = s0[0, 1] = s0[1, 1] = 1.0
+    s, _ = deer.deer_solve(deer.Dynamics.linear(A), s0, T, jac="full", tol=0.0, max_iters=1,
+                           prec=prec, init="zeros", reset=True, chunk=32)
+    got = s.double().cpu().numpy().reshape(2, T, d)
+    t = np.arange(1, T + 1, dtype=np.float64)
+    over = 128 if prec == "fp32" else 1024  # 2^t is not a number of the type from here on
+    with np.errstate(over="ignore", under="ignore"):
+        up, down = np.exp2(t), np.exp2(-t)
+    assert np.array_equal(got[0, :, 0], np.where(up <= limit, up, 0.0))
+    assert np.all(got[:, :, 2:] == 0.0) and np.all(got[1, :, 0] == 0.0)
+    # float32 subnormals and below: not more than the smallest normal number away
+    tiny = 1.2e-38 if prec == "fp32" else 2.3e-308
+    assert np.all(np.abs(got[1, :, 1] - down) <= tiny)
+    # the coordinate beside the growing one: solved before the overflow, zero after it
+    assert np.all(np.abs(got[0, :over - 1, 1] - down[:over - 1]) <= tiny)
+    assert np.all(got[0, over:, 1] == 0.0)
