@@ -534,9 +534,22 @@ DEER_INST(double)
 
 namespace deer {
 
-// consecutive rows per lane group in k_lin_ma_wide: the reaction lists are built once per
-// group and sequence
-constexpr int kMaRows = 8;
+// Consecutive rows per lane group in k_lin_ma_wide (ROWS): the reaction lists are built once per
+// group and sequence, so eight rows where a batch fills the GPU, and two where it does not and a
+// pass waits for one group's chain. Six iterations with two and with eight rows per group, ms:
+// full Jacobian, RK4, d = 32, float32 300 rows 0.78 / 1.12, 10000 1.40 / 1.60, 40000 3.27 / 3.42,
+// 160000 10.65 / 10.26; float64 300 rows 4.7 / 10.3, 40000 73.2 / 78.3, 160000 275.9 / 275.9;
+// diagonal, Euler, d = 16, float32 5000 rows 0.46 / 0.51, 20000 0.61 / 0.55; diagonal, RK4, d = 16,
+// float32 5000 rows 0.61 / 0.70, 20000 0.95 / 0.91. (A row count read at run time costs the
+// float32 d = 16 forms a block per SM: 128000 rows 2.5 -> 3.1 ms.)
+constexpr int kMaRows = 8, kMaRowsFew = 2;
+
+// the rows from which groups walk kMaRows
+static int64_t ma_many_rows(bool f64, int d, bool rk4, int jac) {
+  if (f64) return rk4 ? 160000 : 60000;
+  if (!rk4 || (d == 16 && jac != DEER_JAC_FULL)) return 12000;
+  return 64000;
+}
 constexpr int kMaList = 16;  // entries of a species' list held in shared memory
 
 // products and sums that must not be contracted into one rounding
@@ -569,7 +582,7 @@ struct MaListSmem {
 // and the concentrations are read directly, with the same products and sums: 2.1 M rows, d = 32,
 // 48 reactions 15.0 -> 12.9 ms.
 // ----------------------------------------------------------------------------
-template <class real, int D, bool RK4, int JAC>
+template <class real, int D, bool RK4, int JAC, int ROWS>
 __global__ void __launch_bounds__(128, (D == 32 && sizeof(real) == 4) ? 4 : 1)
     k_lin_ma_wide(LinArgs<real> a) {
   constexpr int GROUPS = 128 / D;          // rows per block
@@ -600,14 +613,14 @@ __global__ void __launch_bounds__(128, (D == 32 && sizeof(real) == 4) ? 4 : 1)
   const bool use_adj = a.adj_off != nullptr;
   int n_list = 0, most = 0;  // entries of this species, most of any of the group's
   if (lane == 0) sC[grp][D] = real(1);
-  // each group walks kMaRows consecutive active rows and flushes the residual statistics
+  // each group walks ROWS consecutive active rows and flushes the residual statistics
   // once per sequence it meets (not once per row): fewer atomics on the accumulator of a
   // long sequence
-  const int64_t ar0 = (blockIdx.x * (int64_t)GROUPS + grp) * kMaRows;
+  const int64_t ar0 = (blockIdx.x * (int64_t)GROUPS + grp) * ROWS;
   int64_t cur = -1;
   real mx = real(0), sq = real(0);
   unsigned long long key = 0ull;  // first failing row (sliding window)
-  for (int ri = 0; ri < kMaRows; ++ri) {
+  for (int ri = 0; ri < ROWS; ++ri) {
     const int64_t ar = ar0 + ri;
     if (ar >= a.bt.act_rows()) break;  // uniform over the group
     int64_t seq, row;
@@ -1000,30 +1013,36 @@ __global__ void __launch_bounds__(128, (D == 32 && sizeof(real) == 4) ? 4 : 1)
   if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gmask);
 }
 
-template <class real, int D, bool RK4, int JAC>
-static cudaError_t lin_ma_wide_launch(const LinArgs<real>& a, unsigned g, cudaStream_t st) {
+template <class real, int D, bool RK4, int JAC, int ROWS>
+static cudaError_t lin_ma_wide_rows(const LinArgs<real>& a, cudaStream_t st) {
   const size_t smem = sizeof(MaListSmem<real, D>);
   static DeviceOnce configured;
-  const cudaError_t e = allow_smem(configured, k_lin_ma_wide<real, D, RK4, JAC>, smem);
+  const cudaError_t e = allow_smem(configured, k_lin_ma_wide<real, D, RK4, JAC, ROWS>, smem);
   if (e != cudaSuccess) return e;
-  k_lin_ma_wide<real, D, RK4, JAC><<<g, 128, smem, st>>>(a);
+  const unsigned g = grid_for(a.bt.act_rows(), 128 / D * ROWS);
+  k_lin_ma_wide<real, D, RK4, JAC, ROWS><<<g, 128, smem, st>>>(a);
   note_launch();
   return cudaGetLastError();
+}
+
+template <class real, int D, bool RK4, int JAC>
+static cudaError_t lin_ma_wide_launch(const LinArgs<real>& a, cudaStream_t st) {
+  return a.bt.act_rows() < ma_many_rows(sizeof(real) == 8, D, RK4, JAC)
+             ? lin_ma_wide_rows<real, D, RK4, JAC, kMaRowsFew>(a, st)
+             : lin_ma_wide_rows<real, D, RK4, JAC, kMaRows>(a, st);
 }
 
 template <class real, int JAC>
 cudaError_t launch_lin_ma_wide(const LinArgs<real>& a, cudaStream_t st) {
   const bool rk4 = a.dv.kind == DEER_F_MASSACTION_RK4;
   const int d = a.dv.d;
-  const int64_t rows_per_block = 128 / d * kMaRows;
-  const unsigned g = grid_for(a.bt.act_rows(), (int)rows_per_block);
   if (d == 16) {
-    if (rk4) return lin_ma_wide_launch<real, 16, true, JAC>(a, g, st);
-    return lin_ma_wide_launch<real, 16, false, JAC>(a, g, st);
+    if (rk4) return lin_ma_wide_launch<real, 16, true, JAC>(a, st);
+    return lin_ma_wide_launch<real, 16, false, JAC>(a, st);
   }
   if (d == 32) {
-    if (rk4) return lin_ma_wide_launch<real, 32, true, JAC>(a, g, st);
-    return lin_ma_wide_launch<real, 32, false, JAC>(a, g, st);
+    if (rk4) return lin_ma_wide_launch<real, 32, true, JAC>(a, st);
+    return lin_ma_wide_launch<real, 32, false, JAC>(a, st);
   }
   return cudaErrorInvalidValue;
 }

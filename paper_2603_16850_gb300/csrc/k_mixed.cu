@@ -640,31 +640,39 @@ __global__ void __launch_bounds__(128, 3) k_lin_ma_mixed_cols(MixedLinArgs a) {
   if (cur >= 0) acc_resid_group<32>(a.acc, cur, mx, sq, key, l32, 0xffffffffu);
 }
 
-// ---- linearisation, d = 32: a lane per species -------------------------------------------
+// ---- linearisation, d = 32 and few rows: a lane per species -------------------------------
+// d = 16 takes two columns per lane from kMixColsRows rows on: its lists cost more to build and its
+// warps hold 32 rows, which fewer rows do not pay for. Six iterations, 24 reactions, a lane per
+// species against two columns: 300 rows 0.61 / 1.10 ms, 10000 rows 0.95 / 1.30, 80000 rows 2.30 /
+// 2.47, 160000 rows 3.94 / 3.49 (64 reactions: 0.69 / 1.56, 1.20 / 1.75, 3.37 / 3.85, 5.98 / 5.27).
+constexpr int64_t kMixColsRows = 1 << 17;
+
 // Two columns of K and of their sum take 128 registers at d = 32, which spills (255 registers,
 // 1124 bytes): 0.8 M rows, 48 reactions take 7.2 ms that way and 6.7 with a lane per species,
-// evaluated in float64 8.1 and 7.0. A warp walks kMixLaneRows consecutive rows: reactions, rate constants and lists are loaded once
-// per warp and sequence, and the residual statistics flushed once.
+// evaluated in float64 8.1 and 7.0. A group walks up to kMixLaneRows consecutive rows: reactions,
+// rate constants and lists are loaded once per group and sequence, and the residual statistics
+// flushed once.
 constexpr int kMixLaneRows = 8;
 
 template <int D>
-struct MixLane {  // one per warp
+struct MixLane {  // one per group
   // rows padded to D + 4 floats: 16-byte row accesses of eight lanes fall in distinct banks
   float G[D][D + 4], K[D][D + 4];
   double rate[kMixReact];               // floats use the first half in float32 mode
   float d1[kMixReact], d2[kMixReact];   // d rate / d c_i1, d c_i2
   uint32_t list[kMixList * D];
+  float pad[D == 16 ? 16 : 4];          // the two groups of a warp in different banks
 };
 
-template <bool RK4>
-__global__ void __launch_bounds__(128) k_lin_ma_mixed_lane(MixedLinArgs a) {
-  constexpr int D = 32, RPL = kMixReact / D;  // reactions per lane
+template <int D, bool RK4>
+__global__ void __launch_bounds__(128) k_lin_ma_mixed_lane(MixedLinArgs a, int per) {
+  constexpr int RPL = kMixReact / D;  // reactions per lane
   extern __shared__ __align__(16) unsigned char mix_smem[];
-  MixLane<D>& S = reinterpret_cast<MixLane<D>*>(mix_smem)[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  constexpr unsigned gm = 0xffffffffu;
+  MixLane<D>& S = reinterpret_cast<MixLane<D>*>(mix_smem)[threadIdx.x / D];
+  const int lane = threadIdx.x % D;
+  const unsigned gm = gmask_mixed<D>();
   const int64_t rows = a.bt.act_rows();
-  const int64_t lo = (blockIdx.x * 4ll + (threadIdx.x >> 5)) * kMixLaneRows;
+  const int64_t lo = (blockIdx.x * (int64_t)(128 / D) + threadIdx.x / D) * per;
   const int R = a.dv.R < kMixReact ? a.dv.R : kMixReact;
   int64_t cur = -1;
   const int4* tt = nullptr;
@@ -676,7 +684,7 @@ __global__ void __launch_bounds__(128) k_lin_ma_mixed_lane(MixedLinArgs a) {
   bool fast = true;
   float mx = 0.f, sq = 0.f;
   unsigned long long key = 0ull;  // first failing row (sliding window)
-  for (int64_t pos = lo; pos < lo + kMixLaneRows && pos < rows; ++pos) {  // uniform over the warp
+  for (int64_t pos = lo; pos < lo + per && pos < rows; ++pos) {  // uniform over the group
     int64_t seq, row;
     act_row(a.bt, pos, seq, row);
     if (seq != cur) {
@@ -718,22 +726,38 @@ __global__ void __launch_bounds__(128) k_lin_ma_mixed_lane(MixedLinArgs a) {
   if (cur >= 0) acc_resid_group<D>(a.acc, cur, mx, sq, key, lane, gm);
 }
 
+// Rows per group of d lanes: kMixLaneRows, fewer while the groups are less than 16 warps per
+// scheduler, where a pass waits for one group's chain. Six iterations with 1, 2, 4, 8 rows, d = 32:
+// 300 rows 1.87, 1.92, 2.07, 2.36 ms; 40000 rows 6.1, 6.0, 6.1, 6.1; 320000 rows 39.6, 37.9, 37.1,
+// 36.6.
+static int mix_lane_rows(int64_t rows, int d) {
+  int n = kMixLaneRows;
+  while (n > 1 && rows / n * d < (int64_t)kSchedulers * 32 * 16) n /= 2;
+  return n;
+}
+
 template <bool RK4>
 static cudaError_t lin_mixed_launch(const MixedLinArgs& a, cudaStream_t st) {
-  static DeviceOnce cols, lanes;
+  static DeviceOnce cols, lane16, lane32;
+  const int64_t rows = a.bt.act_rows();
   cudaError_t e;
-  if (a.dv.d == 16) {
+  if (a.dv.d == 16 && rows >= kMixColsRows) {
     constexpr size_t smem = kMixSmem<16>;
     e = allow_smem(cols, k_lin_ma_mixed_cols<RK4>, smem);
     if (e != cudaSuccess) return e;
-    k_lin_ma_mixed_cols<RK4>
-        <<<grid_for(a.bt.act_rows(), 4 * kMixRows), 128, smem, st>>>(a);
+    k_lin_ma_mixed_cols<RK4><<<grid_for(rows, 4 * kMixRows), 128, smem, st>>>(a);
+  } else if (a.dv.d == 16) {
+    constexpr size_t smem = 8 * sizeof(MixLane<16>);
+    e = allow_smem(lane16, k_lin_ma_mixed_lane<16, RK4>, smem);
+    if (e != cudaSuccess) return e;
+    const int per = mix_lane_rows(rows, 16);
+    k_lin_ma_mixed_lane<16, RK4><<<grid_for(rows, 8 * per), 128, smem, st>>>(a, per);
   } else if (a.dv.d == 32) {
     constexpr size_t smem = 4 * sizeof(MixLane<32>);
-    e = allow_smem(lanes, k_lin_ma_mixed_lane<RK4>, smem);
+    e = allow_smem(lane32, k_lin_ma_mixed_lane<32, RK4>, smem);
     if (e != cudaSuccess) return e;
-    k_lin_ma_mixed_lane<RK4>
-        <<<grid_for(a.bt.act_rows(), 4 * kMixLaneRows), 128, smem, st>>>(a);
+    const int per = mix_lane_rows(rows, 32);
+    k_lin_ma_mixed_lane<32, RK4><<<grid_for(rows, 4 * per), 128, smem, st>>>(a, per);
   } else {
     return cudaErrorInvalidValue;
   }
