@@ -1598,15 +1598,84 @@ __global__ void __launch_bounds__(32) k_adj_apply_ring(AdjScanArgs<real> a) {
   cp_async_wait<0>();
 }
 
+// d = 1: one thread per chunk (per sequence in the carry pass), as in the forward scan: groups of
+// one lane staged through rings took 1.1 to 1.4 times as long (1 x 5000 rows, float32: a gradient
+// call 0.205 ms against 0.147).
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_adj_chunk(AdjScanArgs<real> a) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= a.bt.n_chunks) return;
+  int64_t seq, r0;
+  int n;
+  chunk_rows(a.bt, c, seq, r0, n);
+  const int64_t rend = __ldg(a.bt.offsets + seq + 1);  // one past the last row
+  real P = real(1), v = real(0);
+  for (int64_t row = r0 + n - 1; row >= r0; --row) {
+    // (the last row of the sequence drops the carry, lambda_{T+1} = 0)
+    const real An = row + 1 < rend ? __ldg(a.A + row + 1) : real(0);
+    v = row + 1 < rend ? An * v + __ldg(a.g + row) : __ldg(a.g + row);
+    P = An * P;
+  }
+  a.aggP[c] = P;
+  a.aggv[c] = v;
+}
+
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_adj_carry(AdjScanArgs<real> a) {
+  const int64_t seq = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (seq >= a.bt.B) return;
+  const int64_t c0 = a.bt.chunk_first[seq];
+  real x = real(0);
+  // (loads of kCarry aggregates at a time: they do not depend on x)
+  for (int64_t cb = a.bt.chunk_first[seq + 1] - 1; cb >= c0; cb -= kCarry) {
+    real P[kCarry], v[kCarry];
+#pragma unroll
+    for (int k = 0; k < kCarry; ++k) {
+      const int64_t c = cb - k >= c0 ? cb - k : c0;
+      P[k] = a.aggP[c];
+      v[k] = a.aggv[c];
+    }
+#pragma unroll
+    for (int k = 0; k < kCarry; ++k) {
+      if (cb - k < c0) break;
+      a.cin[cb - k] = x;
+      x = P[k] * x + v[k];
+    }
+  }
+}
+
+template <class real>
+__global__ void __launch_bounds__(128) k_scalar_adj_apply(AdjScanArgs<real> a) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= a.bt.n_chunks) return;
+  int64_t seq, r0;
+  int n;
+  chunk_rows(a.bt, c, seq, r0, n);
+  const int64_t rend = __ldg(a.bt.offsets + seq + 1);
+  real x = a.cin[c];
+  for (int64_t row = r0 + n - 1; row >= r0; --row) {
+    x = row + 1 < rend ? __ldg(a.A + row + 1) * x + __ldg(a.g + row) : __ldg(a.g + row);
+    a.lam[row] = x;
+  }
+}
+
 template <class real, int D>
 static void adj_launch(const AdjScanArgs<real>& a, cudaStream_t st) {
-  constexpr int G = 32 / group_lanes<D>();
-  const unsigned gc = grid_for(a.bt.n_chunks, G);
-  if constexpr (D == 32 && sizeof(real) == 4) k_adj_chunk_tile32<<<gc, 32, 0, st>>>(a);
-  else k_adj_chunk_ring<real, D><<<gc, 32, 0, st>>>(a);
-  k_adj_carry_ring<real, D><<<grid_for(a.bt.B, G), 32, 0, st>>>(a);
-  k_adj_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
-  note_launch(3);
+  if constexpr (D == 1) {
+    const unsigned gc = grid_for(a.bt.n_chunks, 128);
+    k_scalar_adj_chunk<real><<<gc, 128, 0, st>>>(a);
+    k_scalar_adj_carry<real><<<grid_for(a.bt.B, 128), 128, 0, st>>>(a);
+    k_scalar_adj_apply<real><<<gc, 128, 0, st>>>(a);
+    note_launch(3);
+  } else {
+    constexpr int G = 32 / group_lanes<D>();
+    const unsigned gc = grid_for(a.bt.n_chunks, G);
+    if constexpr (D == 32 && sizeof(real) == 4) k_adj_chunk_tile32<<<gc, 32, 0, st>>>(a);
+    else k_adj_chunk_ring<real, D><<<gc, 32, 0, st>>>(a);
+    k_adj_carry_ring<real, D><<<grid_for(a.bt.B, G), 32, 0, st>>>(a);
+    k_adj_apply_ring<real, D><<<gc, 32, 0, st>>>(a);
+    note_launch(3);
+  }
 }
 
 template <class real>
