@@ -51,16 +51,18 @@ __device__ __forceinline__ float half_ulp(float t) {
   return e > 24 ? __int_as_float((e - 24) << 23) : 0.f;
 }
 
-// !(|r| / |s| <= tol) as the division rounds, for |s| > 1 and tol >= 0, without dividing: the
-// quotient rounds to tol or below exactly when |r| <= |s| (tol + half an ulp) (no quotient lies
-// on that midpoint). More than two ulps from tol |s| the bit patterns decide.
+// !(|r| / max(1, |s|) <= tol) as the division rounds, for tol >= 0, without dividing: the quotient
+// rounds to tol or below exactly when |r| <= |s| (tol + half an ulp) (no quotient lies on that
+// midpoint).
 template <class real>
 __device__ __forceinline__ bool over_tol(real r, real s, real tol) {
-  const real lim = tol * rabs(s);
-  const auto rb = mag_bits(r), lb = mag_bits(lim);
-  if (rb - lb + 2u <= 4u) return fma(-tol, rabs(s), rabs(r)) > rabs(s) * half_ulp(tol);
-  return rb > lb;
+  if (!(rabs(s) > real(1))) return rabs(r) > tol;
+  return fma(-tol, rabs(s), rabs(r)) > rabs(s) * half_ulp(tol);
 }
+
+// the leading 32 bits of |x|
+__device__ __forceinline__ unsigned mag_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned mag_hi(float x) { return mag_bits(x); }
 
 template <class real, int D>
 struct Aff {  // the affine map Delta -> P Delta + v
@@ -245,7 +247,7 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
     }
     // 1. linearise, test, this thread's element; F and A are kept for the apply pass
     Aff<real, D> e = aff_identity<real, D>();
-    bool fail = !tol_met, bad = false;
+    bool fail = !tol_met, bad = false, near = false;
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       if (k < nmine) {
@@ -255,9 +257,13 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
         for (int i = 0; i < D; ++i) {
           const real r = s[k][i] - Fk[k][i];
           st.v[i] = -r;
-          const auto rb = mag_bits(r), sb = mag_bits(s[k][i]);
-          fail |= sb > mag_bits(real(1)) ? over_tol(r, s[k][i], tol) : rb > mag_bits(tol);
-          bad |= rb > mag_bits(kRealMax<real>) || sb > mag_bits(kRealMax<real>);
+          const unsigned rh = mag_hi(r), sh = mag_hi(s[k][i]);
+          // |r| against tol max(1, |s|) by their leading 32 bits, where those differ enough
+          const unsigned lh =
+              mag_hi(sh >= mag_hi(real(1)) ? tol * rabs(s[k][i]) : tol);
+          fail |= rh > lh + 2u;
+          near |= rh - lh + 2u <= 4u;
+          bad |= rh >= mag_hi(real(INFINITY)) || sh >= mag_hi(real(INFINITY));
 #pragma unroll
           for (int j = 0; j < D; ++j) {
             if (scale != real(1)) Ak[k][i][j] *= scale;
@@ -269,6 +275,15 @@ __global__ void __launch_bounds__(NT) k_block_solve(BlockSolveArgs<real> a) {
 #pragma unroll
         for (int i = 0; i < D; ++i) sp[i] = s[k][i];
       }
+    }
+    if (__any_sync(0xffffffffu, near)) {  // (rare)
+#pragma unroll
+      for (int k = 0; k < RPT; ++k)
+        if (k < nmine) {
+#pragma unroll
+          for (int i = 0; i < D; ++i)
+            fail |= over_tol(s[k][i] - Fk[k][i], s[k][i], tol);
+        }
     }
     // 2. votes and elements up the trees
     const int vote = (__any_sync(0xffffffffu, fail) ? 1 : 0) | (__any_sync(0xffffffffu, bad) ? 2 : 0);
