@@ -27,8 +27,8 @@
 // and only vectors come down (44 instructions at d = 2, 1024 rows, against 150 for an
 // inclusive scan of whole elements per lane), the rows spread over all four warps of a
 // block, and comparisons work on the bit patterns. Brusselator,
-// float64, T = 1024: 13.0 -> 7.2 us per iteration (start 376, now 278 us a call, of which
-// about 150 is the host); 64 x 2048 rows 3.24 -> 1.77 ms.
+// float64, T = 1024: 13.0 -> 7.2 us per iteration (a call of 28 iterations 374 -> 254 us, of
+// which about 50 is the host); 64 x 2048 rows 3.24 -> 1.77 ms.
 #include <cooperative_groups.h>
 
 #include <cfloat>

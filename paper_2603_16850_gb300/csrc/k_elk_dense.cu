@@ -16,7 +16,7 @@
 // min(32, d^2) lanes, or more in the carry, and every d x d product is spread over all of
 // them, one or a few entries per lane (16 instructions per product at d = 8 against 64 with a
 // row per lane); inverses are in place (half the entries of an augmented elimination) and
-// their reciprocals take four FP64 instructions instead of a division's 23. Mass action d = 8,
+// their reciprocals take four FP64 instructions of 64 clocks instead of a division's 1490. Mass action d = 8,
 // float64, 4 sequences of 4096 rows, per iteration (d lanes per chunk, a row per lane, blocks
 // of 16 chunks before): chunk elements 2626 -> 300 us, carry 1696 (64 steps) -> 536 (128
 // steps, 4.2 us each: pivots in order), restart 1538 -> 194 us.
