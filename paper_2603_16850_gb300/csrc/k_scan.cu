@@ -1223,14 +1223,31 @@ __global__ void __launch_bounds__(128) k_scalar_apply(DenseScanArgs<real> a) {
 // Segments shorten the carry when few sequences have many chunks: a chain of n steps becomes
 // M + n / M + M with M about sqrt(n), at the price of folding the aggregates once more. At
 // 157 chunks (Langevin, d = 4, float64) 28 us against 40 in one level; below 128 the two
-// extra launches cost what is saved. More sequences than SM sub-partitions x groups per warp
-// hide the chain by themselves. The batch size decides, not the active set: the two forms round
-// differently, and a call keeps one of them, whatever else is still active and whichever loop runs.
+// extra launches cost what is saved. The folds are d^3 work per chunk of every sequence, the chain
+// that they save is one sequence's, so they pay up to a number of sequences that hardly depends
+// on their length. Per iteration with segments less without, us, 160 / 1024 chunks a sequence:
+//   float32 d = 8, 256 sequences -8 / -130, 512 +5 / -79; d = 16, 128: -10 / -85, 256: +8 / -15,
+//   512: +34 / +137; d = 32, 16: -1 / -80, 32: +9 / -10, 64: +30 / +119, 256: +152
+//   float64 d = 8, 128: -21 / -263, 256: +4 / -74, 512: +58 / +189; d = 16, 32: -13 / -380, 64: +1 /
+//   -199, 128: +80 / +522; d = 32, 4: -132 / -946, 16: +19 / -129, 32: +263
+// and at d = 4 they pay up to the 512 sequences measured (beyond as many as there are schedulers
+// times groups in a warp the sequences hide the chain by themselves). The batch size decides, not
+// the active set: the two forms round differently, and a call keeps one of them, whatever else is
+// still active and whichever loop runs.
+template <class real, int D>
+constexpr int64_t segment_batch() {
+  constexpr bool f64 = sizeof(real) == 8;
+  if (D <= 4) return kSchedulers * (32 / group_lanes<D>());
+  if (D <= 8) return f64 ? 256 : 512;
+  if (D <= 16) return f64 ? 64 : 224;
+  return f64 ? 12 : 24;
+}
+
 template <class real, int D>
 static void set_segments(DenseScanArgs<real>& a) {
   a.log2M = 0;
   const int64_t n = a.max_chunks;
-  if (!a.segP || n < 128 || a.bt.B > kSchedulers * (32 / group_lanes<D>())) return;
+  if (!a.segP || n < 128 || a.bt.B > segment_batch<real, D>()) return;
   a.log2M = 3;
   while (a.log2M < 6 && ((int64_t)1 << (2 * a.log2M + 2)) <= n) ++a.log2M;
 }

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 
 def test_same_form_while_the_active_set_shrinks():
     import paper_2603_16850_gb300 as deer
-    # 128 chunks of 8 rows; more sequences than SM sub-partitions times groups of 8 lanes in a
-    # warp (608 x 4), most of which start at their solution
+    # 128 chunks of 8 rows; more sequences than the folds are taken for, most of which start at
+    # their solution
     B, T, d, live = 2440, 1024, 8, 40
     p = synth.mean_field_rnn(live, T, d, 0.9, seed=9)
     f = torch.float32
